@@ -17,6 +17,7 @@
 #include <cstddef>
 #include <stdint.h>
 
+#include "lbm_fix64.cuh"
 #include "lbm_internal.h"
 
 namespace axilbm {
@@ -55,6 +56,19 @@ static_assert(offsetof(CaseReal<float>, nu_g) == 12 && offsetof(CaseReal<float>,
                   offsetof(CaseReal<float>, kappa) == 28,
               "FP32 parameter order read by node_macros");
 
+// Combinations of one case's FP64 parameters (lbm_f64.cuh), formed once on the
+// host instead of per node on the FP64 pipe.  s: the phase-field rate of the
+// momenta (compile-time rate patterns).
+struct Case64 {
+    double drho, drho3, dnu;  // rho_l - rho_g, 0.3 / 72 of it, nu_l - nu_g
+    double beta4, mkappa;     // 4 beta, -kappa / 72 (Eq. 4)
+    double neps72;            // 72 n_eps
+    double pad;
+    double lam3;              // 4 / (3 W): r lambda / 3 = lam3 r phi (1 - phi) (Eq. 2)
+    double h3, sh3;           // (1 - s/2) / 3, (1 + s/2) / 3
+    double c2, c4;            // (1 - s) / 2, (1 - s) / 4
+};
+
 // Case c owns the handle's nodes [off, off + plane): node (k, j) is node
 // off + k * pitch + j (pitch = nr rounded up to 32, off a multiple of 32).
 // How nodes are stored is described with Block below.  Node indices inside a
@@ -71,9 +85,14 @@ struct CaseDev {
     // mixed FP16 step against the FP64 block first; FP32 unchanged)
     CaseReal<float> pf;
     CaseReal<double> pd;
+    Case64 p64;
 };
 static_assert(sizeof(CaseDev) % 16 == 0, "CaseDev is copied to shared memory by a bulk copy");
 static_assert(offsetof(CaseDev, pf) % 16 == 0 && offsetof(CaseDev, pd) % 8 == 0, "parameter block alignment");
+// 32-bit words of the record a kernel of this arithmetic reads: the FP32
+// kernels stop before the FP64 parameters.
+template <typename Real>
+constexpr int kCaseWords = (int)((sizeof(Real) == 8 ? sizeof(CaseDev) : offsetof(CaseDev, pd)) / 4);
 
 template <typename Real>
 __device__ __forceinline__ const CaseReal<Real>& case_params(const CaseDev& C);
@@ -507,7 +526,7 @@ __device__ __forceinline__ int ghost_z(int k, int nz, int zper) {
 }
 
 // phi of a node from its raw stored f_0 (F0T) and f_1..8 (Eq. 16): the
-// plain sum in FP64 and FP32 storage, phi_grid in FP16 storage (Sa: S_a of
+// plain sum in FP32 storage, sum64's in FP64 storage, phi_grid in FP16 storage (Sa: S_a of
 // the node's column; unused otherwise), phi_from_halves in bfloat16 storage.
 template <class Codec>
 __device__ __forceinline__ typename Codec::Real phi_of(const typename Codec::F0T& f0raw,
@@ -518,6 +537,9 @@ __device__ __forceinline__ typename Codec::Real phi_of(const typename Codec::F0T
         return phi_grid(f0_value(f0raw), fraw, inv_r, Sa);
     } else if constexpr (sizeof(typename Codec::PT) == 2) {
         return phi_from_halves(f0_value(f0raw), fraw, inv_r);
+    } else if constexpr (sizeof(Real) == 8) {
+        const double f[9] = {f0raw, fraw[0], fraw[1], fraw[2], fraw[3], fraw[4], fraw[5], fraw[6], fraw[7]};
+        return sum64(f) * inv_r;
     } else {
         Real s = (Real)f0_value(f0raw);
 #pragma unroll
@@ -537,13 +559,13 @@ __device__ __forceinline__ void load_phi_raw(const Node<Codec>& n, typename Code
     for (int i = 1; i < 9; ++i) f[i - 1] = n.f(i);
 }
 
-// phi at an in-domain node from its stored populations (Eq. 16).  FP64 and
-// FP32: each load feeds the running sum (the order phi_of sums in).
+// phi at an in-domain node from its stored populations (Eq. 16).  FP32: each
+// load feeds the running sum (the order phi_of sums in).
 template <class Codec>
 __device__ __forceinline__ typename Codec::Real node_phi(const Node<Codec>& n, typename Codec::Real inv_r,
                                                           float Sa = 0.0f) {
     using Real = typename Codec::Real;
-    if constexpr (sizeof(typename Codec::PT) == 2) {
+    if constexpr (sizeof(typename Codec::PT) != 4) {
         typename Codec::PT fraw[8];
 #pragma unroll
         for (int i = 1; i < 9; ++i) fraw[i - 1] = n.f(i);
@@ -561,13 +583,42 @@ __device__ __forceinline__ typename Codec::Real node_phi(const Node<Codec>& n, t
 // subnormal inputs and results flushed to zero (PTX .approx.ftz): values
 // below 2^-126 arise only in the far field at rest, and the forms that keep
 // them cost 1.7 % (FP32) to 3.5 % (16-bit storage) of the step;
-// FP64: IEEE division and square root, as in the oracle.
+// FP64: reciprocal and square root from the hardware's FP64 approximations with
+// one third-order step (3 and 5 operations on the FP64 pipe; the IEEE forms take
+// as long as 4.5 and 7.6 and stay for operands near the ends of the range), IEEE
+// division.
 __device__ __forceinline__ float rcp_(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
+// 1 / x: y0 from the hardware (relative error below 2^-20), e = 1 - x y0,
+// y0 (1 + e + e^2): the truncation is below 2^-60, so the last rounding is all
+// that is left.  Outside 2^-1000 .. 2^1000 (and for 0, infinities and NaN) the
+// IEEE division.
+__device__ __forceinline__ double rcp64(double x) {
+    double y0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double e = fma(-x, y0, 1.0);
+    double y = fma(fma(e, e, e), y0, y0);
+    const uint32_t ex = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
+    if (ex - 23u > 2000u) y = 1.0 / x;
+    return y;
+}
+// sqrt(x), x >= 0: y0 = 1 / sqrt(x) from the hardware, e = 1 - x y0^2,
+// x y0 (1 + e / 2 + 3 e^2 / 8): truncation below 2^-57.
+__device__ __forceinline__ double sqrt64(double x) {
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double s = x * y0;
+    const double e = fma(-s, y0, 1.0);
+    double y = fma(s * e, fma(0.375, e, 0.5), s);
+    const uint32_t hi = (uint32_t)__double2hiint(x), ex = hi >> 20;  // a sign bit counts as out of range
+    if ((hi | (uint32_t)__double2loint(x)) == 0u) y = 0.0;  // no gradient: whole tiles of the far field
+    else if (ex - 23u > 2000u) y = sqrt(x);
+    return y;
+}
+__device__ __forceinline__ double rcp_(double x) { return rcp64(x); }
 __device__ __forceinline__ float div_(float a, float b) {
     float y;
     asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
@@ -579,7 +630,7 @@ __device__ __forceinline__ float sqrt_(float x) {
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+__device__ __forceinline__ double sqrt_(double x) { return sqrt64(x); }
 
 // ---------------------------------------------------------------- macroscopic part
 template <typename Real>

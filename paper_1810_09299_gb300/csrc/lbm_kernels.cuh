@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_device.cuh"
+#include "lbm_f64.cuh"
 #include "lbm_internal.h"
 #include "lbm_lane.cuh"
 
@@ -483,6 +484,61 @@ __device__ __forceinline__ void node_update_grid(const CaseDev& C, const CaseVie
     node_post_grid<Codec>(C, V, k, j, loc, fp, gp, chz, chr, m.p, pre.mf[0], cols);
 }
 
+// The FP64 node update of a compile-time rate pattern (lbm_f64.cuh) with its
+// stores: the push of node_update_pre without radii (FP64 populations are
+// stored as they are).
+template <int RM, int LD>
+__device__ __forceinline__ void node_update64(const CaseDev& C, const CaseView<CodecF64>& V, const Win64& W, int a,
+                                              int b, double phi, int k, int j, int loc, const Col64& K, const Pre64& pre,
+                                              double chz_prev, double chr_prev, double p_prev) {
+    double fp[9], gp[9], chz, chr, p;
+    update64<LD, RM>(C, W, a, b, phi, K, pre, chz_prev, chr_prev, p_prev, fp, gp, chz, chr, p);
+    const Node<CodecF64> own = V.out_node(loc);
+    own.chz() = chz;
+    own.chr() = chr;
+    if (C.p_coupling == 1) own.p() = p;
+    const bool axis = (j == 0), wall = (j + 1 == C.nr), zlo = (k == 0), zhi = (k + 1 == C.nz);
+    constexpr int kB = Block<CodecF64>::bytes, kPS = (int)sizeof(double2);
+    const int lane = loc & 31;
+    unsigned char* const q0 = V.out_pt(loc).q;  // the node's own pair pointer
+    const int row = (C.pitch >> 5) * kB;         // one z row of blocks
+    const int step_r = lane == 31 ? kB - 31 * kPS : kPS;
+    const int step_l = lane == 0 ? -(kB - 31 * kPS) : -kPS;
+    if ((zlo || zhi) && !C.zper) {
+#define AXILBM_PUSH(I)                                                                         \
+    {                                                                                          \
+        const Dest d = destination<I>(k, j, C.nr, C.nz, C.zper);                               \
+        V.out_pt(d.k * C.pitch + d.j).pair(d.dir) = make_double2(fp[I], gp[I]);                \
+    }
+        AXILBM_PUSH(1)
+        AXILBM_PUSH(2)
+        AXILBM_PUSH(3)
+        AXILBM_PUSH(4)
+        AXILBM_PUSH(5)
+        AXILBM_PUSH(6)
+        AXILBM_PUSH(7)
+        AXILBM_PUSH(8)
+#undef AXILBM_PUSH
+    } else {
+        const int rowp = zhi ? -(C.nz - 1) * row : row;
+        const int rowm = zlo ? (C.nz - 1) * row : -row;
+#define AXILBM_PUSH(I)                                                                                            \
+    *reinterpret_cast<double2*>(q0 + push_offset<CodecF64, I>(axis, wall, rowp, rowm, step_r, step_l)) =          \
+        make_double2(fp[I], gp[I]);
+        AXILBM_PUSH(1)
+        AXILBM_PUSH(2)
+        AXILBM_PUSH(3)
+        AXILBM_PUSH(4)
+        AXILBM_PUSH(5)
+        AXILBM_PUSH(6)
+        AXILBM_PUSH(7)
+        AXILBM_PUSH(8)
+#undef AXILBM_PUSH
+    }
+    own.g(0) = gp[0];
+    own.f0() = fp[0];
+}
+
 // One time step for every node of every tile in `tiles`: one CTA per tile of
 // BZ rows (z) x 32 columns (r), one node per thread.  Each thread first issues
 // the loads of its own node; the node's phi goes to the shared window straight
@@ -499,7 +555,14 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     constexpr int LD = kTR + 4;
     constexpr int NRING = 4 * kTR + 4 * (TZ + 4);
     static_assert(NRING == (TZ + 4) * LD - TZ * kTR, "the ring is the window without the tile");
-    __shared__ Real sphi[(TZ + 4) * LD];
+    // FP64 with a compile-time rate pattern: the update of lbm_f64.cuh, whose
+    // phi window holds unpacked numbers
+    constexpr bool kU64 = sizeof(Real) == 8 && RM != kRatesGeneral;
+    constexpr int NWIN = (TZ + 4) * LD;
+    __shared__ Real sphi[kU64 ? 1 : NWIN];
+    __shared__ long long swm[kU64 ? NWIN : 1];
+    __shared__ int swe[kU64 ? NWIN : 1];
+    const Win64 W{swm, swe};
     // The case's parameters go to shared memory: read from there, the
     // collision's many per-case constants need no global loads.
     __shared__ __align__(16) CaseDev sC;
@@ -509,6 +572,8 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     // FP64 pipe); the same correctly rounded quotients the nodes would form
     constexpr bool kInvrTable = sizeof(Real) == 8;
     __shared__ Real s_invr[kInvrTable ? LD : 1];
+    __shared__ double s_col_raw[kU64 ? sizeof(ColTab64) / 8 : 1];
+    ColTab64& s_col = *reinterpret_cast<ColTab64*>(s_col_raw);
     // 16-bit storage: the column constants of the window's columns
     constexpr bool kG = Codec::kGrid;
     __shared__ float4 sgA[kG ? LD : 1], sgD[kG ? LD : 1];
@@ -516,7 +581,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     const GridTab T{sgA, sgD, sgH};
     const TileGeo g = reinterpret_cast<const TileGeo*>(tiles + ntiles)[blockIdx.x];
     const int q = threadIdx.y * kTR + threadIdx.x;
-    constexpr int kCW = (int)(sizeof(CaseDev) / 4);                // words of the case record
+    constexpr int kCW = kCaseWords<Real>;                // words of the case record
     constexpr int kRC = (NRING + kTR * BZ - 1) / (kTR * BZ);        // ring cells per thread
     constexpr int kB = Block<Codec>::bytes;
     // 1. every global load of the window phase leaves before any of them is
@@ -565,6 +630,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
         if constexpr (kG) return grid_sa<Codec>(jj);
         else return 0.0f;
     };
+    Real ring_sum[kInvrTable ? kRC : 1];  // FP64: as own_sum below
 #pragma unroll
     for (int c = 0; c < kRC; ++c) {
         if (q + c * kTR * BZ < NRING) {
@@ -574,25 +640,31 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
             F0T rf0;
             PT rf[8];
             load_phi_raw<Codec>(node_at(ghost_z(g.k0 - 2 + ra, g.nz, g.zper), rj), rf0, rf);
-            sphi[ra * LD + rb] = phi_of<Codec>(rf0, rf, rcp_((Real)rj + (Real)0.5), sa_of(rj));
+            if constexpr (kInvrTable) ring_sum[c] = phi_of<Codec>(rf0, rf, (Real)1);
+            else sphi[ra * LD + rb] = phi_of<Codec>(rf0, rf, rcp_((Real)rj + (Real)0.5), sa_of(rj));
         }
     }
     const Real r = (Real)j + (Real)0.5;
     const int bo = threadIdx.x + 2;
-    Real own_sum = (Real)0;  // FP64: the node's f summed; phi once the 1 / r table is filled
+    Real own_sum = (Real)0, own_phi = (Real)0;  // FP64: the node's f summed; phi once the 1 / r table is filled
     if (inside) {
         if constexpr (sizeof(PT) == 2) {
             sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_(r), sa_of(j));
         } else {
-            Real sum = (Real)f0_value(f0raw);
+            if constexpr (kU64) {
+            } else if constexpr (kInvrTable) {
+                own_sum = phi_of<Codec>(f0raw, fraw, (Real)1);
+            } else {
+                Real sum = (Real)f0_value(f0raw);
 #pragma unroll
-            for (int i = 1; i < 9; ++i) sum += Codec::dec_f(fraw[i - 1], (Real)w_of(i) * r);
-            if constexpr (kInvrTable) own_sum = sum;
-            else sphi[(threadIdx.y + 2) * LD + bo] = sum * rcp_(r);
+                for (int i = 1; i < 9; ++i) sum += Codec::dec_f(fraw[i - 1], (Real)w_of(i) * r);
+                sphi[(threadIdx.y + 2) * LD + bo] = sum * rcp_(r);
+            }
         }
     } else {
         const int jm = ghost_r(j, g.nr);
-        sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_((Real)jm + (Real)0.5), sa_of(jm));
+        if constexpr (kInvrTable) own_sum = phi_of<Codec>(f0raw, fraw, (Real)1);
+        else sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_((Real)jm + (Real)0.5), sa_of(jm));
     }
     // FP64: the node's moments while other warps still wait for their loads
     // (19.67 against 19.99 ms on the 512-case batch, bit-identical; in FP32
@@ -600,12 +672,26 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     // 0.761 against 0.735 ms)
     constexpr bool kPreEarly = sizeof(Real) == 8;
     PreCollision<Real> pre;
-    if constexpr (kPreEarly) {
+    Pre64 pre6;
+    if constexpr (kU64) {
+        if (inside) {
+            const Real f[9] = {f0raw, fraw[0], fraw[1], fraw[2], fraw[3], fraw[4], fraw[5], fraw[6], fraw[7]};
+            pre64<RM>(f, graw, pre6);
+            own_sum = pre6.T;
+        }
+    } else if constexpr (kPreEarly) {
         if (inside) node_pre<Codec>(f0raw, fraw, graw, r, pre, nullptr, GridCol{});
     }
     // 3. the column tables and the case record into shared memory
     if constexpr (kInvrTable) {
-        if (q < LD) s_invr[q] = (Real)1 / ((Real)(g.j0 - 2 + q) + (Real)0.5);
+        if (q < LD) {
+            const int jm = ghost_r(g.j0 - 2 + q, g.nr);
+            const Real ir = rcp_((Real)jm + (Real)0.5);
+            s_invr[q] = ir;
+            if constexpr (kU64) {
+                if (q >= 2 && q < kTR + 2) s_col.put(q - 2, col64(jm, ir));
+            }
+        }
     }
     if constexpr (kG) {
         if (q < LD) grid_tab_fill<Codec>(T, q, g.j0, g.nr);
@@ -613,9 +699,22 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     if (q < kCW) reinterpret_cast<int32_t*>(&sC)[q] = cw;
     if constexpr (kInvrTable) {
         // FP64: one division per column, not per node (a division is a long
-        // sequence on the FP64 pipe), so the own phi waits for the table
+        // sequence on the FP64 pipe), so the phi of the window waits for the table
+        auto put_phi = [&](int cell, Real v) {
+            if constexpr (kU64) W.put(cell, v);
+            else sphi[cell] = v;
+        };
         __syncthreads();
-        if (inside) sphi[(threadIdx.y + 2) * LD + bo] = own_sum * s_invr[bo];
+        own_phi = own_sum * s_invr[bo];
+        put_phi((threadIdx.y + 2) * LD + bo, own_phi);
+#pragma unroll
+        for (int c = 0; c < kRC; ++c) {
+            if (q + c * kTR * BZ < NRING) {
+                int ra, rb;
+                ring_cell<TZ>(q + c * kTR * BZ, ra, rb);
+                put_phi(ra * LD + rb, ring_sum[c] * s_invr[rb]);
+            }
+        }
     }
     __syncthreads();
     if (!inside) return;
@@ -644,6 +743,9 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
         const TabCols cols{T, j == 0 ? bo : bo - 1, bo, j + 1 == C.nr ? bo : bo + 1};
         node_update_grid<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
                                         chr_prev, p_prev, f, cols);
+    } else if constexpr (kU64) {
+        node_update64<RM, LD>(C, V, W, threadIdx.y + 2, bo, own_phi, k, j, loc, s_col.get(threadIdx.x), pre6,
+                              chz_prev, chr_prev, p_prev);
     } else {
         if constexpr (kPreEarly) {
             node_update_pre<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, pre, chz_prev, chr_prev,
@@ -706,7 +808,7 @@ step_kernel_seq2(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
     const GridTab T{sgA, sgD, sgH};
     const TileGeo g = reinterpret_cast<const TileGeo*>(tiles + ntiles)[blockIdx.x];
     const int q = threadIdx.y * kTR + threadIdx.x;
-    constexpr int kCW = (int)(sizeof(CaseDev) / 4);  // words of the case record
+    constexpr int kCW = kCaseWords<Real>;  // words of the case record
     static_assert(NRING <= kTR * BZ, "one ring cell per thread at most");
     constexpr int kB = Block<Codec>::bytes;
     // 1. every global load of the window phase leaves before any of them is
@@ -964,7 +1066,7 @@ step_kernel_pack2(const CaseDev* __restrict__ cases, const TileGeo* __restrict__
     const GridTab T{sgA, sgD, sgH};
     const TileGeo g = geo[blockIdx.x];
     const int q = threadIdx.y * kTR + threadIdx.x;
-    constexpr int kCW = (int)(sizeof(CaseDev) / 4);  // words of the case record
+    constexpr int kCW = kCaseWords<float>;  // words of the case record
     // 1. every load of the window phase is issued before any of them is used:
     //    the case record word of this thread, both nodes' own values and the
     //    raw values of this thread's ring cell
@@ -1082,7 +1184,8 @@ struct TmaTile {
     // two stages when they fit, else one (FP64 with tall tiles)
     static constexpr int NS = (2 * stage_bytes + 16384 <= 200 * 1024) ? 2 : 1;
     static constexpr size_t off_phi = NS * stage_bytes;
-    static constexpr size_t off_bar = al(off_phi + (size_t)HR * LD * sizeof(Real));
+    // FP64: 12 bytes a window cell (Win64)
+    static constexpr size_t off_bar = al(off_phi + (size_t)HR * LD * (sizeof(Real) == 8 ? 12 : sizeof(Real)));
     static constexpr size_t bytes = off_bar + 128;
 };
 
@@ -1164,6 +1267,12 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
     constexpr int kWaitTries = 1 << 22;
     extern __shared__ __align__(128) unsigned char smem[];
     Real* sphi = (Real*)(smem + L::off_phi);  // [HR][LD]
+    constexpr bool kU64 = sizeof(Real) == 8 && RM != kRatesGeneral;
+    const Win64 W{(long long*)(smem + L::off_phi), (int*)(smem + L::off_phi + 8 * (size_t)L::HR * LD)};
+    auto put_phi = [&](int cell, Real v) {
+        if constexpr (kU64) W.put(cell, v);
+        else sphi[cell] = v;
+    };
     uint64_t* bar = (uint64_t*)(smem + L::off_bar);
     const int tid = threadIdx.y * kTR + threadIdx.x;
     if ((int)blockIdx.x >= ntiles) return;
@@ -1222,7 +1331,7 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
         for (int q = tid; q < NRING; q += kTR * BZ) {
             int a, b;
             ring_cell<TZ>(q, a, b);
-            sphi[a * LD + b] = staged_phi<Codec, TZ>(st, C, V, tt, a, b);
+            put_phi(a * LD + b, staged_phi<Codec, TZ>(st, C, V, tt, a, b));
         }
         // the node's own phi (Eq. 16) from its staged populations
         const Real r = (Real)j + (Real)0.5;
@@ -1234,6 +1343,11 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
 #pragma unroll
                 for (int i = 1; i < 9; ++i) f[i] = Codec::dec_f(fraw[i - 1], g, i > 4);
                 sphi[(threadIdx.y + 2) * LD + threadIdx.x + 2] = phi_of<Codec>(f0raw, fraw, rcp_(r), g.S_a);
+            } else if constexpr (sizeof(Real) == 8) {
+                f[0] = f0raw;
+#pragma unroll
+                for (int i = 1; i < 9; ++i) f[i] = fraw[i - 1];
+                put_phi((threadIdx.y + 2) * LD + threadIdx.x + 2, phi_of<Codec>(f0raw, fraw, rcp_(r)));
             } else {
                 f[0] = (Real)f0_value(f0raw);
                 Real sum = f[0];
@@ -1246,8 +1360,8 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
                     sizeof(PT) == 2 ? phi_of<Codec>(f0raw, fraw, rcp_(r)) : sum * rcp_(r);
             }
         } else {
-            sphi[(threadIdx.y + 2) * LD + threadIdx.x + 2] =
-                staged_phi<Codec, TZ>(st, C, V, tt, threadIdx.y + 2, threadIdx.x + 2);
+            put_phi((threadIdx.y + 2) * LD + threadIdx.x + 2,
+                    staged_phi<Codec, TZ>(st, C, V, tt, threadIdx.y + 2, threadIdx.x + 2));
         }
         __syncthreads();
         if (inside) {
@@ -1256,6 +1370,12 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
                 const CalcCols<Codec> cols{j == 0 ? j : j - 1, j, j + 1 == C.nr ? j : j + 1};
                 node_update_grid<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, threadIdx.x + 2, k, j, loc, f0raw,
                                                 fraw, graw, chz_prev, chr_prev, p_prev, f, cols);
+            } else if constexpr (sizeof(Real) == 8 && RM != kRatesGeneral) {
+                Pre64 pre;
+                pre64<RM>(f, graw, pre);
+                const Real ir = rcp_(r);
+                node_update64<RM, LD>(C, V, W, threadIdx.y + 2, threadIdx.x + 2, pre.T * ir, k, j, loc, col64(j, ir),
+                                      pre, chz_prev, chr_prev, p_prev);
             } else {
                 node_update<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, threadIdx.x + 2, k, j, loc, f0raw, fraw,
                                            graw, chz_prev, chr_prev, p_prev, nullptr,
