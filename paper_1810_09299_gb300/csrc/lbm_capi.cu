@@ -268,16 +268,21 @@ CaseDev make_case(const lbm_params& p, int64_t off, int64_t dense_off) {
     fill_params<float>(C.pf, p);
     const double s = C.pd.sf[p.collision == LBM_MRT_RAW ? 1 : 3];
     C.p64.drho = p.rho_l - p.rho_g;
-    C.p64.drho3 = 0.3 / 72.0 * C.p64.drho;
     C.p64.dnu = p.nu_l - p.nu_g;
     C.p64.beta4 = 4.0 * C.pd.beta;
-    C.p64.mkappa = -C.pd.kappa / 72.0;
-    C.p64.neps72 = 72.0 * p.n_eps;
     C.p64.lam3 = 4.0 / (3.0 * p.W);
-    C.p64.h3 = (1.0 - 0.5 * s) / 3.0;
-    C.p64.sh3 = (1.0 + 0.5 * s) / 3.0;
-    C.p64.c2 = 0.5 * (1.0 - s);
-    C.p64.c4 = 0.25 * (1.0 - s);
+    C.p64.neps72 = 72.0 * p.n_eps;
+    C.p64.c2 = (long long)std::ldexp(0.5 * (1.0 - s), 62);
+    C.p64.c4 = (long long)std::ldexp(0.25 * (1.0 - s), 62);
+    auto sf = [](double x, long long& m, int32_t& e) {
+        int ex = 0;
+        m = (long long)std::ldexp(std::frexp(x, &ex), 62);  // 2^61 <= |m| < 2^62
+        e = x == 0.0 ? kZeroE : ex - 62;
+    };
+    sf(-C.pd.kappa / 72.0, C.p64.mkappa_m, C.p64.mkappa_e);
+    sf(0.3 / 72.0 * C.p64.drho, C.p64.drho3_m, C.p64.drho3_e);
+    sf((1.0 - 0.5 * s) / 3.0, C.p64.h3_m, C.p64.h3_e);
+    sf((1.0 + 0.5 * s) / 3.0, C.p64.sh3_m, C.p64.sh3_e);
     return C;
 }
 

@@ -29,19 +29,23 @@
 
 namespace axilbm {
 
-// One cell of the phi window: phi = m 2^(e - 1075), m with its sign.
+constexpr int kWinK = 3;  // 72 grad of at most 108 and 9 lap of at most 80 largest values stay below 2^63
+// One cell of the phi window: phi = m 2^(e - 1075 - kWinK), m with its sign.
 struct Win64 {
     long long* m;
     int* e;
     __device__ __forceinline__ void put(int c, double x) const {
         const int hi = __double2hiint(x), ex = exp64(x);
         const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
-        const long long v = (long long)(((unsigned long long)mh << 32) | (uint32_t)__double2loint(x));
+        const long long v = (long long)((((unsigned long long)mh << 32) | (uint32_t)__double2loint(x)) << kWinK);
         const long long sg = (long long)(hi >> 31);
-        m[c] = ex == 0 ? 0ll : (v ^ sg) - sg;
+        m[c] = (v ^ sg) - sg;  // zero (ex = 0) leaves every block: E - ex >= kMinE
         e[c] = ex;
     }
 };
+
+// v 2^e with |v| < 2^63, normalised
+__device__ __forceinline__ Sf norm_any(long long v, int e) { return norm(Sf{v >> 1, e + 1}); }
 
 // The stencils of Eq. 39-40 in the block of their 17 values, times 72:
 //   72 grad = 4 (8 X_1 - X_2) + (8 D_1 - D_2) with X, D the differences of the
@@ -49,8 +53,7 @@ struct Win64 {
 //   72 lap = 4 (16 A_1 - A_2) + 16 B_1 - B_2 with A, B the sums of the axis and
 // diagonal values minus four times the centre.
 template <int LD>
-__device__ __forceinline__ void stencil64(const Win64& W, int a, int b, double& gz, double& gr, double& lap) {
-    constexpr int K = 3;  // |72 grad| <= 108 and 9 |lap| <= 80 largest values: below 2^63
+__device__ __forceinline__ void stencil64(const Win64& W, int a, int b, Sf& gz, Sf& gr, Sf& lap, bool& bad) {
     const int c = a * LD + b;
     int E = max(W.e[c], kMinE);
     int ex[2][9];
@@ -67,9 +70,9 @@ __device__ __forceinline__ void stencil64(const Win64& W, int a, int b, double& 
     for (int i = 1; i < 9; ++i) {
 #pragma unroll
         for (int n = 0; n < 2; ++n)
-            x[n][i] = (W.m[c + (n + 1) * (cz_of(i) * LD + cr_of(i))] << K) >> min(E - ex[n][i], 63);
+            x[n][i] = shr64(W.m[c + (n + 1) * (cz_of(i) * LD + cr_of(i))], E - ex[n][i]);
     }
-    const long long c4 = ((W.m[c] << K) >> min(E - W.e[c], 63)) * 4;
+    const long long c4 = shr64(W.m[c], E - W.e[c]) * 4;
     long long X[2], Y[2], Z[2], R[2], A[2], B[2];
 #pragma unroll
     for (int n = 0; n < 2; ++n) {
@@ -81,21 +84,26 @@ __device__ __forceinline__ void stencil64(const Win64& W, int a, int b, double& 
         A[n] = (x[n][1] + x[n][3]) + (x[n][2] + x[n][4]) - c4;
         B[n] = (x[n][5] + x[n][7]) + (x[n][6] + x[n][8]) - c4;
     }
-    const bool bad = E >= kBadE;
-    gz = bad ? nan64() : unfix64<K>(X[0] * 32 - X[1] * 4 + Z[0] * 8 - Z[1], E);
-    gr = unfix64<K>(Y[0] * 32 - Y[1] * 4 + R[0] * 8 - R[1], E);
+    const int e = E - 1075 - kWinK;
+    gz = norm_any(X[0] * 32 - X[1] * 4 + Z[0] * 8 - Z[1], e);
+    gr = norm_any(Y[0] * 32 - Y[1] * 4 + R[0] * 8 - R[1], e);
     // 9 lap in units of the block, from values of at most 8 (A, B)
-    lap = unfix64<K - 3>(A[0] * 8 - (A[1] >> 1) + B[0] * 2 - (B[1] >> 3), E);
+    lap = norm_any(A[0] * 8 - (A[1] >> 1) + B[0] * 2 - (B[1] >> 3), e + 3);
+    bad = E >= kBadE;
 }
 
-// What the collisions take from a node's own populations.
+// What the collisions take from a node's own populations: sum f = r phi as a
+// double, the differences that the phase-field collision acts on in the block
+// of f, and the moments of g.
 struct Pre64 {
-    double T;             // sum f = r phi
-    double fz, fe, fr, fo;  // f_1 - f_3, f_5 - f_7 - f_6 + f_8, f_2 - f_4, f_5 - f_7 + f_6 - f_8
-    double S0;            // g_1 + .. + g_8
-    double q;             // the even moment that relaxes with 1/tau_g: M g's e, raw: sum c^2 g
-    double Jz, Jr;        // sum c g
-    double m7, m8;        // sum (c_z^2 - c_r^2) g, sum c_z c_r g
+    double T;
+    int Ef;                    // the block exponent of f
+    bool bad;                  // a value out of the range of the sums, infinite or NaN
+    long long t, fz, fe, fr, fo;  // sum f, f_1 - f_3, f_5 - f_7 - f_6 + f_8, f_2 - f_4, f_5 - f_7 + f_6 - f_8
+    Sf S0;                     // g_1 + .. + g_8
+    Sf q;                      // the even moment that relaxes with 1/tau_g: M g's e, raw: sum c^2 g
+    Sf Jz, Jr;                 // sum c g
+    Sf m7, m8;                 // sum (c_z^2 - c_r^2) g, sum c_z c_r g
 };
 
 template <int RM>
@@ -105,173 +113,223 @@ __device__ __forceinline__ void pre64(const double* fd, const double* gd, Pre64&
         long long f[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i] = fix64<kPopK>(fd[i], E);
-        const double T = unfix64<kPopK>((f[0] + f[1] + f[2]) + (f[3] + f[4] + f[5]) + (f[6] + f[7] + f[8]), E);
-        P.T = E >= kBadE ? nan64() : T;
+        P.Ef = E;
+        P.t = (f[0] + f[1] + f[2]) + (f[3] + f[4] + f[5]) + (f[6] + f[7] + f[8]);
+        P.T = unfix64<kPopK>(P.t, E);
+        P.bad = E >= kBadE;
+        if (P.bad) P.T = nan64();
         const long long f57 = f[5] - f[7], f68 = f[6] - f[8];
-        P.fz = unfix64<kPopK>(f[1] - f[3], E);
-        P.fe = unfix64<kPopK>(f57 - f68, E);
-        P.fr = unfix64<kPopK>(f[2] - f[4], E);
-        P.fo = unfix64<kPopK>(f57 + f68, E);
+        P.fz = f[1] - f[3];
+        P.fe = f57 - f68;
+        P.fr = f[2] - f[4];
+        P.fo = f57 + f68;
     }
     {
         const int E = block_exp<9>(gd);
+        const int e = E - 1075 - kPopK;
         long long g[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) g[i] = fix64<kPopK>(gd[i], E);
         const long long s13 = g[1] + g[3], s24 = g[2] + g[4], s57 = g[5] + g[7], s68 = g[6] + g[8];
         const long long d57 = g[5] - g[7], d68 = g[6] - g[8];
         const long long a14 = s13 + s24, a58 = s57 + s68;
-        P.S0 = unfix64<kPopK>(a14 + a58, E);
-        P.q = unfix64<kPopK>(RM == kRatesPaperRaw ? a58 * 2 + a14 : a58 * 2 - a14 - g[0] * 4, E);
-        const double Jz = unfix64<kPopK>((g[1] - g[3]) + (d57 - d68), E);
-        P.Jz = E >= kBadE ? nan64() : Jz;
-        P.Jr = unfix64<kPopK>((g[2] - g[4]) + (d57 + d68), E);
-        P.m7 = unfix64<kPopK>(s13 - s24, E);
-        P.m8 = unfix64<kPopK>(s57 - s68, E);
+        P.S0 = norm_any(a14 + a58, e);
+        P.q = norm_any(RM == kRatesPaperRaw ? a58 * 2 + a14 : a58 * 2 - a14 - g[0] * 4, e);
+        P.Jz = norm_any((g[1] - g[3]) + (d57 - d68), e);
+        P.Jr = norm_any((g[2] - g[4]) + (d57 + d68), e);
+        P.m7 = norm_any(s13 - s24, e);
+        P.m8 = norm_any(s57 - s68, e);
+        P.bad = P.bad || E >= kBadE;
     }
 }
 
 // What the update takes from a node's column, r = j + 1/2.
 struct Col64 {
-    double r, inv_r, i6, i4, i2, r03, r3, r72;  // r, 1/r, 0.6/r, -4/(15 r), -2/r, r/0.3, 3 r, r/72
+    double r, inv_r, i4, i2;            // r, 1/r, -2/(15 r) (raw: -4/(15 r)), -2/r
+    Sf sr, s_inv_r, s_i6, r03, r3, r72;  // r, 1/r, 0.6/r, r/0.3, 3 r, r/72
 };
+template <int RM>
 __device__ __forceinline__ Col64 col64(int j, double inv_r) {
     const double r = (double)j + 0.5;
-    return Col64{r, inv_r, 0.6 * inv_r, (-4.0 / 15.0) * inv_r, -2.0 * inv_r, (1.0 / 0.3) * r, 3.0 * r, (1.0 / 72.0) * r};
+    return Col64{r, inv_r, (RM == kRatesPaperRaw ? -4.0 / 15.0 : -2.0 / 15.0) * inv_r, -2.0 * inv_r, sf_of(r),
+                 sf_of(inv_r), sf_of(0.6 * inv_r), sf_of((1.0 / 0.3) * r), sf_of(3.0 * r), sf_of((1.0 / 72.0) * r)};
 }
-// The columns of a tile in shared memory, filled once per CTA (five operations
-// per column instead of per node).
+// The columns of a tile in shared memory, filled once per CTA.
 struct ColTab64 {
-    double v[8][32];
+    double d[4][32];
+    Sf s[6][32];
     __device__ __forceinline__ void put(int x, const Col64& c) {
-        v[0][x] = c.r, v[1][x] = c.inv_r, v[2][x] = c.i6, v[3][x] = c.i4, v[4][x] = c.i2, v[5][x] = c.r03, v[6][x] = c.r3, v[7][x] = c.r72;
+        d[0][x] = c.r, d[1][x] = c.inv_r, d[2][x] = c.i4, d[3][x] = c.i2;
+        s[0][x] = c.sr, s[1][x] = c.s_inv_r, s[2][x] = c.s_i6, s[3][x] = c.r03, s[4][x] = c.r3, s[5][x] = c.r72;
     }
     __device__ __forceinline__ Col64 get(int x) const {
-        return Col64{v[0][x], v[1][x], v[2][x], v[3][x], v[4][x], v[5][x], v[6][x], v[7][x]};
+        return Col64{d[0][x], d[1][x], d[2][x], d[3][x], s[0][x], s[1][x], s[2][x], s[3][x], s[4][x], s[5][x]};
     }
 };
 
+__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+// a's integer in units of 2^e, e >= a.e
+__device__ __forceinline__ long long in_units(Sf a, int e) { return shr64(a.m, e - a.e); }
+
 // Macroscopic step, both collisions and both inverse transforms of a node of
-// column constants K; the phi window is centred on (a, b).
+// column constants K; the phi window is centred on (a, b).  What depends on
+// phi alone, the reciprocals and the square roots stay on the FP64 pipe
+// (about 50 operations), the rest runs beside it in integers.
 template <int LD, int RM>
 __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a, int b, double phi, const Col64& K,
                                          const Pre64& Q, double chz_prev, double chr_prev, double p_prev, double* fp,
-                                         double* gp, double& chz, double& chr, double& p_out) {
+                                         double* gp, double& chz_out, double& chr_out, double& p_out) {
     static_assert(RM == kRatesPaper || RM == kRatesPaperRaw, "a compile-time rate pattern");
     constexpr bool kRaw = RM == kRatesPaperRaw;
     const CaseReal<double>& P = C.pd;
     const Case64& H = C.p64;
-    double gz, gr, lap;  // 72 grad phi, 72 lap phi
-    stencil64<LD>(W, a, b, gz, gr, lap);
-    const double rho = fma(phi, H.drho, P.rho_g);               // Eq. 17
-    const double nu = fma(phi, H.dnu, P.nu_g);                  // Eq. 35
-    const double tau = fma(3.0, nu, 0.5);                       // Eq. 34
-    // 1 / tau_g, 1 / (r rho + nu rho / r) and 1 / (r rho) of Eq. 32
-    const double s = rcp64(tau);
+    Sf gz, gr, lap;  // 72 grad phi, 72 lap phi
+    bool bad;
+    stencil64<LD>(W, a, b, gz, gr, lap, bad);
+    // of phi alone: Eq. 17, 35, 34, then 1 / tau_g, 1 / (r rho + nu rho / r) and 1 / (r rho) of Eq. 32
+    const double rho_d = fma(phi, H.drho, P.rho_g);
+    const double nu = fma(phi, H.dnu, P.nu_g);
+    const double tau = fma(3.0, nu, 0.5);
+    const double s_d = rcp_in(tau);
     const double rv = fma(nu, K.inv_r, K.r);
-    const double D = rcp64(rho * rv);
-    const double irr = K.inv_r * (D * rv);
-    // Eq. 4, mu~ = mu - k d_r phi / r, and Eq. 30's F_z = r (F_s + G)_z
-    const double w = fma(phi, phi - 1.5, 0.5);                  // (phi - 1)(phi - 1/2)
-    const double mut = fma(H.beta4 * phi, w, H.mkappa * fma(gr, K.inv_r, lap));
-    const double rm = K.r72 * mut;
-    const double Fz = fma(rm, gz, K.r * ((rho - P.rho_l) * P.grav_z));
-    const double rFsr = rm * gr;
-    const double Z3 = H.drho3 * gz, R3 = H.drho3 * gr;          // 0.3 grad rho
-    const double uz = fma(0.5, Fz, Q.Jz) * irr;                 // Eq. 32 (z)
-    const double rz = rho * uz;
+    const double D_d = rcp_in(rho_d * rv);
+    const Sf rho = sf_of(rho_d), s = sf_of(s_d), D = sf_of(D_d), irr = sf_of(K.inv_r * (D_d * rv));
+    // Eq. 4: mu~ = mu - k d_r phi / r; Eq. 30's F_z = r (F_s + G)_z
+    const Sf mut = norm29(sf_of((H.beta4 * phi) * fma(phi, phi - 1.5, 0.5)) + Sf{H.mkappa_m, H.mkappa_e} * norm29(gr * K.s_inv_r + lap));
+    const Sf rm = K.r72 * mut;
+    Sf Fz = rm * gz;
+    if (abs_hi(P.grav_z) != 0) Fz = Fz + sf_of(K.r * ((rho_d - P.rho_l) * P.grav_z));
+    const Sf rFsr = rm * gr;
+    const Sf d3{H.drho3_m, H.drho3_e};
+    const Sf Z3 = d3 * gz, R3 = d3 * gr;  // 0.3 grad rho
+    const Sf uz = norm29(scale2(Fz, -1) + Q.Jz) * irr;  // Eq. 32 (z)
+    const Sf rz = rho * uz;
     // Eq. 33 with s_p = tau_g / 2 (raw: 3 tau_g / 2 - 1)
-    const double A2 = 0.4 * rho;
-    const double A0 = fma(uz, fma(-A2, uz, Z3), K.i6 * Q.S0);
-    const double sp = kRaw ? fma(1.5, tau, -1.0) : 0.5 * tau;
-    double ur, p, ps;
+    const Sf A2 = sf_of(0.4 * rho_d);
+    const Sf A0 = uz * norm29(Z3 - A2 * uz) + K.s_i6 * Q.S0;
+    const Sf A1 = norm29(sf_of(((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * K.i4) + R3);
+    // numbers that are not finite do not exist in integers: seen here, put out as NaN
+    int top = max(max(abs_hi(s_d), abs_hi(D_d)), max(abs_hi(chz_prev), abs_hi(chr_prev)));
+    Sf ur, p, ps;
     if (C.p_coupling == 1) {
-        ps = p_prev;
-        ur = fma(0.5, rFsr + ps, Q.Jr) * D;
-        p = fma(ur, fma(sp * rho, K.i4, fma(-A2, ur, R3)), A0);
+        ps = sf_of(p_prev);
+        top = max(top, abs_hi(p_prev));
+        ur = norm29(scale2(rFsr + ps, -1) + Q.Jr) * D;
+        p = norm29(ur * norm29(A1 - A2 * ur) + A0);
     } else {
         // u_r = ca + D p / 2 and p = A0 + A1 u_r - A2 u_r^2 together
-        const double ca = fma(0.5, rFsr, Q.Jr) * D;
-        const double A1 = fma(sp * rho, K.i4, R3);
-        const double t1 = A2 * ca;
-        const double qb = fma(D, fma(-0.5, A1, t1), 1.0);
-        const double qc = fma(ca, A1 - t1, A0);
-        const double disc = fma((A2 * D) * D, qc, qb * qb);
-        const bool two = __double2hiint(disc) >= 0;  // the sign bit: a comparison would take the FP64 pipe
-        p = (two ? qc + qc : qc) * rcp64(two ? qb + sqrt64(disc) : qb);
+        const Sf ca = norm29(scale2(rFsr, -1) + Q.Jr) * D;
+        const Sf t1 = A2 * ca;
+        const Sf one{1ll << 61, -61};
+        const Sf qb = norm29(one + D * norm29(t1 - scale2(A1, -1)));
+        const Sf qc = norm29(A0 + ca * norm29(A1 - t1));
+        const Sf disc = qb * qb + ((A2 * D) * D) * qc;
+        const bool two = disc.m >= 0;
+        const double qb_d = double_of(qb);
+        const double y = rcp_in(two ? qb_d + sqrt_in(double_of(disc)) : qb_d);
+        top = max(top, abs_hi(y));
+        p = scale2(qc, two ? 1 : 0) * sf_of(y);
         ps = p;
-        ur = fma(0.5 * D, p, ca);
+        ur = norm29(ca + scale2(D, -1) * p);
     }
-    const double rr = rho * ur;
-    const double Fr = fma(K.i2, nu * rr, rFsr + ps);    // Eq. 30 (r)
-    p_out = p;
+    const Sf rr = rho * ur;
+    const Sf Fr = (rFsr + ps) + sf_of(nu * K.i2) * rr;  // Eq. 30 (r)
+    p_out = double_of(p);
     // phase field (Eq. 19-23, 38): chi, then t / 3 of both directions
-    chz = Q.T * uz;
-    chr = fma(Q.T, ur, P.mob * phi);
+    const Sf T = norm_any(Q.t, Q.Ef - 1075 - kPopK);
+    const Sf chz = T * uz, chr = T * ur + sf_of(P.mob * phi);
+    chz_out = double_of(chz);
+    chr_out = double_of(chr);
     {
-        // r lambda / (3 (|grad phi| + n_eps)): the normal's factor of grad phi
+        // r lambda / (3 (|grad phi| + n_eps)): the normal's factor of grad phi (72 in both)
         const double lam = H.lam3 * (K.r * fma(-phi, phi, phi));
-        const double L = lam * rcp64(sqrt64(fma(gz, gz, gr * gr)) + H.neps72);
-        const double tz = fma(H.h3, fma(L, gz, -chz_prev), H.sh3 * chz);
-        const double tr = fma(H.h3, fma(L, gr, -chr_prev), H.sh3 * chr);
-        const double jz = fma(H.c2, Q.fz, tz), jr = fma(H.c2, Q.fr, tr);
-        const double qz = fma(0.25, tz, H.c4 * Q.fe), qr = fma(0.25, tr, H.c4 * Q.fo);
-        const double e = Q.T * (1.0 / 9.0), d = Q.T * (1.0 / 36.0);
-        const double qp = qz + qr, qm = qz - qr;
-        fp[0] = Q.T * (4.0 / 9.0);
-        fp[1] = e + jz;
-        fp[3] = e - jz;
-        fp[2] = e + jr;
-        fp[4] = e - jr;
-        fp[5] = d + qp;
-        fp[7] = d - qp;
-        fp[8] = d + qm;
-        fp[6] = d - qm;
+        const double Ld = lam * rcp_in(sqrt_in(double_of(gz * gz + gr * gr)) + H.neps72);
+        top = max(top, abs_hi(Ld));
+        const Sf L = sf_of(Ld);
+        const Sf h3{H.h3_m, H.h3_e}, sh3{H.sh3_m, H.sh3_e};
+        const Sf tz = h3 * norm29(L * gz - sf_of(chz_prev)) + sh3 * chz;
+        const Sf tr = h3 * norm29(L * gr - sf_of(chr_prev)) + sh3 * norm29(chr);
+        // the sums of the inverse transform in units of the largest part, 2^E
+        // (the block's values take up to 63 bits)
+        const int eb = Q.Ef - 1075 - kPopK;
+        const int E = max(max(max(tz.e, tr.e), eb), -990), sb = E - eb;
+        bad = bad || E > 890;
+        const long long e = ninth_double(shr64(Q.t, sb));
+        const long long tz0 = in_units(tz, E), tr0 = in_units(tr, E);
+        const long long jz = mul62(shr64(Q.fz, sb), H.c2) + tz0, jr = mul62(shr64(Q.fr, sb), H.c2) + tr0;
+        const long long qz = mul62(shr64(Q.fe, sb), H.c4) + (tz0 >> 2), qr = mul62(shr64(Q.fo, sb), H.c4) + (tr0 >> 2);
+        const long long d = e >> 2, qp = qz + qr, qm = qz - qr;
+        fp[0] = double_in(e, E + 2);
+        fp[1] = double_in(e + jz, E);
+        fp[3] = double_in(e - jz, E);
+        fp[2] = double_in(e + jr, E);
+        fp[4] = double_in(e - jr, E);
+        fp[5] = double_in(d + qp, E);
+        fp[7] = double_in(d - qp, E);
+        fp[8] = double_in(d + qm, E);
+        fp[6] = double_in(d - qm, E);
     }
     // hydrodynamics (Eq. 24, 36-37)
-    const double az = K.r03 * Z3, br = fma(K.r03, R3, rho);               // grad (r rho)
-    const double P1 = uz * az, P2 = ur * br, udr = P1 + P2;
-    const double E1 = rz * uz, E2 = rr * ur, E = E1 + E2;       // rho u^2
-    const double pK = fma(2.0, p, E);
-    const double c = 1.0 - s, h2 = 2.0 - s;                     // 1 - s, 2 (1 - s/2)
-    const double h6 = h2 * (1.0 / 6.0);
-    const double jz = Q.Jz + Fz, jr = Q.Jr + Fr;                // unit rates on the momenta
-    const double m7 = fma(2.0 * h6, P1 - P2, fma(s, K.r * (E1 - E2), c * Q.m7));
-    const double m8 = fma(h6, fma(uz, br, ur * az), fma(s, (K.r * rr) * uz, c * Q.m8));
-    const double m0 = 0.5 * (udr - rr);
-    double ep, em, dp, dm;
+    const Sf az = K.r03 * Z3, br = norm29(K.r03 * R3 + rho);      // grad (r rho)
+    const Sf P1 = uz * az, P2 = ur * br, udr = P1 + P2;
+    const Sf E1 = rz * uz, E2 = rr * ur, EE = E1 + E2;          // rho u^2
+    const Sf pK = scale2(p, 1) + EE;
+    const Sf c = sf_of(1.0 - s_d), h2 = sf_of(2.0 - s_d), h6 = sf_of((2.0 - s_d) * (1.0 / 6.0));  // 1 - s, 2 (1 - s/2)
+    const Sf jz = Q.Jz + Fz, jr = Q.Jr + Fr;                    // unit rates on the momenta
+    const Sf m7 = (c * Q.m7 + s * (K.sr * norm29(E1 - E2))) + scale2(h6, 1) * norm29(P1 - P2);
+    const Sf m8 = (c * Q.m8 + s * norm29((K.sr * rr) * uz)) + h6 * norm29(uz * br + ur * az);
+    const Sf m0 = scale2(udr - rr, -1);
     if constexpr (kRaw) {
         // raw moments: k_3 = sum c^2 g relaxes with 1/tau_g, k_0 and k_8 take
         // equilibrium and half the source
-        const double k3 = fma(2.0 * h6, fma(2.0, udr, -rr), fma(s, K.r * pK, c * Q.q));
-        const double k8 = fma(K.r3 * (1.0 / 9.0), p + E, fma(3.0, udr, -rr) * (1.0 / 18.0));
-        gp[0] = (m0 - k3) + k8;
-        const double ax = fma(-0.5, k8, 0.25 * k3);
-        ep = fma(0.25, m7, ax);
-        em = fma(-0.25, m7, ax);
-        dp = 0.25 * (k8 + m8);
-        dm = 0.25 * (k8 - m8);
+        const Sf rr3{third64(rr.m), rr.e};
+        const Sf k3 = (c * Q.q + s * (K.sr * norm29(pK))) + scale2(h6, 1) * norm29(scale2(udr, 1) - rr);
+        const Sf w = K.r3 * norm29(p + EE);   // 3 r (p + rho u^2)
+        const Sf v = udr - rr3;             // 6 times the rest of k_8
+        const int E = max(-994, max(max(max(k3.e, m0.e), max(w.e, v.e)), max(max(m7.e, m8.e), max(jz.e, jr.e)))) + 4;
+        bad = bad || E > 890;
+        const long long M0 = in_units(m0, E), K3 = in_units(k3, E), M7 = in_units(m7, E), M8 = in_units(m8, E);
+        const long long K8 = ninth64(in_units(w, E)) + (third64(in_units(v, E)) >> 1);
+        const long long JZ = in_units(jz, E), JR = in_units(jr, E);
+        // 12 g in units of 2^E
+        const long long ax = K3 * 3 - K8 * 6, p7 = M7 * 3;
+        gp[0] = double_in(M0 - K3 + K8, E);
+        gp[1] = double_in(third64(ax + p7 + JZ * 4), E - 2);
+        gp[3] = double_in(third64(ax + p7 - JZ * 4), E - 2);
+        gp[2] = double_in(third64(ax - p7 + JR * 4), E - 2);
+        gp[4] = double_in(third64(ax - p7 - JR * 4), E - 2);
+        const long long dp = (K8 + M8) * 3, dm = (K8 - M8) * 3;
+        gp[5] = double_in(third64(dp + JZ + JR), E - 2);
+        gp[7] = double_in(third64(dp - JZ - JR), E - 2);
+        gp[8] = double_in(third64(dm + JZ - JR), E - 2);
+        gp[6] = double_in(third64(dm - JZ + JR), E - 2);
     } else {
-        const double m1 = fma(h2, rr, fma(s, K.r3 * pK, c * Q.q));
-        const double m2 = fma(-K.r3, pK + p, -(m0 + rr));
-        const double n0 = m0 * (1.0 / 9.0);
-        gp[0] = fma(1.0 / 9.0, m2 - m1, n0);
-        const double e = fma(-1.0 / 36.0, m1, fma(-1.0 / 18.0, m2, n0));
-        const double d = fma(1.0 / 18.0, m1, fma(1.0 / 36.0, m2, n0));
-        ep = fma(0.25, m7, e);
-        em = fma(-0.25, m7, e);
-        dp = fma(0.25, m8, d);
-        dm = fma(-0.25, m8, d);
+        const Sf m1 = (c * Q.q + s * (K.r3 * norm29(pK))) + h2 * rr;
+        const Sf m2 = neg((K.r3 * norm29(pK + p)) + (m0 + rr));
+        // 36 g = 4 m0 - m1 - 2 m2 +- 9 m7 +- 12 j (axes), 4 m0 + 2 m1 + m2 +- 9 m8
+        // +- 3 j (diagonals), 4 (m0 - m1 + m2) (rest), in units of 2^E: the
+        // coefficients add up to 28 at most
+        const int E = max(-994, max(max(max(m0.e, m1.e), max(m2.e, jz.e)), max(max(m7.e, m8.e), jr.e))) + 4;
+        bad = bad || E > 890;
+        const long long M0 = in_units(m0, E) * 4, M1 = in_units(m1, E), M2 = in_units(m2, E);
+        const long long M7 = in_units(m7, E) * 9, M8 = in_units(m8, E) * 9;
+        const long long JZ = in_units(jz, E) * 3, JR = in_units(jr, E) * 3;
+        const long long ax = M0 - M1 - M2 * 2, dg = M0 + M1 * 2 + M2;
+        gp[0] = double_in(ninth64(M0 - (M1 - M2) * 4), E - 2);
+        gp[1] = double_in(ninth64(ax + M7 + JZ * 4), E - 2);
+        gp[3] = double_in(ninth64(ax + M7 - JZ * 4), E - 2);
+        gp[2] = double_in(ninth64(ax - M7 + JR * 4), E - 2);
+        gp[4] = double_in(ninth64(ax - M7 - JR * 4), E - 2);
+        gp[5] = double_in(ninth64(dg + M8 + JZ + JR), E - 2);
+        gp[7] = double_in(ninth64(dg + M8 - JZ - JR), E - 2);
+        gp[8] = double_in(ninth64(dg - M8 + JZ - JR), E - 2);
+        gp[6] = double_in(ninth64(dg - M8 - JZ + JR), E - 2);
     }
-    const double q1 = jz + jr, q2 = jz - jr;
-    gp[1] = fma(1.0 / 3.0, jz, ep);
-    gp[3] = fma(-1.0 / 3.0, jz, ep);
-    gp[2] = fma(1.0 / 3.0, jr, em);
-    gp[4] = fma(-1.0 / 3.0, jr, em);
-    gp[5] = fma(1.0 / 12.0, q1, dp);
-    gp[7] = fma(-1.0 / 12.0, q1, dp);
-    gp[8] = fma(1.0 / 12.0, q2, dm);
-    gp[6] = fma(-1.0 / 12.0, q2, dm);
+    if (bad || Q.bad || top >= 0x7ff00000) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fp[i] = gp[i] = nan64();
+        chz_out = chr_out = p_out = nan64();
+    }
 }
 
 }  // namespace axilbm

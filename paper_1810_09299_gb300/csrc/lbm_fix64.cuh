@@ -21,6 +21,17 @@ namespace axilbm {
 constexpr int kMinE = 64, kBadE = 2030;
 
 __device__ __forceinline__ int exp64(double x) { return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu); }
+// shifts whose amounts may exceed 63 (PTX: all bits leave, or the sign fills)
+__device__ __forceinline__ unsigned long long shr64u(unsigned long long v, int s) {
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+    return r;
+}
+__device__ __forceinline__ long long shr64(long long v, int s) {
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+    return r;
+}
 __device__ __forceinline__ double nan64() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 // x in the block of exponent E >= exp64(x), truncated towards zero.
@@ -29,7 +40,7 @@ __device__ __forceinline__ long long fix64(double x, int E) {
     const int hi = __double2hiint(x);
     const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
     const unsigned long long m = (((unsigned long long)mh << 32) | (uint32_t)__double2loint(x)) << K;
-    const long long v = (long long)(m >> min(E - exp64(x), 63)), sg = (long long)(hi >> 31);
+    const long long v = (long long)shr64u(m, E - exp64(x)), sg = (long long)(hi >> 31);
     return (v ^ sg) - sg;
 }
 // v 2^(E - 1075 - K) as a double (rounded to nearest, ties away from zero).
@@ -62,5 +73,113 @@ __device__ __forceinline__ double sum64(const double* f) {
     const double r = unfix64<kPopK>(t, E);
     return E >= kBadE ? nan64() : r;
 }
+
+// ---------------------------------------------------------------- numbers of 62 bits
+// x = m 2^e with |m| < 2^62 in integer registers, for products and sums that
+// would wait for the FP64 pipe: a product is 10 integer instructions (3 of
+// them wide multiply-adds), a sum 9, against 0.62 cycles per node and SM for an
+// FP64 operation of either kind.  A product keeps all but 1 bit of normalised
+// operands (|m| >= 2^61) and is exact to about 2^-59 of itself; a sum is exact to
+// the last place of its larger operand.  A factor that may have cancelled
+// (a sum) is normalised first; zero carries a large negative exponent, so that
+// it never shifts the other operand of a sum.
+struct Sf {
+    long long m;
+    int e;
+};
+constexpr int kZeroE = -(1 << 17);
+
+// a b 2^-62, |a|, |b| < 2^62 (the low words' product, at most 4 units, is left out)
+__device__ __forceinline__ long long mul62(long long a, long long b) {
+    const int ah = (int)(a >> 32), bh = (int)(b >> 32);
+    const uint32_t al = (uint32_t)a, bl = (uint32_t)b;
+    const long long cross = (long long)ah * (int)(bl >> 1) + (long long)bh * (int)(al >> 1);
+    return (long long)(ah * 2) * (bh * 2) + (cross >> 29);
+}
+__device__ __forceinline__ Sf operator*(Sf a, Sf b) { return Sf{mul62(a.m, b.m), a.e + b.e + 62}; }
+__device__ __forceinline__ Sf operator+(Sf a, Sf b) {
+    const int e = max(a.e, b.e) + 1;
+    return Sf{shr64(a.m, e - a.e) + shr64(b.m, e - b.e), e};
+}
+__device__ __forceinline__ Sf operator-(Sf a, Sf b) {
+    const int e = max(a.e, b.e) + 1;
+    return Sf{shr64(a.m, e - a.e) - shr64(b.m, e - b.e), e};
+}
+__device__ __forceinline__ Sf scale2(Sf a, int n) { return Sf{a.m, a.e + n}; }  // a 2^n
+__device__ __forceinline__ Sf neg(Sf a) { return Sf{-a.m, a.e}; }
+// The same value with 2^61 <= |m| < 2^62 (zero: see above).
+__device__ __forceinline__ Sf norm(Sf a) {
+    int sh;  // places from the leading non-sign bit to bit 63; -1 for 0 and -1
+    asm("bfind.shiftamt.s64 %0, %1;" : "=r"(sh) : "l"(a.m));
+    Sf r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r.m) : "l"(a.m), "r"(sh - 2));
+    r.e = sh < 0 ? kZeroE : a.e - (sh - 2);
+    return r;
+}
+// The same by at most 29 places, from the high word alone: enough for a factor
+// that is a sum, since bits further down carry the sum's own rounding.
+__device__ __forceinline__ Sf norm29(Sf a) {
+    uint32_t sh;
+    asm("bfind.shiftamt.s32 %0, %1;" : "=r"(sh) : "r"((int)(a.m >> 32)));
+    const int n = (int)min(sh, 31u) - 2;
+    return Sf{a.m << n, a.e - n};
+}
+// An ordinary double (zero and subnormal numbers count as numbers near 2^-1022;
+// infinities and NaN: the caller replaces the result).
+__device__ __forceinline__ Sf sf_of(double x) {
+    const int hi = __double2hiint(x);
+    const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
+    const long long v = (long long)((((unsigned long long)mh << 32) | (uint32_t)__double2loint(x)) << 9);
+    const long long sg = (long long)(hi >> 31);
+    return Sf{(v ^ sg) - sg, exp64(x) - 1084};
+}
+// m 2^e as a double, rounded to nearest, for -1000 <= e <= 900.
+__device__ __forceinline__ double double_in(long long m, int e) {
+    const long long sg = m >> 63;
+    unsigned long long x = (unsigned long long)((m ^ sg) - sg);
+    const int n = __clzll((long long)x);
+    x <<= n & 63;
+    unsigned long long b = (x >> 11) + ((x >> 10) & 1ull) + ((unsigned long long)(uint32_t)(e - n + 1085) << 52);
+    b |= (unsigned long long)sg << 63;
+    return m == 0 ? 0.0 : __longlong_as_double((long long)b);
+}
+// The same for any e: below the normal numbers zero, above them NaN.
+__device__ __forceinline__ double double_of(Sf a) {
+    const double d = double_in(a.m, min(max(a.e, -1000), 900));
+    return a.e < -1000 ? 0.0 : (a.e > 900 ? nan64() : d);
+}
+// 1 / x and sqrt(x) of lbm_device.cuh's rcp64 and sqrt64 for numbers the
+// integers above can hold (x normal, or for the root zero): without their IEEE
+// forms, whose instructions a warp passes through even when no lane needs
+// them.  Zero (rcp), infinities and NaN give NaN.
+__device__ __forceinline__ double rcp_in(double x) {
+    double y0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double e = fma(-x, y0, 1.0);
+    return fma(fma(e, e, e), y0, y0);
+}
+__device__ __forceinline__ double sqrt_in(double x) {
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double s = x * y0;
+    const double e = fma(-s, y0, 1.0);
+    const double y = fma(s * e, fma(0.375, e, 0.5), s);
+    return (((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x)) == 0u ? 0.0 : y;
+}
+// v / 3 and v / 9: v times 2^64 / 3 (or 9), words H and L, without the low words' product
+template <uint32_t H, uint32_t L>
+__device__ __forceinline__ long long mul_const(long long v) {
+    const int h = (int)(v >> 32);
+    const long long t = (long long)((unsigned long long)(uint32_t)v * H) + (long long)h * (int)L;
+    return (long long)h * (int)H + (t >> 32);
+}
+__device__ __forceinline__ long long third64(long long v) { return mul_const<0x55555555u, 0x55555555u>(v); }
+__device__ __forceinline__ long long ninth64(long long v) { return mul_const<0x1c71c71cu, 0x71c71c72u>(v); }
+// v times the double nearest 1/9 (5.6e-17 below it), for the weights of the phase
+// field: the conserved sum of f takes this factor every step.  With 1/9 itself it
+// drifts by 4e-15 instead of 1.1e-13 over 2000 steps, but the oracle and the
+// general kernels hold the weights as doubles, and on the 64 x 128 static drop runs
+// with and without that drift part by 2e-12 (phi) and 1e-11 (p) in that time.
+__device__ __forceinline__ long long ninth_double(long long v) { return mul_const<0x1c71c71cu, 0x71c71c00u>(v); }
 
 }  // namespace axilbm

@@ -132,13 +132,16 @@ __device__ __forceinline__ void ring_cell(int q, int& a, int& b) {
 #ifndef AXILBM_GRID16_CTAS
 #define AXILBM_GRID16_CTAS 4
 #endif
+#ifndef AXILBM_F64_CTAS
+#define AXILBM_F64_CTAS 2
+#endif
 template <class Codec, int BZ, int RM>
 constexpr int step_min_blocks() {
     constexpr int bz8 = Codec::kGrid ? AXILBM_GRID16_CTAS
                         : (RM == kRatesPaperRaw && sizeof(typename Codec::PT) == 2)
                             ? 4
                             : (sizeof(typename Codec::PT) == 2 ? AXILBM_STEP16_CTAS : 5);
-    return sizeof(typename Codec::Real) == 8 ? 1
+    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ >= 16 ? 1 : AXILBM_F64_CTAS * (8 / BZ)))
            : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
                 : (BZ >= 16 ? 1 : (BZ >= 8 ? AXILBM_GENERAL_CTAS : 2 * AXILBM_GENERAL_CTAS));
 }
@@ -572,7 +575,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     // FP64 pipe); the same correctly rounded quotients the nodes would form
     constexpr bool kInvrTable = sizeof(Real) == 8;
     __shared__ Real s_invr[kInvrTable ? LD : 1];
-    __shared__ double s_col_raw[kU64 ? sizeof(ColTab64) / 8 : 1];
+    __shared__ __align__(16) double s_col_raw[kU64 ? sizeof(ColTab64) / 8 : 1];
     ColTab64& s_col = *reinterpret_cast<ColTab64*>(s_col_raw);
     // 16-bit storage: the column constants of the window's columns
     constexpr bool kG = Codec::kGrid;
@@ -689,7 +692,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
             const Real ir = rcp_((Real)jm + (Real)0.5);
             s_invr[q] = ir;
             if constexpr (kU64) {
-                if (q >= 2 && q < kTR + 2) s_col.put(q - 2, col64(jm, ir));
+                if (q >= 2 && q < kTR + 2) s_col.put(q - 2, col64<RM>(jm, ir));
             }
         }
     }
@@ -1374,7 +1377,7 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
                 Pre64 pre;
                 pre64<RM>(f, graw, pre);
                 const Real ir = rcp_(r);
-                node_update64<RM, LD>(C, V, W, threadIdx.y + 2, threadIdx.x + 2, pre.T * ir, k, j, loc, col64(j, ir),
+                node_update64<RM, LD>(C, V, W, threadIdx.y + 2, threadIdx.x + 2, pre.T * ir, k, j, loc, col64<RM>(j, ir),
                                       pre, chz_prev, chr_prev, p_prev);
             } else {
                 node_update<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, threadIdx.x + 2, k, j, loc, f0raw, fraw,
