@@ -1,16 +1,25 @@
 // lbm_f64.cuh -- the FP64 node update for the two compile-time rate patterns
 // (kRatesPaper, kRatesPaperRaw), written for the fewest FP64 operations.
 //
-// What bounds it: the FP64 pipe, which issues 1.6 operations per SM and cycle
-// on this chip (integer instructions: about 100).  The general form of
-// lbm_device.cuh takes 383 FP64 operations per node (0.71 ns of the whole GPU, 86 %
-// of it that pipe).  Here (ncu counters, 32 batched cases of 1.89 M nodes, one
-// step): 280 by the algebra below, 1342 -> 1005 us; 202 with the sums of
-// populations and of the phi stencil in 64-bit integers (lbm_fix64.cuh), 724 us,
-// the pipe still 87 % busy.  The integers also round once where the sums rounded
-// at every addition: one step's error against 80-bit arithmetic fell from
-// 1.25e-16 to 0.88e-16 (f) and from 2.1e-15 to 0.75e-15 (g) of their 2-norms on
-// a 64 x 128 oscillating drop.
+// What bounds it: the FP64 pipe issues 1.6 operations per SM and cycle on this
+// chip, the integer pipes about 100 instructions.  The general form of
+// lbm_device.cuh takes 383 FP64 operations per node and is bound by that pipe.
+// Here the sums of populations and of the phi stencil, both collisions and both
+// inverse transforms run in 64-bit integers (lbm_fix64.cuh) beside about 60 FP64
+// operations: what depends on phi alone, the reciprocals and the roots, and the
+// conversion of the nine g.  32 batched cases (1.89 M nodes), us a step:
+//   general form, 383 operations per node                          1342
+//   the algebra below, 280                                         1005
+//   sums of populations and of the stencil in integers, 202         724
+//   collisions and inverse transforms in integers, 83               516
+//   no IEEE fallbacks, cheaper conversions and normalisations, 55   408
+//   shared alignments, the nine g converted on the FP64 pipe, 61    383
+// (all eighteen converted there: 399, none: 397).  Now the ALU is 58 % and the
+// FP64 pipe 48 % busy (ncu).  More warps do not help: 3 CTAs of 80 registers
+// (460 bytes of spill) 387 us; with 4-row tiles 4, 5, 6 CTAs 446, 442, 441.
+// The error of one step against 80-bit arithmetic is below that of the general
+// form: 7.8e-17 against 1.25e-16 (f), 7.4e-16 against 2.1e-15 (g), 1.0e-16
+// against 2.5e-16 (chi) of their 2-norms on a 64 x 128 oscillating drop.
 // The rate pattern fixes:
 //   * the phase-field collision acts on four differences of populations, not
 //     on nine moments: with t = s chi + (1 - s/2) R and T = r phi,
@@ -202,7 +211,8 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     const Sf rFsr = rm * gr;
     const Sf d3{H.drho3_m, H.drho3_e};
     const Sf Z3 = d3 * gz, R3 = d3 * gr;  // 0.3 grad rho
-    const Sf uz = norm29(scale2(Fz, -1) + Q.Jz) * irr;  // Eq. 32 (z)
+    const Two JFz = align(Q.Jz, Fz);
+    const Sf uz = norm29(Sf{JFz.a + (JFz.b >> 1), JFz.e}) * irr;  // Eq. 32 (z)
     const Sf rz = rho * uz;
     // Eq. 33 with s_p = tau_g / 2 (raw: 3 tau_g / 2 - 1)
     const Sf A2 = sf_of(0.4 * rho_d);
@@ -221,8 +231,9 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         const Sf ca = norm29(scale2(rFsr, -1) + Q.Jr) * D;
         const Sf t1 = A2 * ca;
         const Sf one{1ll << 61, -61};
-        const Sf qb = norm29(one + D * norm29(t1 - scale2(A1, -1)));
-        const Sf qc = norm29(A0 + ca * norm29(A1 - t1));
+        const Two tA = align(t1, A1);
+        const Sf qb = norm29(one + D * norm29(Sf{tA.a - (tA.b >> 1), tA.e}));
+        const Sf qc = norm29(A0 + ca * norm29(Sf{tA.b - tA.a, tA.e}));
         const Sf disc = qb * qb + ((A2 * D) * D) * qc;
         const bool two = disc.m >= 0;
         const double qb_d = double_of(qb);
@@ -271,20 +282,23 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     }
     // hydrodynamics (Eq. 24, 36-37)
     const Sf az = K.r03 * Z3, br = norm29(K.r03 * R3 + rho);      // grad (r rho)
-    const Sf P1 = uz * az, P2 = ur * br, udr = P1 + P2;
-    const Sf E1 = rz * uz, E2 = rr * ur, EE = E1 + E2;          // rho u^2
-    const Sf pK = scale2(p, 1) + EE;
-    const Sf c = sf_of(1.0 - s_d), h2 = sf_of(2.0 - s_d), h6 = sf_of((2.0 - s_d) * (1.0 / 6.0));  // 1 - s, 2 (1 - s/2)
-    const Sf jz = Q.Jz + Fz, jr = Q.Jr + Fr;                    // unit rates on the momenta
-    const Sf m7 = (c * Q.m7 + s * (K.sr * norm29(E1 - E2))) + scale2(h6, 1) * norm29(P1 - P2);
+    const Two PP = align(uz * az, ur * br);
+    const Sf udr{PP.a + PP.b, PP.e};
+    const Two E12 = align(rz * uz, rr * ur);
+    const Two pE = align(scale2(p, 1), Sf{E12.a + E12.b, E12.e});  // 2 p and rho u^2
+    const Sf pK = norm29(Sf{pE.a + pE.b, pE.e});
+    const Two s1 = align(Sf{1ll << 61, -61}, s);                // 1 - s, 2 (1 - s/2) and a sixth of that
+    const Sf c = norm29(Sf{s1.a - s1.b, s1.e}), h2 = norm29(Sf{s1.a - (s1.b >> 1), s1.e + 1}), h6{third64(h2.m), h2.e - 1};
+    const Sf jz{JFz.a + JFz.b, JFz.e}, jr = Q.Jr + Fr;                    // unit rates on the momenta
+    const Sf m7 = (c * Q.m7 + s * (K.sr * norm29(Sf{E12.a - E12.b, E12.e}))) + scale2(h6, 1) * norm29(Sf{PP.a - PP.b, PP.e});
     const Sf m8 = (c * Q.m8 + s * norm29((K.sr * rr) * uz)) + h6 * norm29(uz * br + ur * az);
     const Sf m0 = scale2(udr - rr, -1);
     if constexpr (kRaw) {
         // raw moments: k_3 = sum c^2 g relaxes with 1/tau_g, k_0 and k_8 take
         // equilibrium and half the source
         const Sf rr3{third64(rr.m), rr.e};
-        const Sf k3 = (c * Q.q + s * (K.sr * norm29(pK))) + scale2(h6, 1) * norm29(scale2(udr, 1) - rr);
-        const Sf w = K.r3 * norm29(p + EE);   // 3 r (p + rho u^2)
+        const Sf k3 = (c * Q.q + s * (K.sr * pK)) + scale2(h6, 1) * norm29(scale2(udr, 1) - rr);
+        const Sf w = K.r3 * norm29(Sf{(pE.a >> 1) + pE.b, pE.e});   // 3 r (p + rho u^2)
         const Sf v = udr - rr3;             // 6 times the rest of k_8
         const int E = max(-994, max(max(max(k3.e, m0.e), max(w.e, v.e)), max(max(m7.e, m8.e), max(jz.e, jr.e)))) + 4;
         bad = bad || E > 890;
@@ -293,19 +307,19 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         const long long JZ = in_units(jz, E), JR = in_units(jr, E);
         // 12 g in units of 2^E
         const long long ax = K3 * 3 - K8 * 6, p7 = M7 * 3;
-        gp[0] = double_in(M0 - K3 + K8, E);
-        gp[1] = double_in(third64(ax + p7 + JZ * 4), E - 2);
-        gp[3] = double_in(third64(ax + p7 - JZ * 4), E - 2);
-        gp[2] = double_in(third64(ax - p7 + JR * 4), E - 2);
-        gp[4] = double_in(third64(ax - p7 - JR * 4), E - 2);
+        gp[0] = double_cvt(M0 - K3 + K8, E);
+        gp[1] = double_cvt(third64(ax + p7 + JZ * 4), E - 2);
+        gp[3] = double_cvt(third64(ax + p7 - JZ * 4), E - 2);
+        gp[2] = double_cvt(third64(ax - p7 + JR * 4), E - 2);
+        gp[4] = double_cvt(third64(ax - p7 - JR * 4), E - 2);
         const long long dp = (K8 + M8) * 3, dm = (K8 - M8) * 3;
-        gp[5] = double_in(third64(dp + JZ + JR), E - 2);
-        gp[7] = double_in(third64(dp - JZ - JR), E - 2);
-        gp[8] = double_in(third64(dm + JZ - JR), E - 2);
-        gp[6] = double_in(third64(dm - JZ + JR), E - 2);
+        gp[5] = double_cvt(third64(dp + JZ + JR), E - 2);
+        gp[7] = double_cvt(third64(dp - JZ - JR), E - 2);
+        gp[8] = double_cvt(third64(dm + JZ - JR), E - 2);
+        gp[6] = double_cvt(third64(dm - JZ + JR), E - 2);
     } else {
-        const Sf m1 = (c * Q.q + s * (K.r3 * norm29(pK))) + h2 * rr;
-        const Sf m2 = neg((K.r3 * norm29(pK + p)) + (m0 + rr));
+        const Sf m1 = (c * Q.q + s * (K.r3 * pK)) + h2 * rr;
+        const Sf m2 = neg((K.r3 * norm29(Sf{((pE.a + pE.b) >> 1) + (pE.a >> 2), pE.e + 1})) + (m0 + rr));
         // 36 g = 4 m0 - m1 - 2 m2 +- 9 m7 +- 12 j (axes), 4 m0 + 2 m1 + m2 +- 9 m8
         // +- 3 j (diagonals), 4 (m0 - m1 + m2) (rest), in units of 2^E: the
         // coefficients add up to 28 at most
@@ -315,15 +329,15 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         const long long M7 = in_units(m7, E) * 9, M8 = in_units(m8, E) * 9;
         const long long JZ = in_units(jz, E) * 3, JR = in_units(jr, E) * 3;
         const long long ax = M0 - M1 - M2 * 2, dg = M0 + M1 * 2 + M2;
-        gp[0] = double_in(ninth64(M0 - (M1 - M2) * 4), E - 2);
-        gp[1] = double_in(ninth64(ax + M7 + JZ * 4), E - 2);
-        gp[3] = double_in(ninth64(ax + M7 - JZ * 4), E - 2);
-        gp[2] = double_in(ninth64(ax - M7 + JR * 4), E - 2);
-        gp[4] = double_in(ninth64(ax - M7 - JR * 4), E - 2);
-        gp[5] = double_in(ninth64(dg + M8 + JZ + JR), E - 2);
-        gp[7] = double_in(ninth64(dg + M8 - JZ - JR), E - 2);
-        gp[8] = double_in(ninth64(dg - M8 + JZ - JR), E - 2);
-        gp[6] = double_in(ninth64(dg - M8 - JZ + JR), E - 2);
+        gp[0] = double_cvt(ninth64(M0 - (M1 - M2) * 4), E - 2);
+        gp[1] = double_cvt(ninth64(ax + M7 + JZ * 4), E - 2);
+        gp[3] = double_cvt(ninth64(ax + M7 - JZ * 4), E - 2);
+        gp[2] = double_cvt(ninth64(ax - M7 + JR * 4), E - 2);
+        gp[4] = double_cvt(ninth64(ax - M7 - JR * 4), E - 2);
+        gp[5] = double_cvt(ninth64(dg + M8 + JZ + JR), E - 2);
+        gp[7] = double_cvt(ninth64(dg + M8 - JZ - JR), E - 2);
+        gp[8] = double_cvt(ninth64(dg - M8 + JZ - JR), E - 2);
+        gp[6] = double_cvt(ninth64(dg - M8 - JZ + JR), E - 2);
     }
     if (bad || Q.bad || top >= 0x7ff00000) {
 #pragma unroll

@@ -12,9 +12,8 @@ namespace axilbm {
 // K extra bits below the last place of the largest value), added exactly, and
 // the result is rounded once to a double.  An addition costs two integer
 // instructions of the ~100 per SM and cycle instead of one of the 1.6 FP64
-// operations, a conversion into the block 0.27 and out of it 0.31 cycles per
-// node and SM against 0.62 for an FP64 operation, and both run beside the FP64
-// pipe.  The rounding is at most that of the FP64 sums it replaces: the bits a
+// operations, a conversion into the block 0.21 and out of it 0.3 cycles per node
+// and SM against 0.62 for an FP64 operation, and both run beside the FP64 pipe.  The rounding is at most that of the FP64 sums it replaces: the bits a
 // smaller value loses lie K bits below the largest one's last place.
 // E is at least kMinE (values below 2^-959 lose their low bits, as subnormal
 // numbers do); from kBadE on (2^1007, infinities, NaN) the results are NaN.
@@ -76,13 +75,14 @@ __device__ __forceinline__ double sum64(const double* f) {
 
 // ---------------------------------------------------------------- numbers of 62 bits
 // x = m 2^e with |m| < 2^62 in integer registers, for products and sums that
-// would wait for the FP64 pipe: a product is 10 integer instructions (3 of
-// them wide multiply-adds), a sum 9, against 0.62 cycles per node and SM for an
-// FP64 operation of either kind.  A product keeps all but 1 bit of normalised
-// operands (|m| >= 2^61) and is exact to about 2^-59 of itself; a sum is exact to
-// the last place of its larger operand.  A factor that may have cancelled
-// (a sum) is normalised first; zero carries a large negative exponent, so that
-// it never shifts the other operand of a sum.
+// would wait for the FP64 pipe.  Cycles per node and SM (measured): a product
+// 0.22 (three wide multiply-adds at 16 per SM and cycle), a sum 0.09, norm29
+// 0.08, norm 0.19, sf_of 0.15, against 0.62 for an FP64 operation of either
+// kind.  A product keeps all but 1 bit of normalised operands (|m| >= 2^61) and
+// is exact to about 2^-59 of itself; a sum is exact to the last place of its
+// larger operand.  A factor that may have cancelled (a sum) is normalised
+// first; zero carries a large negative exponent, so that it never shifts the
+// other operand of a sum.
 struct Sf {
     long long m;
     int e;
@@ -104,6 +104,15 @@ __device__ __forceinline__ Sf operator+(Sf a, Sf b) {
 __device__ __forceinline__ Sf operator-(Sf a, Sf b) {
     const int e = max(a.e, b.e) + 1;
     return Sf{shr64(a.m, e - a.e) - shr64(b.m, e - b.e), e};
+}
+// a and b as integers of one unit 2^e, each below 2^61, for several sums of them
+struct Two {
+    long long a, b;
+    int e;
+};
+__device__ __forceinline__ Two align(Sf a, Sf b) {
+    const int e = max(a.e, b.e) + 1;
+    return Two{shr64(a.m, e - a.e), shr64(b.m, e - b.e), e};
 }
 __device__ __forceinline__ Sf scale2(Sf a, int n) { return Sf{a.m, a.e + n}; }  // a 2^n
 __device__ __forceinline__ Sf neg(Sf a) { return Sf{-a.m, a.e}; }
@@ -133,19 +142,27 @@ __device__ __forceinline__ Sf sf_of(double x) {
     const long long sg = (long long)(hi >> 31);
     return Sf{(v ^ sg) - sg, exp64(x) - 1084};
 }
-// m 2^e as a double, rounded to nearest, for -1000 <= e <= 900.
+// m 2^e as a double, rounded to nearest, for |m| < 2^63 and -1000 <= e <= 900.
 __device__ __forceinline__ double double_in(long long m, int e) {
     const long long sg = m >> 63;
-    unsigned long long x = (unsigned long long)((m ^ sg) - sg);
-    const int n = __clzll((long long)x);
-    x <<= n & 63;
-    unsigned long long b = (x >> 11) + ((x >> 10) & 1ull) + ((unsigned long long)(uint32_t)(e - n + 1085) << 52);
-    b |= (unsigned long long)sg << 63;
-    return m == 0 ? 0.0 : __longlong_as_double((long long)b);
+    const unsigned long long x = (unsigned long long)((m ^ sg) - sg);
+    const int n = __clzll((long long)x);  // 1 .. 64
+    unsigned long long y;                 // the leading bit at 62, ten bits below the last place
+    asm("shl.b64 %0, %1, %2;" : "=l"(y) : "l"(x), "r"(n - 1));
+    y = (y + 0x200ull) >> 10;
+    const uint32_t hi = (uint32_t)(y >> 32) + ((uint32_t)(e - n + 1085) << 20);
+    return __hiloint2double((int)((n == 64 ? 0u : hi) | ((uint32_t)sg & 0x80000000u)), (int)(uint32_t)y);
+}
+// The same by the FP64 pipe's conversion (0.53 cycles per node and SM, against
+// 0.3 on the integer pipes, which have more to do).
+__device__ __forceinline__ double double_cvt(long long m, int e) {
+    const double d = __ll2double_rn(m);
+    const int hi = __double2hiint(d);
+    return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(d));
 }
 // The same for any e: below the normal numbers zero, above them NaN.
 __device__ __forceinline__ double double_of(Sf a) {
-    const double d = double_in(a.m, min(max(a.e, -1000), 900));
+    const double d = double_in(a.m, a.e);
     return a.e < -1000 ? 0.0 : (a.e > 900 ? nan64() : d);
 }
 // 1 / x and sqrt(x) of lbm_device.cuh's rcp64 and sqrt64 for numbers the

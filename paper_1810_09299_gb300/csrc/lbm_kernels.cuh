@@ -132,16 +132,15 @@ __device__ __forceinline__ void ring_cell(int q, int& a, int& b) {
 #ifndef AXILBM_GRID16_CTAS
 #define AXILBM_GRID16_CTAS 4
 #endif
-#ifndef AXILBM_F64_CTAS
-#define AXILBM_F64_CTAS 2
-#endif
+// FP64 with a compile-time rate pattern: 16 warps per SM at 128 registers (the
+// figures in lbm_f64.cuh).
 template <class Codec, int BZ, int RM>
 constexpr int step_min_blocks() {
     constexpr int bz8 = Codec::kGrid ? AXILBM_GRID16_CTAS
                         : (RM == kRatesPaperRaw && sizeof(typename Codec::PT) == 2)
                             ? 4
                             : (sizeof(typename Codec::PT) == 2 ? AXILBM_STEP16_CTAS : 5);
-    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ >= 16 ? 1 : AXILBM_F64_CTAS * (8 / BZ)))
+    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ >= 16 ? 1 : (BZ == 4 ? 4 : 2)))
            : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
                 : (BZ >= 16 ? 1 : (BZ >= 8 ? AXILBM_GENERAL_CTAS : 2 * AXILBM_GENERAL_CTAS));
 }
