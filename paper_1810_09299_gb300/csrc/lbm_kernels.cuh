@@ -592,6 +592,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     //    its ghost node's f), and the f of this thread's ring cells
     int32_t cw = 0;
     if (q < kCW) cw = reinterpret_cast<const int32_t*>(cases + g.c)[q];
+    pdl_wait();
     // L2 prefetch of the blocks of the tile one resident wave ahead (a CTA
     // that will start about when this one ends): one tensor prefetch, issued
     // by one thread; the tensor maps are absent when they could not be made
@@ -819,6 +820,7 @@ step_kernel_seq2(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
     //    the ghost node's f) and the f of this thread's ring cell
     int32_t cw = 0;
     if (q < kCW) cw = reinterpret_cast<const int32_t*>(cases + g.c)[q];
+    pdl_wait();
     if (maps != nullptr && q == 0 && (int)blockIdx.x + ahead < ntiles) {
         const TileDev tp = tiles[blockIdx.x + ahead];
         const CUtensorMap* M = maps + ((size_t)tp.c * 2 + map_set) * kMapsPerCase + 2 + parity;
@@ -1074,6 +1076,7 @@ step_kernel_pack2(const CaseDev* __restrict__ cases, const TileGeo* __restrict__
     //    raw values of this thread's ring cell
     int32_t cw = 0;
     if (q < kCW) cw = reinterpret_cast<const int32_t*>(cases + g.c)[q];
+    pdl_wait();
     if (maps != nullptr && q == 0 && (int)blockIdx.x + ahead < ntiles) {
         // L2 prefetch of the tile one resident wave ahead
         const TileGeo tp = geo[blockIdx.x + ahead];
@@ -1150,6 +1153,10 @@ step_kernel_pack2(const CaseDev* __restrict__ cases, const TileGeo* __restrict__
     float2 mf[9], mg[9], g0;
     pack2_moments<Codec>(grid_col<Codec>(j), f0raw, fraw, graw, mf, mg, g0);
     __syncthreads();
+    // more tiles than CTAs at once: the next step's first CTAs may take the
+    // places that free up (512 cases 565.7 -> 558.0 us); with fewer the early start
+    // packs them unevenly on the SMs (the 200 x 600 thread 4.97 -> 5.40 us)
+    if (ntiles > ahead) pdl_trigger();
     if (!in[0]) return;  // the second node lies below the first
     const CaseDev& C = sC;
     const CaseView<Codec> V = case_view<Codec>(S, C);
@@ -1660,6 +1667,22 @@ void launch_tma(int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* t
         cs, tiles, ntiles, S, (const CUtensorMap*)D.tmaps, BZ == 8 ? 0 : 1, parity, D.status);
 }
 
+// A step launch that may overlap the end of the launch before it on the stream
+// (programmatic stream serialisation; see pdl_wait).
+template <class... P, class... A>
+void launch_step_kernel(void (*kernel)(P...), int grid, dim3 block, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <class Codec, int RM>
 void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* tiles,
                        const StateDev<Codec>& S, const DeviceState& D, int parity) {
@@ -1674,47 +1697,37 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
     const CUtensorMap* maps = (const CUtensorMap*)D.tmaps;
     switch (variant) {
         case 0:
-            step_kernel<Codec, 8, RM><<<ntiles, dim3(kTR, 8), 0, st>>>(
-                cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 8, RM>() / 4);
+            launch_step_kernel(step_kernel<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 8, RM>() / 4);
             break;
         case 1:
-            step_kernel<Codec, 16, RM><<<ntiles, dim3(kTR, 16), 0, st>>>(
-                cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+            launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         case 2:
-            step_kernel<Codec, 4, RM><<<ntiles, dim3(kTR, 4), 0, st>>>(
-                cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
+            launch_step_kernel(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
             break;
         case 3: launch_tma<Codec, 8, RM>(ntiles, st, cs, tiles, S, D, parity); break;
         case 4: launch_tma<Codec, 16, RM>(ntiles, st, cs, tiles, S, D, parity); break;
         case 5:
             if constexpr (sizeof(typename Codec::Real) == 4)
-                step_kernel_seq2<Codec, 8, RM><<<ntiles, dim3(kTR, 8), 0, st>>>(
-                    cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
+                launch_step_kernel(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
             else
-                step_kernel<Codec, 16, RM><<<ntiles, dim3(kTR, 16), 0, st>>>(
-                    cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         case 7:
             if constexpr (Codec::kGrid)
-                step_kernel_pack2<Codec, RM><<<ntiles, dim3(kTR, 8), 0, st>>>(
-                    cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps, parity, ntiles,
+                launch_step_kernel(step_kernel_pack2<Codec, RM>, ntiles, dim3(kTR, 8), st, cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps, parity, ntiles,
                     kPrefetchQuarters * sms * AXILBM_PACK2_CTAS / 4);
             else if constexpr (sizeof(typename Codec::Real) == 4)
-                step_kernel_seq2<Codec, 8, RM><<<ntiles, dim3(kTR, 8), 0, st>>>(
-                    cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
+                launch_step_kernel(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
             else
-                step_kernel<Codec, 16, RM><<<ntiles, dim3(kTR, 16), 0, st>>>(
-                    cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         default:
             if constexpr (sizeof(typename Codec::Real) == 4)
-                step_kernel_seq2<Codec, 8, RM, true><<<ntiles, dim3(kTR, 8), 0, st>>>(
-                    cs, tiles, S, maps, 1, parity, ntiles,
+                launch_step_kernel(step_kernel_seq2<Codec, 8, RM, true>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles,
                     kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM, true>() / 4);
             else
-                step_kernel<Codec, 16, RM><<<ntiles, dim3(kTR, 16), 0, st>>>(
-                    cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
     }
 }
