@@ -102,7 +102,7 @@ struct lbm_sim {
     double* state = nullptr;    // [21][nz][nr]
     double* partials = nullptr;
     double* diag_out = nullptr;
-    double* axis_rows = nullptr;   // nz doubles of the tallest case
+    double* axis_rows = nullptr;   // 2 nz doubles of the tallest case
     double* axis_out = nullptr;    // the drops record, 3 + 4 * kMaxAxisDrops doubles
     double* axis_host = nullptr;   // pinned copy of axis_out
     // pinned host staging for small reads (a diagnostics record and the
@@ -167,14 +167,15 @@ cudaError_t launch_step_any(lbm_sim* h, int parity, int variant, cudaStream_t st
     }
 }
 
-cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st) {
+// The fields of case icase: all five, or phi alone.
+cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st, bool phi_only = false) {
     const TileDev* t = h->ftiles_d[icase];
     const int n = h->nftiles[icase];
     switch (h->precision) {
-        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, h->fields, st);
-        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, h->fields, st);
-        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, h->fields, st);
-        default: return launch_fields_b16(h->D, h->parity, t, n, h->fields, st);
+        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, h->fields, st);
+        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, h->fields, st);
+        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, h->fields, st);
+        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, h->fields, st);
     }
 }
 
@@ -452,7 +453,7 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
     A((void**)&h->state, 21 * (size_t)h->max_nodes * sizeof(double));
     A((void**)&h->partials, diag_partials_size() * sizeof(double));
     A((void**)&h->diag_out, 16 * sizeof(double));
-    A((void**)&h->axis_rows, (size_t)max_nz * sizeof(double));
+    A((void**)&h->axis_rows, 2 * (size_t)max_nz * sizeof(double));
     A((void**)&h->axis_out, (3 + 4 * kMaxAxisDrops) * sizeof(double));
     A((void**)&h->D.status, 128);
     if (rc == LBM_OK && cudaMallocHost((void**)&h->host_small, 16 * sizeof(double)) != cudaSuccess) {
@@ -566,13 +567,17 @@ int step_direct(lbm_sim* h, int64_t n) {
     return LBM_OK;
 }
 
-// Device status word: set by a bounded wait that gave up (TMA-staged step).
-int check_status(lbm_sim* h) {
-    int st = 0;
-    if (cudaMemcpyAsync(&st, h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-        cudaStreamSynchronize(h->stream) != cudaSuccess)
-        return fail(h, LBM_ERR_CUDA);
-    if (st != 0) {
+// Device status word: set by a bounded wait that gave up (TMA-staged step).  A
+// read-back enqueues its copy (into pinned memory) beside its own and looks at
+// it after the one synchronisation that ends the call.
+int* status_host(lbm_sim* h) { return (int*)(h->host_small + 12); }
+int enqueue_status(lbm_sim* h) {
+    return cuda_ok(h, cudaMemcpyAsync(status_host(h), h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+}
+int finish_status(lbm_sim* h) {
+    const int rc = cuda_ok(h, cudaStreamSynchronize(h->stream));
+    if (rc != LBM_OK) return rc;
+    if (*status_host(h) != 0) {
         h->sticky = LBM_ERR_TIMEOUT;
         return LBM_ERR_TIMEOUT;
     }
@@ -730,22 +735,25 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
     if (rc != LBM_OK) return rc;
     if (check_case(h, icase) != LBM_OK || !host_out || mask <= 0 || mask > 31) return LBM_ERR_INVALID_ARG;
     if (!h->initialized[icase]) return LBM_ERR_STATE;
-    rc = check_status(h);
-    if (rc != LBM_OK) return rc;
     rc = join_diagnostics(h);
     if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream));
+    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI));
+    if (rc == LBM_OK) rc = enqueue_status(h);
     if (rc != LBM_OK) return rc;
     const int64_t n = (int64_t)h->prm[icase].nz * h->prm[icase].nr;
-    int slot = 0;
-    for (int b = 0; b < 5; ++b) {
-        if (!(mask & (1 << b))) continue;
-        rc = cuda_ok(h, cudaMemcpyAsync(host_out + slot * n, h->fields + b * n, n * sizeof(double),
-                                        cudaMemcpyDeviceToHost, h->stream));
-        if (rc != LBM_OK) return rc;
-        ++slot;
+    int64_t slot = 0;
+    for (int b = 0; b < 5;) {
+        int e = b;  // neighbouring planes leave in one copy
+        while (e < 5 && (mask & (1 << e))) ++e;
+        if (e > b) {
+            rc = cuda_ok(h, cudaMemcpyAsync(host_out + slot * n, h->fields + b * n, (e - b) * n * sizeof(double),
+                                            cudaMemcpyDeviceToHost, h->stream));
+            if (rc != LBM_OK) return rc;
+            slot += e - b;
+        }
+        b = e > b ? e : b + 1;
     }
-    return cuda_ok(h, cudaStreamSynchronize(h->stream));
+    return finish_status(h);
 }
 
 int lbm_get_fields(lbm_handle* h, int32_t mask, double* host_out) { return lbm_case_get_fields(h, 0, mask, host_out); }
@@ -757,15 +765,9 @@ int lbm_case_diagnostics(lbm_handle* h, int32_t icase, lbm_diag* out) {
     if (!h->initialized[icase]) return LBM_ERR_STATE;
     // the record and the device status word come back with one synchronisation
     double* buf = h->host_small;          // 11 doubles of the record
-    int* st_h = (int*)(h->host_small + 12);  // the status word
-    rc = enqueue_diagnostics(h, icase, buf, st_h, h->stream);
+    rc = enqueue_diagnostics(h, icase, buf, status_host(h), h->stream);
+    if (rc == LBM_OK) rc = finish_status(h);
     if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, cudaStreamSynchronize(h->stream));
-    if (rc != LBM_OK) return rc;
-    if (*st_h != 0) {
-        h->sticky = LBM_ERR_TIMEOUT;
-        return LBM_ERR_TIMEOUT;
-    }
     static_assert(sizeof(lbm_diag) == 11 * sizeof(double), "diag layout");
     std::memcpy(out, buf, sizeof(lbm_diag));
     if (out->nonfinite > 0) return fail(h, LBM_ERR_NONFINITE);
@@ -784,11 +786,9 @@ int lbm_case_axis_drops(lbm_handle* h, int32_t icase, int32_t max_drops, lbm_dro
         (max_drops > 0 && !drops))
         return LBM_ERR_INVALID_ARG;
     if (!h->initialized[icase]) return LBM_ERR_STATE;
-    rc = check_status(h);
-    if (rc != LBM_OK) return rc;
     rc = join_diagnostics(h);
     if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream));
+    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, true));
     if (rc != LBM_OK) return rc;
     const lbm_params& p = h->prm[icase];
     rc = cuda_ok(h, launch_axis_drops(h->fields, p.nz, p.nr, p.z_periodic, max_drops, h->axis_rows, h->axis_out,
@@ -796,8 +796,8 @@ int lbm_case_axis_drops(lbm_handle* h, int32_t icase, int32_t max_drops, lbm_dro
     if (rc != LBM_OK) return rc;
     rc = cuda_ok(h, cudaMemcpyAsync(h->axis_host, h->axis_out, (3 + 4 * (size_t)max_drops) * sizeof(double),
                                     cudaMemcpyDeviceToHost, h->stream));
-    if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, cudaStreamSynchronize(h->stream));
+    if (rc == LBM_OK) rc = enqueue_status(h);
+    if (rc == LBM_OK) rc = finish_status(h);
     if (rc != LBM_OK) return rc;
     const int n = (int)h->axis_host[0];
     *n_drops = n;

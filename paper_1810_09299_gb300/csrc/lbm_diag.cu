@@ -268,150 +268,205 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
 // out[2] = row of that minimum + 1/2 (its z), then for each of the first
 // min(number, max_drops) drops in z order (z_start, z_end, volume, radius of
 // the sphere of that volume); z_end < z_start for a drop that wraps a periodic
-// boundary.  rows: scratch of nz doubles.
+// boundary.  rows: scratch of 2 nz doubles.
+//
+// Two kernels.  axis_rows_kernel, one warp per row of the case: rows[k] = sum_j
+// r_j phi(k, j), lanes along r and a fixed shuffle tree, and the axis row copied
+// to rows[nz + k].  axis_drops_kernel, one block: both arrays in shared memory
+// (global for nz > kAxisRows), the runs found by a block scan over contiguous
+// chunks of the axis row, then one warp per drop for its two cuts and its sum.
+// What bounds it is latency: one block and one thread walking the rows one by
+// one took 225 us on a 600 x 200 case and 650 us on a 1024 x 256 one; these two
+// take about 12 and 15.
 constexpr int kAxisThreads = 256;
+constexpr int kAxisRows = 2816;  // rows whose two doubles fit 44 KB of shared memory
 
-__device__ __forceinline__ double axis_phi(const double* F, int nr, int k) { return F[(int64_t)k * nr]; }
-
-// z of the phi = 1/2 crossing between axis rows k and k + 1 (k + 1 taken
-// modulo nz, positions unwrapped: z may exceed nz by less than one row).
-__device__ __forceinline__ double axis_crossing(const double* F, int nz, int nr, int k) {
-    const double a = axis_phi(F, nr, k), b = axis_phi(F, nr, (k + 1) % nz);
-    return (k + 0.5) + (0.5 - a) / (b - a);
+__global__ void __launch_bounds__(kAxisThreads) axis_rows_kernel(const double* __restrict__ F, int nz, int nr,
+                                                                 double* __restrict__ rows) {
+    const int k = blockIdx.x * (kAxisThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k >= nz) return;
+    const double* P = F + (int64_t)k * nr;
+    double s = 0.0;
+    for (int j = lane; j < nr; j += 32) s += (j + 0.5) * P[j];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    if (lane == 0) {
+        rows[k] = s;
+        rows[nz + k] = P[0];
+    }
 }
 
-__global__ void __launch_bounds__(kAxisThreads) axis_drops_kernel(const double* __restrict__ F, int nz, int nr,
-                                                                  int zper, int max_drops,
-                                                                  double* __restrict__ rows,
-                                                                  double* __restrict__ out) {
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-        double s = 0.0;
-        // separately rounded products and sums in r order (no contraction)
-        for (int j = 0; j < nr; ++j) s = __dadd_rn(s, __dmul_rn(j + 0.5, F[(int64_t)k * nr + j]));
-        rows[k] = s;
+// The first row of least weight of the gap of scan indices [a, b), a < b, in
+// row k0 + i of the scan (a row is replaced only by a strictly lighter one, so a
+// NaN at a keeps the cut there); the whole warp calls it.
+__device__ __forceinline__ int lightest_row(const double* rows, int nz, int k0, int a, int b) {
+    const auto at = [&](int i) { return rows[k0 + i < nz ? k0 + i : k0 + i - nz]; };
+    const double first = at(a);
+    if (!(first == first)) return a;
+    const int lane = threadIdx.x & 31;
+    double v = INFINITY;
+    int c = a;
+    for (int i = a + lane; i < b; i += 32) {
+        const double x = at(i);
+        if (x < v) v = x, c = i;
     }
+    for (int off = 16; off > 0; off >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, v, off);
+        const int oc = __shfl_xor_sync(0xffffffffu, c, off);
+        if (ov < v || (ov == v && oc < c)) v = ov, c = oc;
+    }
+    return v < first ? c : a;
+}
+
+// Sum of the rows of scan indices [a, b) (lanes, then a fixed tree); valid in lane 0.
+__device__ __forceinline__ double sum_rows(const double* rows, int nz, int k0, int a, int b) {
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int i = a + lane; i < b; i += 32) s += rows[k0 + i < nz ? k0 + i : k0 + i - nz];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    return s;
+}
+
+__global__ void __launch_bounds__(kAxisThreads) axis_drops_kernel(const double* __restrict__ rows_g, int nz, int zper,
+                                                                  int max_drops, double* __restrict__ out) {
+    constexpr int kWarps = kAxisThreads / 32;
+    __shared__ double sbuf[2 * kAxisRows];
+    __shared__ double s_min[kWarps];
+    __shared__ int s_kmin[kWarps], s_gas[kWarps], s_last[kWarps], s_cnt[kWarps];
+    __shared__ int s_a[kMaxAxisDrops + 1], s_b[kMaxAxisDrops + 1];  // runs of the first drops, scan indices
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const bool fits = nz <= kAxisRows;
+    for (int i = t; fits && i < 2 * nz; i += kAxisThreads) sbuf[i] = rows_g[i];
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    const double two_pi = 6.283185307179586;
-    double pmin = INFINITY;
-    int kmin = 0;
-    int start = -1;  // a gas row of the axis to start the scan at (periodic)
-    for (int k = 0; k < nz; ++k) {
-        const double v = axis_phi(F, nr, k);
-        if (v < pmin) {
-            pmin = v;
-            kmin = k;
-        }
-        if (start < 0 && !(v > 0.5)) start = k;
+    const double* rows = fits ? sbuf : rows_g;
+    const double* axis = rows + nz;
+    const int chunk = (nz + kAxisThreads - 1) / kAxisThreads;
+    // the least phi of the axis row (the first such row) and the first gas row
+    double vmin = INFINITY;
+    int kmin = 0, gas = nz;
+    for (int i = t * chunk; i < min((t + 1) * chunk, nz); ++i) {
+        const double v = axis[i];
+        if (v < vmin) vmin = v, kmin = i;
+        if (gas == nz && !(v > 0.5)) gas = i;
     }
-    out[1] = pmin;
-    out[2] = kmin + 0.5;
-    const auto put = [&](int drop, int field, double v) {
-        if (drop < max_drops) out[3 + 4 * drop + field] = v;
-    };
-    const auto close_drop = [&](int drop, double v) {
+    for (int off = 16; off > 0; off >>= 1) {
+        const double ov = __shfl_down_sync(0xffffffffu, vmin, off);
+        const int ok = __shfl_down_sync(0xffffffffu, kmin, off), og = __shfl_down_sync(0xffffffffu, gas, off);
+        if (ov < vmin || (ov == vmin && ok < kmin)) vmin = ov, kmin = ok;
+        gas = min(gas, og);
+    }
+    if (lane == 0) s_min[w] = vmin, s_kmin[w] = kmin, s_gas[w] = gas;
+    __syncthreads();
+    gas = nz;
+    for (int i = 0; i < kWarps; ++i) gas = min(gas, s_gas[i]);
+    if (t == 0) {
+        for (int i = 1; i < kWarps; ++i)
+            if (s_min[i] < vmin) vmin = s_min[i], kmin = s_kmin[i];
+        out[1] = vmin;
+        out[2] = kmin + 0.5;
+    }
+    const double two_pi = 6.283185307179586;
+    const auto put = [&](int drop, int field, double v) { out[3 + 4 * drop + field] = v; };
+    const auto put_volume = [&](int drop, double v) {
         put(drop, 2, two_pi * v);
         put(drop, 3, cbrt(3.0 * two_pi * v / (4.0 * M_PI)));
     };
-    if (start < 0) {  // liquid along the whole axis: one unbroken body
-        double vol = 0.0;
-        for (int k = 0; k < nz; ++k) vol += rows[k];
-        out[0] = 1.0;
-        put(0, 0, 0.0);
-        put(0, 1, (double)nz);
-        close_drop(0, vol);
+    if (gas == nz) {  // liquid along the whole axis: one unbroken body
+        if (w == 0) {
+            const double vol = sum_rows(rows, nz, 0, 0, nz);
+            if (lane == 0) {
+                out[0] = 1.0;
+                if (max_drops > 0) {
+                    put(0, 0, 0.0);
+                    put(0, 1, (double)nz);
+                    put_volume(0, vol);
+                }
+            }
+        }
         return;
     }
+    // The scan starts at row 0, or in a periodic case at the first row of the
+    // gas gap that the first gas row lies in, so that the rows before it
+    // (cyclically) end the last drop.
+    int k0 = 0;
     if (zper) {
-        // start the scan at the first row of a gas gap, so that the rows
-        // before it (cyclically) end the last drop
-        int n = 0;
-        while (n < nz && !(axis_phi(F, nr, (start + nz - 1) % nz) > 0.5)) {
-            start = (start + nz - 1) % nz;
-            ++n;
-        }
-        if (n == nz) {  // gas along the whole axis: no drop
-            out[0] = 0.0;
-            return;
-        }
-    } else {
-        start = 0;
-    }
-    // One pass over the rows in scan order.  Inside a gap the rows before its
-    // lightest row go to the drop before the gap, the rest to the drop after it.
-    int ndrops = 0;
-    double vol = 0.0;                      // rows of the current drop so far
-    double gap_before = 0.0, gap_after = 0.0, gap_min = 0.0;
-    double lead_before = 0.0;              // periodic: first gap's share of the last drop
-    bool in_gap = false, first_row = true;
-    for (int i = 0; i < nz; ++i) {
-        const int k = zper ? (start + i) % nz : i;
-        const int kp = (k + nz - 1) % nz;  // the row before k (cyclically)
-        const bool liquid = axis_phi(F, nr, k) > 0.5;
-        if (!liquid) {
-            if (!in_gap) {
-                // a gap opens: the drop before it (if any) ends before this row
-                if (!first_row) {
-                    double ze = axis_crossing(F, nz, nr, kp);
-                    if (ze >= nz) ze -= nz;
-                    put(ndrops - 1, 1, ze);
-                }
-                in_gap = true;
-                gap_before = 0.0;
-                gap_after = rows[k];
-                gap_min = rows[k];
-            } else if (rows[k] < gap_min) {
-                gap_before += gap_after;
-                gap_after = rows[k];
-                gap_min = rows[k];
-            } else {
-                gap_after += rows[k];
+        if (gas > 0) {
+            k0 = gas;
+        } else {  // row 0 is gas: its gap starts after the last liquid row
+            int last = -1;
+            for (int i = t * chunk; i < min((t + 1) * chunk, nz); ++i)
+                if (axis[i] > 0.5) last = i;
+            for (int off = 16; off > 0; off >>= 1) last = max(last, __shfl_down_sync(0xffffffffu, last, off));
+            if (lane == 0) s_last[w] = last;
+            __syncthreads();
+            last = -1;
+            for (int i = 0; i < kWarps; ++i) last = max(last, s_last[i]);
+            if (last < 0) {  // gas along the whole axis: no drop
+                if (t == 0) out[0] = 0.0;
+                return;
             }
-        } else {
-            if (in_gap || first_row) {
-                // a drop starts at this row
-                if (ndrops > 0) {
-                    close_drop(ndrops - 1, vol + gap_before);
-                    vol = gap_after;
-                } else {
-                    // the first drop: a leading gap of a walled case is all its;
-                    // in a periodic case the part before the cut wraps to the last drop
-                    if (zper) {
-                        lead_before = gap_before;
-                        vol = gap_after;
-                    } else {
-                        vol = gap_before + gap_after;
-                    }
-                }
-                double zs = 0.0;  // a drop touching the wall z = 0 starts at the wall plane
-                if (!(first_row && !zper)) {
-                    zs = axis_crossing(F, nz, nr, kp);
-                    if (zs >= nz) zs -= nz;
-                }
-                put(ndrops, 0, zs);
-                ++ndrops;
-                in_gap = false;
-                gap_before = gap_after = 0.0;
-            }
-            vol += rows[k];
-        }
-        first_row = false;
-    }
-    if (ndrops > 0) {
-        if (zper) {
-            // the scan started at a gap's first row, so it ends inside the last drop
-            double ze = axis_crossing(F, nz, nr, (start + nz - 1) % nz);
-            if (ze >= nz) ze -= nz;
-            put(ndrops - 1, 1, ze);
-            close_drop(ndrops - 1, vol + lead_before);
-        } else if (in_gap) {
-            close_drop(ndrops - 1, vol + gap_before + gap_after);
-        } else {
-            put(ndrops - 1, 1, (double)nz);  // the drop reaches the wall z = nz
-            close_drop(ndrops - 1, vol);
+            k0 = last + 1 < nz ? last + 1 : 0;
         }
     }
-    out[0] = (double)ndrops;
+    const auto liquid = [&](int i) { return axis[k0 + i < nz ? k0 + i : k0 + i - nz] > 0.5; };
+    // runs of liquid in scan order: each thread counts the starts of its chunk
+    // of scan indices, then numbers them from the block's exclusive sum
+    const int i0 = min(t * chunk, nz), i1 = min(i0 + chunk, nz);
+    int count = 0;
+    bool prev = i0 > 0 && i0 < nz && liquid(i0 - 1);
+    for (int i = i0; i < i1; ++i) {
+        const bool l = liquid(i);
+        count += l && !prev;
+        prev = l;
+    }
+    int incl = count;
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
+    }
+    if (lane == 31) s_cnt[w] = incl;
+    __syncthreads();
+    int d = incl - count, ndrops = 0;
+    for (int i = 0; i < kWarps; ++i) {
+        if (i < w) d += s_cnt[i];
+        ndrops += s_cnt[i];
+    }
+    prev = i0 > 0 && i0 < nz && liquid(i0 - 1);
+    for (int i = i0; i < i1; ++i) {
+        const bool l = liquid(i);
+        if (l && !prev) {
+            if (d <= kMaxAxisDrops) s_a[d] = i;
+            ++d;
+        }
+        if (l && (i + 1 == nz || !liquid(i + 1)) && d - 1 <= kMaxAxisDrops) s_b[d - 1] = i;
+        prev = l;
+    }
+    __syncthreads();
+    if (t == 0) out[0] = (double)ndrops;
+    // z of the phi = 1/2 crossing between the rows of scan indices i and i + 1
+    const auto crossing = [&](int i) {
+        const int k = k0 + i < nz ? k0 + i : k0 + i - nz, kn = k + 1 < nz ? k + 1 : 0;
+        const double a = axis[k], b = axis[kn];
+        const double z = (k + 0.5) + (0.5 - a) / (b - a);
+        return z >= nz ? z - nz : z;
+    };
+    // One warp per drop: the rows from the lightest row of the gap before it to
+    // the one before the lightest row of the gap after it; at walls the whole
+    // gap; in a periodic case the first gap's rows before its cut end the last
+    // drop.
+    for (int q = w; q < min(ndrops, max_drops); q += kWarps) {
+        const bool last = q + 1 == ndrops;
+        int lo = 0, hi = nz;
+        if (q > 0) lo = lightest_row(rows, nz, k0, s_b[q - 1] + 1, s_a[q]);
+        else if (zper) lo = lightest_row(rows, nz, k0, 0, s_a[0]);
+        if (!last) hi = lightest_row(rows, nz, k0, s_b[q] + 1, s_a[q + 1]);
+        double vol = sum_rows(rows, nz, k0, lo, hi);
+        if (last && zper) vol += sum_rows(rows, nz, k0, 0, lightest_row(rows, nz, k0, 0, s_a[0]));
+        if (lane == 0) {
+            put(q, 0, !zper && s_a[q] == 0 ? 0.0 : crossing(s_a[q] == 0 ? nz - 1 : s_a[q] - 1));
+            put(q, 1, !zper && s_b[q] + 1 == nz ? (double)nz : crossing(s_b[q]));
+            put_volume(q, vol);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- shapes
@@ -474,7 +529,9 @@ cudaError_t launch_diag(const double* fields, int nz, int nr, int zper, double s
 
 cudaError_t launch_axis_drops(const double* fields, int nz, int nr, int zper, int max_drops, double* rows, double* out,
                               cudaStream_t st) {
-    axis_drops_kernel<<<1, kAxisThreads, 0, st>>>(fields, nz, nr, zper, max_drops, rows, out);
+    constexpr int per = kAxisThreads / 32;
+    axis_rows_kernel<<<(nz + per - 1) / per, kAxisThreads, 0, st>>>(fields, nz, nr, rows);
+    axis_drops_kernel<<<1, kAxisThreads, 0, st>>>(rows, nz, zper, max_drops, out);
     return cudaGetLastError();
 }
 

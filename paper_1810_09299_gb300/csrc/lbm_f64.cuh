@@ -115,41 +115,44 @@ struct Pre64 {
     Sf m7, m8;                 // sum (c_z^2 - c_r^2) g, sum c_z c_r g
 };
 
+__device__ __forceinline__ void pre64_f(const double* fd, Pre64& P) {
+    const int E = block_exp<9>(fd);
+    long long f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = fix64<kPopK>(fd[i], E);
+    P.Ef = E;
+    P.t = (f[0] + f[1] + f[2]) + (f[3] + f[4] + f[5]) + (f[6] + f[7] + f[8]);
+    P.T = unfix64<kPopK>(P.t, E);
+    P.bad = E >= kBadE;
+    if (P.bad) P.T = nan64();
+    const long long f57 = f[5] - f[7], f68 = f[6] - f[8];
+    P.fz = f[1] - f[3];
+    P.fe = f57 - f68;
+    P.fr = f[2] - f[4];
+    P.fo = f57 + f68;
+}
+template <int RM>
+__device__ __forceinline__ void pre64_g(const double* gd, Pre64& P) {
+    const int E = block_exp<9>(gd);
+    const int e = E - 1075 - kPopK;
+    long long g[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = fix64<kPopK>(gd[i], E);
+    const long long s13 = g[1] + g[3], s24 = g[2] + g[4], s57 = g[5] + g[7], s68 = g[6] + g[8];
+    const long long d57 = g[5] - g[7], d68 = g[6] - g[8];
+    const long long a14 = s13 + s24, a58 = s57 + s68;
+    P.S0 = norm_any(a14 + a58, e);
+    P.q = norm_any(RM == kRatesPaperRaw ? a58 * 2 + a14 : a58 * 2 - a14 - g[0] * 4, e);
+    P.Jz = norm_any((g[1] - g[3]) + (d57 - d68), e);
+    P.Jr = norm_any((g[2] - g[4]) + (d57 + d68), e);
+    P.m7 = norm_any(s13 - s24, e);
+    P.m8 = norm_any(s57 - s68, e);
+    P.bad = P.bad || E >= kBadE;
+}
 template <int RM>
 __device__ __forceinline__ void pre64(const double* fd, const double* gd, Pre64& P) {
-    {
-        const int E = block_exp<9>(fd);
-        long long f[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = fix64<kPopK>(fd[i], E);
-        P.Ef = E;
-        P.t = (f[0] + f[1] + f[2]) + (f[3] + f[4] + f[5]) + (f[6] + f[7] + f[8]);
-        P.T = unfix64<kPopK>(P.t, E);
-        P.bad = E >= kBadE;
-        if (P.bad) P.T = nan64();
-        const long long f57 = f[5] - f[7], f68 = f[6] - f[8];
-        P.fz = f[1] - f[3];
-        P.fe = f57 - f68;
-        P.fr = f[2] - f[4];
-        P.fo = f57 + f68;
-    }
-    {
-        const int E = block_exp<9>(gd);
-        const int e = E - 1075 - kPopK;
-        long long g[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = fix64<kPopK>(gd[i], E);
-        const long long s13 = g[1] + g[3], s24 = g[2] + g[4], s57 = g[5] + g[7], s68 = g[6] + g[8];
-        const long long d57 = g[5] - g[7], d68 = g[6] - g[8];
-        const long long a14 = s13 + s24, a58 = s57 + s68;
-        P.S0 = norm_any(a14 + a58, e);
-        P.q = norm_any(RM == kRatesPaperRaw ? a58 * 2 + a14 : a58 * 2 - a14 - g[0] * 4, e);
-        P.Jz = norm_any((g[1] - g[3]) + (d57 - d68), e);
-        P.Jr = norm_any((g[2] - g[4]) + (d57 + d68), e);
-        P.m7 = norm_any(s13 - s24, e);
-        P.m8 = norm_any(s57 - s68, e);
-        P.bad = P.bad || E >= kBadE;
-    }
+    pre64_f(fd, P);
+    pre64_g<RM>(gd, P);
 }
 
 // What the update takes from a node's column, r = j + 1/2.
@@ -180,21 +183,29 @@ __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7
 // a's integer in units of 2^e, e >= a.e
 __device__ __forceinline__ long long in_units(Sf a, int e) { return shr64(a.m, e - a.e); }
 
-// Macroscopic step, both collisions and both inverse transforms of a node of
-// column constants K; the phi window is centred on (a, b).  What depends on
-// phi alone, the reciprocals and the square roots stay on the FP64 pipe
-// (about 50 operations), the rest runs beside it in integers.
+// The macroscopic step of a node of column constants K; the phi window is
+// centred on (a, b).  What depends on phi alone, the reciprocals and the square
+// roots stay on the FP64 pipe, the rest runs beside it in integers.
+struct Macro64 {
+    Sf gz, gr, Z3, R3;     // 72 grad phi; 0.3 grad rho
+    double nu;
+    Sf rho, s, D;          // s = 1 / tau_g, D = 1 / (r rho + nu rho / r)
+    Sf uz, rz, ur, p, ps;  // rz = rho u_z; ps: the p of Eq. 30 and Eq. 32
+    Sf rFsr;               // r F_s,r
+    Two JFz;               // J_z and F_z (Eq. 30)
+    bool bad;              // a value out of the range of the sums, infinite or NaN
+};
 template <int LD, int RM>
-__device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a, int b, double phi, const Col64& K,
-                                         const Pre64& Q, double chz_prev, double chr_prev, double p_prev, double* fp,
-                                         double* gp, double& chz_out, double& chr_out, double& p_out) {
+__device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, int a, int b, double phi, const Col64& K,
+                                            const Pre64& Q, double p_prev) {
     static_assert(RM == kRatesPaper || RM == kRatesPaperRaw, "a compile-time rate pattern");
     constexpr bool kRaw = RM == kRatesPaperRaw;
     const CaseReal<double>& P = C.pd;
     const Case64& H = C.p64;
-    Sf gz, gr, lap;  // 72 grad phi, 72 lap phi
-    bool bad;
-    stencil64<LD>(W, a, b, gz, gr, lap, bad);
+    Macro64 m;
+    Sf lap;  // 72 lap phi
+    stencil64<LD>(W, a, b, m.gz, m.gr, lap, m.bad);
+    const Sf gz = m.gz, gr = m.gr;
     // of phi alone: Eq. 17, 35, 34, then 1 / tau_g, 1 / (r rho + nu rho / r) and 1 / (r rho) of Eq. 32
     const double rho_d = fma(phi, H.drho, P.rho_g);
     const double nu = fma(phi, H.dnu, P.nu_g);
@@ -219,7 +230,7 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     const Sf A0 = uz * norm29(Z3 - A2 * uz) + K.s_i6 * Q.S0;
     const Sf A1 = norm29(sf_of(((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * K.i4) + R3);
     // numbers that are not finite do not exist in integers: seen here, put out as NaN
-    int top = max(max(abs_hi(s_d), abs_hi(D_d)), max(abs_hi(chz_prev), abs_hi(chr_prev)));
+    int top = max(abs_hi(s_d), abs_hi(D_d));
     Sf ur, p, ps;
     if (C.p_coupling == 1) {
         ps = sf_of(p_prev);
@@ -243,8 +254,27 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         ps = p;
         ur = norm29(ca + scale2(D, -1) * p);
     }
+    m.bad = m.bad || Q.bad || top >= 0x7ff00000;
+    m.Z3 = Z3, m.R3 = R3, m.nu = nu, m.rho = rho, m.s = s, m.D = D;
+    m.uz = uz, m.rz = rz, m.ur = ur, m.p = p, m.ps = ps, m.rFsr = rFsr, m.JFz = JFz;
+    return m;
+}
+
+// The macroscopic step, both collisions and both inverse transforms.
+template <int LD, int RM>
+__device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a, int b, double phi, const Col64& K,
+                                         const Pre64& Q, double chz_prev, double chr_prev, double p_prev, double* fp,
+                                         double* gp, double& chz_out, double& chr_out, double& p_out) {
+    constexpr bool kRaw = RM == kRatesPaperRaw;
+    const CaseReal<double>& P = C.pd;
+    const Case64& H = C.p64;
+    const Macro64 m = macros64<LD, RM>(C, W, a, b, phi, K, Q, p_prev);
+    bool bad = m.bad;
+    int top = max(abs_hi(chz_prev), abs_hi(chr_prev));
+    const Sf gz = m.gz, gr = m.gr, Z3 = m.Z3, R3 = m.R3, rho = m.rho, s = m.s, uz = m.uz, rz = m.rz, ur = m.ur, p = m.p;
+    const Two JFz = m.JFz;
     const Sf rr = rho * ur;
-    const Sf Fr = (rFsr + ps) + sf_of(nu * K.i2) * rr;  // Eq. 30 (r)
+    const Sf Fr = (m.rFsr + m.ps) + sf_of(m.nu * K.i2) * rr;  // Eq. 30 (r)
     p_out = double_of(p);
     // phase field (Eq. 19-23, 38): chi, then t / 3 of both directions
     const Sf T = norm_any(Q.t, Q.Ef - 1075 - kPopK);
@@ -339,7 +369,7 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         gp[8] = double_cvt(ninth64(dg - M8 + JZ - JR), E - 2);
         gp[6] = double_cvt(ninth64(dg - M8 - JZ + JR), E - 2);
     }
-    if (bad || Q.bad || top >= 0x7ff00000) {
+    if (bad || top >= 0x7ff00000) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) fp[i] = gp[i] = nan64();
         chz_out = chr_out = p_out = nan64();

@@ -40,7 +40,7 @@ struct DeviceState {
     cudaError_t launch_step_##NAME(const DeviceState& D, int parity, int variant, const TileDev* tiles, int ntiles, \
                                    cudaStream_t st);                                                               \
     cudaError_t launch_fields_##NAME(const DeviceState& D, int parity, const TileDev* tiles, int ntiles,            \
-                                     double* out, cudaStream_t st);                                                \
+                                     bool phi_only, double* out, cudaStream_t st);                                 \
     cudaError_t launch_init_##NAME(const DeviceState& D, int parity, const TileDev* tiles8, int ntiles,             \
                                    const double* phi0, int64_t base, cudaStream_t st);                             \
     cudaError_t launch_get_state_##NAME(const DeviceState& D, int parity, const CaseDev& C, double* f, double* g,   \
@@ -79,7 +79,7 @@ cudaError_t launch_diag(const double* fields, int nz, int nr, int zper, double s
                         double* out, cudaStream_t st);
 
 // Drops on the axis row (lbm_diag.cu): out[3 + 4 * kMaxAxisDrops] doubles,
-// rows: nz doubles of scratch.
+// rows: 2 nz doubles of scratch.
 constexpr int kMaxAxisDrops = 64;
 cudaError_t launch_axis_drops(const double* fields, int nz, int nr, int zper, int max_drops, double* rows, double* out,
                               cudaStream_t st);

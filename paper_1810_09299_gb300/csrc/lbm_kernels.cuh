@@ -1403,47 +1403,76 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
     }
 }
 
-// phi, rho, u_z, u_r, p of one case into dense FP64 arrays out[5][nz][nr].
-template <class Codec>
+// phi, rho, u_z, u_r, p of one case into dense FP64 arrays out[5][nz][nr]; with
+// PHI phi alone, which needs no window.  RM is the handle's rate mode in
+// FP64 (the update's own macroscopic step, lbm_f64.cuh: 116 -> %FP64% us for the
+// diagnostics of a 600 x 200 case) and kRatesGeneral otherwise.
+template <class Codec, int RM, bool PHI>
 __global__ void __launch_bounds__(kTR * 8)
 fields_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles, StateDev<Codec> S,
               double* __restrict__ out) {
     using Real = typename Codec::Real;
     constexpr int TZ = 8;
-    constexpr int LD = kTR + 4;
-    __shared__ Real sphi[(TZ + 4) * LD];
+    constexpr int LD = kTR + 4, NWIN = PHI ? 1 : (TZ + 4) * LD;
+    constexpr bool kU64 = sizeof(Real) == 8 && RM != kRatesGeneral;
+    __shared__ Real sphi[kU64 ? 1 : NWIN];
+    __shared__ long long swm[kU64 ? NWIN : 1];
+    __shared__ int swe[kU64 ? NWIN : 1];
+    const Win64 W{swm, swe};
     const TileDev t = tiles[blockIdx.x];
     const CaseDev& C = cases[t.c];
     const CaseView<Codec> V = case_view<Codec>(S, C);
-    for (int idx = threadIdx.y * kTR + threadIdx.x; idx < (TZ + 4) * LD; idx += kTR * 8)
-        sphi[idx] = window_phi<Codec>(C, V, t, idx / LD, idx % LD);
-    __syncthreads();
     const int j = t.j0 + threadIdx.x, k = t.k0 + threadIdx.y;
-    if (j >= C.nr || k >= C.nz) return;
-    const int loc = k * C.pitch + j;
-    const Real r = (Real)j + (Real)0.5;
-    const Node<Codec> nd = V.in_node(loc);
-    Real g[9];
-    if constexpr (Codec::kGrid) {
-        const GridCol gc = grid_col<Codec>(j);
-        g[0] = Codec::dec_g0(nd.g(0), gc);
-#pragma unroll
-        for (int i = 1; i < 9; ++i) g[i] = Codec::dec_g(nd.g(i), gc, i > 4);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = Codec::dec_g(nd.g(i), (Real)w_of(i) * r);
-    }
-    Macro<Real> m;
-    Real mg[9];
-    moments<Real>(g, mg);
-    node_macros<Real, LD>(C, sphi, threadIdx.y + 2, threadIdx.x + 2, j, mg, g[0], C.p_coupling == 1 ? nd.p() : (Real)0,
-                          m);
     const int64_t n = (int64_t)C.nz * C.nr, o = (int64_t)k * C.nr + j;
-    out[o] = (double)m.phi;
-    out[n + o] = (double)m.rho;
-    out[2 * n + o] = (double)m.uz;
-    out[3 * n + o] = (double)m.ur;
-    out[4 * n + o] = (double)m.p;
+    if constexpr (PHI) {
+        if (j >= C.nr || k >= C.nz) return;
+        out[o] = (double)node_phi_at<Codec>(V, k * C.pitch + j, j);
+    } else {
+        for (int idx = threadIdx.y * kTR + threadIdx.x; idx < (TZ + 4) * LD; idx += kTR * 8) {
+            const Real v = window_phi<Codec>(C, V, t, idx / LD, idx % LD);
+            if constexpr (kU64) W.put(idx, v);
+            else sphi[idx] = v;
+        }
+        __syncthreads();
+        if (j >= C.nr || k >= C.nz) return;
+        const int loc = k * C.pitch + j;
+        const Real r = (Real)j + (Real)0.5;
+        const Node<Codec> nd = V.in_node(loc);
+        Real g[9];
+        if constexpr (Codec::kGrid) {
+            const GridCol gc = grid_col<Codec>(j);
+            g[0] = Codec::dec_g0(nd.g(0), gc);
+#pragma unroll
+            for (int i = 1; i < 9; ++i) g[i] = Codec::dec_g(nd.g(i), gc, i > 4);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) g[i] = Codec::dec_g(nd.g(i), (Real)w_of(i) * r);
+        }
+        if constexpr (kU64) {
+            Pre64 pre;
+            pre.bad = false;
+            pre64_g<RM>(g, pre);
+            const double ir = rcp_(r), phi = node_phi_at<Codec>(V, loc, j);
+            const Macro64 m = macros64<LD, RM>(C, W, threadIdx.y + 2, threadIdx.x + 2, phi, col64<RM>(j, ir), pre,
+                                               C.p_coupling == 1 ? nd.p() : 0.0);
+            out[o] = phi;
+            out[n + o] = fma(phi, C.p64.drho, C.pd.rho_g);
+            out[2 * n + o] = m.bad ? nan64() : double_of(m.uz);
+            out[3 * n + o] = m.bad ? nan64() : double_of(m.ur);
+            out[4 * n + o] = m.bad ? nan64() : double_of(m.p);
+        } else {
+            Macro<Real> m;
+            Real mg[9];
+            moments<Real>(g, mg);
+            node_macros<Real, LD>(C, sphi, threadIdx.y + 2, threadIdx.x + 2, j, mg, g[0],
+                                  C.p_coupling == 1 ? nd.p() : (Real)0, m);
+            out[o] = (double)m.phi;
+            out[n + o] = (double)m.rho;
+            out[2 * n + o] = (double)m.uz;
+            out[3 * n + o] = (double)m.ur;
+            out[4 * n + o] = (double)m.p;
+        }
+    }
 }
 
 // Initial condition of node (k, j) of case C from its phi0 (Eq. 11): f =
@@ -1746,11 +1775,19 @@ cudaError_t launch_step_t(const DeviceState& D, int parity, int variant, const T
 }
 
 template <class Codec>
-cudaError_t launch_fields_t(const DeviceState& D, int parity, const TileDev* tiles, int ntiles, double* out,
-                            cudaStream_t st) {
+cudaError_t launch_fields_t(const DeviceState& D, int parity, const TileDev* tiles, int ntiles, bool phi_only,
+                            double* out, cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
     StateDev<Codec> S = make_state<Codec>(D, parity);
-    fields_kernel<Codec><<<ntiles, dim3(kTR, 8), 0, st>>>((const CaseDev*)D.cases, tiles, S, out);
+    const CaseDev* cs = (const CaseDev*)D.cases;
+    const dim3 block(kTR, 8);
+    constexpr bool f64 = sizeof(typename Codec::Real) == 8;
+    if (phi_only) fields_kernel<Codec, kRatesGeneral, true><<<ntiles, block, 0, st>>>(cs, tiles, S, out);
+    else if (f64 && D.rate_mode == kRatesPaper)
+        fields_kernel<Codec, f64 ? kRatesPaper : kRatesGeneral, false><<<ntiles, block, 0, st>>>(cs, tiles, S, out);
+    else if (f64 && D.rate_mode == kRatesPaperRaw)
+        fields_kernel<Codec, f64 ? kRatesPaperRaw : kRatesGeneral, false><<<ntiles, block, 0, st>>>(cs, tiles, S, out);
+    else fields_kernel<Codec, kRatesGeneral, false><<<ntiles, block, 0, st>>>(cs, tiles, S, out);
     return cudaGetLastError();
 }
 
@@ -1790,8 +1827,8 @@ cudaError_t launch_set_state_t(const DeviceState& D, int parity, const CaseDev& 
         return launch_step_t<CODEC>(D, parity, variant, tiles, ntiles, st);                                      \
     }                                                                                                            \
     cudaError_t launch_fields_##NAME(const DeviceState& D, int parity, const TileDev* tiles, int ntiles,         \
-                                     double* out, cudaStream_t st) {                                             \
-        return launch_fields_t<CODEC>(D, parity, tiles, ntiles, out, st);                                        \
+                                     bool phi_only, double* out, cudaStream_t st) {                              \
+        return launch_fields_t<CODEC>(D, parity, tiles, ntiles, phi_only, out, st);                              \
     }                                                                                                            \
     cudaError_t launch_init_##NAME(const DeviceState& D, int parity, const TileDev* tiles8, int ntiles,          \
                                    const double* phi0, int64_t base, cudaStream_t st) {                          \
