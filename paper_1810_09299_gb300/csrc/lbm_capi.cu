@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <cmath>
@@ -21,6 +22,7 @@ using namespace axilbm;
 
 namespace {
 
+constexpr size_t kTouchBytes = 1 << 18;  // smaller destinations come from the heap's used pages
 constexpr int kGraphSteps = 32;  // steps per captured graph (even: parity returns)
 constexpr int kMax16BitNr = 65536;  // largest nr of the 16-bit storage forms
 
@@ -584,6 +586,24 @@ int finish_status(lbm_sim* h) {
     return LBM_OK;
 }
 
+// Write to each page of a pageable host destination before the copy into it:
+// pages that the process has never touched are otherwise mapped one by one
+// from the GPU's side of the copy (the f, g, aux of a 1024 x 256 case into fresh
+// arrays: 35 ms against 2).  Memory known to CUDA is left alone.
+void touch_pages(void* dst, size_t bytes) {
+    cudaPointerAttributes at{};
+    if (bytes < kTouchBytes) return;
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (at.type != cudaMemoryTypeUnregistered) return;
+    static const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
+    volatile char* p = (volatile char*)dst;
+    for (size_t o = 0; o < bytes; o += page) p[o] = 0;
+    p[bytes - 1] = 0;
+}
+
 int check_case(lbm_sim* h, int icase) {
     if (icase < 0 || icase >= h->ncases) return LBM_ERR_INVALID_ARG;
     return LBM_OK;
@@ -746,6 +766,7 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
         int e = b;  // neighbouring planes leave in one copy
         while (e < 5 && (mask & (1 << e))) ++e;
         if (e > b) {
+            touch_pages(host_out + slot * n, (e - b) * n * sizeof(double));
             rc = cuda_ok(h, cudaMemcpyAsync(host_out + slot * n, h->fields + b * n, (e - b) * n * sizeof(double),
                                             cudaMemcpyDeviceToHost, h->stream));
             if (rc != LBM_OK) return rc;
@@ -850,6 +871,10 @@ int lbm_get_state(lbm_handle* h, int32_t icase, double* f, double* g, double* au
     double* da = h->state + 18 * n;
     rc = cuda_ok(h, launch_get_state_any(h, icase, f ? df : nullptr, g ? dg : nullptr, aux ? da : nullptr));
     if (rc != LBM_OK) return rc;
+    // while the kernel runs
+    if (f) touch_pages(f, 9 * n * sizeof(double));
+    if (g) touch_pages(g, 9 * n * sizeof(double));
+    if (aux) touch_pages(aux, 3 * n * sizeof(double));
     if (f) rc = cuda_ok(h, cudaMemcpyAsync(f, df, 9 * n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     if (rc == LBM_OK && g)
         rc = cuda_ok(h, cudaMemcpyAsync(g, dg, 9 * n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));

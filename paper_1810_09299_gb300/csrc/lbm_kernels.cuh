@@ -1405,7 +1405,7 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
 
 // phi, rho, u_z, u_r, p of one case into dense FP64 arrays out[5][nz][nr]; with
 // PHI phi alone, which needs no window.  RM is the handle's rate mode in
-// FP64 (the update's own macroscopic step, lbm_f64.cuh: 116 -> %FP64% us for the
+// FP64 (the update's own macroscopic step, lbm_f64.cuh: 116 -> 80 us for the
 // diagnostics of a 600 x 200 case) and kRatesGeneral otherwise.
 template <class Codec, int RM, bool PHI>
 __global__ void __launch_bounds__(kTR * 8)

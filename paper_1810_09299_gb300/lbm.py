@@ -253,7 +253,7 @@ class Simulation:
         for k in which:
             mask |= 1 << FIELDS.index(k)
         order = [k for k in FIELDS if mask & (1 << FIELDS.index(k))]
-        out = np.zeros((len(order), c["nz"], c["nr"]))
+        out = np.empty((len(order), c["nz"], c["nr"]))  # every value is written by the call
         _check(lib().lbm_case_get_fields(self._h, icase, mask, _dp(out)), "lbm_get_fields")
         return {k: out[i] for i, k in enumerate(order)}
 
@@ -289,9 +289,9 @@ class Simulation:
 
     def state(self, icase: int = 0):
         c = self.cases[icase]
-        f = np.zeros((9, c["nz"], c["nr"]))
-        g = np.zeros((9, c["nz"], c["nr"]))
-        aux = np.zeros((3, c["nz"], c["nr"]))
+        f = np.empty((9, c["nz"], c["nr"]))  # every value is written by the call
+        g = np.empty((9, c["nz"], c["nr"]))
+        aux = np.empty((3, c["nz"], c["nr"]))
         _check(lib().lbm_get_state(self._h, icase, _dp(f), _dp(g), _dp(aux)), "lbm_get_state")
         return f, g, aux
 
