@@ -485,6 +485,14 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
             cudaStreamCreateWithPriority(&h->diag_stream, cudaStreamNonBlocking, greatest) != cudaSuccess)
             rc = LBM_ERR_CUDA;
     }
+    if (rc == LBM_OK && h->precision == LBM_FP64) {
+        for (const CaseDev& C : h->cases) h->D.ncols = std::max(h->D.ncols, C.pitch);
+        void* cols = nullptr;
+        A(&cols, col_tab64_size(h->D.ncols));
+        if (rc == LBM_OK && launch_col_tab64((double*)cols, h->D.ncols, h->D.rate_mode, h->stream) != cudaSuccess)
+            rc = LBM_ERR_CUDA;
+        h->D.cols = (const double*)cols;
+    }
     if (rc == LBM_OK) {
         std::vector<CUtensorMap> maps;
         h->tma_ok = encode_tensor_maps(h, maps);

@@ -475,6 +475,8 @@ template <class Codec>
 struct StateDev {
     const unsigned char* in;  // the buffer the step reads
     unsigned char* out;       // the buffer it writes
+    const double* cols;       // FP64: the column table (ColTab64 of lbm_f64.cuh)
+    int ncols;
 };
 
 // The buffers of one case; nodes are addressed by loc = k * pitch + j.

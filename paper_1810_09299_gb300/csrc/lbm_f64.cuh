@@ -166,18 +166,56 @@ __device__ __forceinline__ Col64 col64(int j, double inv_r) {
     return Col64{r, inv_r, (RM == kRatesPaperRaw ? -4.0 / 15.0 : -2.0 / 15.0) * inv_r, -2.0 * inv_r, sf_of(r),
                  sf_of(inv_r), sf_of(0.6 * inv_r), sf_of((1.0 / 0.3) * r), sf_of(3.0 * r), sf_of((1.0 / 72.0) * r)};
 }
-// The columns of a tile in shared memory, filled once per CTA.
+// The columns 0 .. n - 1 of a handle in device memory, filled once when it is
+// created: with them formed per tile in shared memory the window waited for a
+// chain of FP64 operations behind a barrier of its own.
 struct ColTab64 {
-    double d[4][32];
-    Sf s[6][32];
-    __device__ __forceinline__ void put(int x, const Col64& c) {
-        d[0][x] = c.r, d[1][x] = c.inv_r, d[2][x] = c.i4, d[3][x] = c.i2;
-        s[0][x] = c.sr, s[1][x] = c.s_inv_r, s[2][x] = c.s_i6, s[3][x] = c.r03, s[4][x] = c.r3, s[5][x] = c.r72;
+    const double* d;  // [4][n] doubles, then Sf [6][n]
+    int n;
+    __device__ __forceinline__ double inv_r(int j) const { return __ldg(d + n + j); }
+    __device__ __forceinline__ const longlong2* sf(int i) const {
+        return reinterpret_cast<const longlong2*>(d + 4 * n) + (int64_t)i * n;
     }
-    __device__ __forceinline__ Col64 get(int x) const {
-        return Col64{d[0][x], d[1][x], d[2][x], d[3][x], s[0][x], s[1][x], s[2][x], s[3][x], s[4][x], s[5][x]};
-    }
+    __device__ __forceinline__ struct ColRef64 at(int j) const;
 };
+// One column of the table, its values loaded where they are used.
+struct ColRef64 {
+    ColTab64 t;
+    int j;
+    __device__ __forceinline__ double dv(int i) const {
+        double v;
+        asm("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(t.d + i * t.n + j));
+        return v;
+    }
+    __device__ __forceinline__ Sf sv(int i) const {
+        long long m, e;
+        asm("ld.global.nc.v2.s64 {%0, %1}, [%2];" : "=l"(m), "=l"(e) : "l"(t.sf(i) + j));
+        return Sf{m, (int)e};
+    }
+    __device__ __forceinline__ double r() const { return dv(0); }
+    __device__ __forceinline__ double inv_r() const { return dv(1); }
+    __device__ __forceinline__ double i4() const { return dv(2); }
+    __device__ __forceinline__ double i2() const { return dv(3); }
+    __device__ __forceinline__ Sf sr() const { return sv(0); }
+    __device__ __forceinline__ Sf s_inv_r() const { return sv(1); }
+    __device__ __forceinline__ Sf s_i6() const { return sv(2); }
+    __device__ __forceinline__ Sf r03() const { return sv(3); }
+    __device__ __forceinline__ Sf r3() const { return sv(4); }
+    __device__ __forceinline__ Sf r72() const { return sv(5); }
+};
+__device__ __forceinline__ ColRef64 ColTab64::at(int j) const { return ColRef64{*this, j}; }
+// 16 bytes per column and Sf, 8 per double
+constexpr size_t col_tab64_bytes(int n) { return (size_t)n * (4 * 8 + 6 * 16); }
+template <int RM>
+__global__ void col_tab64_kernel(double* d, int n) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const Col64 c = col64<RM>(j, rcp_((double)j + 0.5));
+    d[j] = c.r, d[n + j] = c.inv_r, d[2 * n + j] = c.i4, d[3 * n + j] = c.i2;
+    longlong2* s = reinterpret_cast<longlong2*>(d + 4 * n);
+    const Sf v[6] = {c.sr, c.s_inv_r, c.s_i6, c.r03, c.r3, c.r72};
+    for (int i = 0; i < 6; ++i) s[(int64_t)i * n + j] = longlong2{v[i].m, (long long)v[i].e};
+}
 
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
 // a's integer in units of 2^e, e >= a.e
@@ -196,7 +234,7 @@ struct Macro64 {
     bool bad;              // a value out of the range of the sums, infinite or NaN
 };
 template <int LD, int RM>
-__device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, int a, int b, double phi, const Col64& K,
+__device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, int a, int b, double phi, const ColRef64& K,
                                             const Pre64& Q, double p_prev) {
     static_assert(RM == kRatesPaper || RM == kRatesPaperRaw, "a compile-time rate pattern");
     constexpr bool kRaw = RM == kRatesPaperRaw;
@@ -211,14 +249,14 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
     const double nu = fma(phi, H.dnu, P.nu_g);
     const double tau = fma(3.0, nu, 0.5);
     const double s_d = rcp_in(tau);
-    const double rv = fma(nu, K.inv_r, K.r);
+    const double rv = fma(nu, K.inv_r(), K.r());
     const double D_d = rcp_in(rho_d * rv);
-    const Sf rho = sf_of(rho_d), s = sf_of(s_d), D = sf_of(D_d), irr = sf_of(K.inv_r * (D_d * rv));
+    const Sf rho = sf_of(rho_d), s = sf_of(s_d), D = sf_of(D_d), irr = sf_of(K.inv_r() * (D_d * rv));
     // Eq. 4: mu~ = mu - k d_r phi / r; Eq. 30's F_z = r (F_s + G)_z
-    const Sf mut = norm29(sf_of((H.beta4 * phi) * fma(phi, phi - 1.5, 0.5)) + Sf{H.mkappa_m, H.mkappa_e} * norm29(gr * K.s_inv_r + lap));
-    const Sf rm = K.r72 * mut;
+    const Sf mut = norm29(sf_of((H.beta4 * phi) * fma(phi, phi - 1.5, 0.5)) + Sf{H.mkappa_m, H.mkappa_e} * norm29(gr * K.s_inv_r() + lap));
+    const Sf rm = K.r72() * mut;
     Sf Fz = rm * gz;
-    if (abs_hi(P.grav_z) != 0) Fz = Fz + sf_of(K.r * ((rho_d - P.rho_l) * P.grav_z));
+    if (abs_hi(P.grav_z) != 0) Fz = Fz + sf_of(K.r() * ((rho_d - P.rho_l) * P.grav_z));
     const Sf rFsr = rm * gr;
     const Sf d3{H.drho3_m, H.drho3_e};
     const Sf Z3 = d3 * gz, R3 = d3 * gr;  // 0.3 grad rho
@@ -227,8 +265,8 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
     const Sf rz = rho * uz;
     // Eq. 33 with s_p = tau_g / 2 (raw: 3 tau_g / 2 - 1)
     const Sf A2 = sf_of(0.4 * rho_d);
-    const Sf A0 = uz * norm29(Z3 - A2 * uz) + K.s_i6 * Q.S0;
-    const Sf A1 = norm29(sf_of(((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * K.i4) + R3);
+    const Sf A0 = uz * norm29(Z3 - A2 * uz) + K.s_i6() * Q.S0;
+    const Sf A1 = norm29(sf_of(((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * K.i4()) + R3);
     // numbers that are not finite do not exist in integers: seen here, put out as NaN
     int top = max(abs_hi(s_d), abs_hi(D_d));
     Sf ur, p, ps;
@@ -262,7 +300,7 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
 
 // The macroscopic step, both collisions and both inverse transforms.
 template <int LD, int RM>
-__device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a, int b, double phi, const Col64& K,
+__device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a, int b, double phi, const ColRef64& K,
                                          const Pre64& Q, double chz_prev, double chr_prev, double p_prev, double* fp,
                                          double* gp, double& chz_out, double& chr_out, double& p_out) {
     constexpr bool kRaw = RM == kRatesPaperRaw;
@@ -274,7 +312,7 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     const Sf gz = m.gz, gr = m.gr, Z3 = m.Z3, R3 = m.R3, rho = m.rho, s = m.s, uz = m.uz, rz = m.rz, ur = m.ur, p = m.p;
     const Two JFz = m.JFz;
     const Sf rr = rho * ur;
-    const Sf Fr = (m.rFsr + m.ps) + sf_of(m.nu * K.i2) * rr;  // Eq. 30 (r)
+    const Sf Fr = (m.rFsr + m.ps) + sf_of(m.nu * K.i2()) * rr;  // Eq. 30 (r)
     p_out = double_of(p);
     // phase field (Eq. 19-23, 38): chi, then t / 3 of both directions
     const Sf T = norm_any(Q.t, Q.Ef - 1075 - kPopK);
@@ -283,7 +321,7 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     chr_out = double_of(chr);
     {
         // r lambda / (3 (|grad phi| + n_eps)): the normal's factor of grad phi (72 in both)
-        const double lam = H.lam3 * (K.r * fma(-phi, phi, phi));
+        const double lam = H.lam3 * (K.r() * fma(-phi, phi, phi));
         const double Ld = lam * rcp_in(sqrt_in(double_of(gz * gz + gr * gr)) + H.neps72);
         top = max(top, abs_hi(Ld));
         const Sf L = sf_of(Ld);
@@ -311,7 +349,7 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         fp[6] = double_in(d - qm, E);
     }
     // hydrodynamics (Eq. 24, 36-37)
-    const Sf az = K.r03 * Z3, br = norm29(K.r03 * R3 + rho);      // grad (r rho)
+    const Sf az = K.r03() * Z3, br = norm29(K.r03() * R3 + rho);      // grad (r rho)
     const Two PP = align(uz * az, ur * br);
     const Sf udr{PP.a + PP.b, PP.e};
     const Two E12 = align(rz * uz, rr * ur);
@@ -320,15 +358,15 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     const Two s1 = align(Sf{1ll << 61, -61}, s);                // 1 - s, 2 (1 - s/2) and a sixth of that
     const Sf c = norm29(Sf{s1.a - s1.b, s1.e}), h2 = norm29(Sf{s1.a - (s1.b >> 1), s1.e + 1}), h6{third64(h2.m), h2.e - 1};
     const Sf jz{JFz.a + JFz.b, JFz.e}, jr = Q.Jr + Fr;                    // unit rates on the momenta
-    const Sf m7 = (c * Q.m7 + s * (K.sr * norm29(Sf{E12.a - E12.b, E12.e}))) + scale2(h6, 1) * norm29(Sf{PP.a - PP.b, PP.e});
-    const Sf m8 = (c * Q.m8 + s * norm29((K.sr * rr) * uz)) + h6 * norm29(uz * br + ur * az);
+    const Sf m7 = (c * Q.m7 + s * (K.sr() * norm29(Sf{E12.a - E12.b, E12.e}))) + scale2(h6, 1) * norm29(Sf{PP.a - PP.b, PP.e});
+    const Sf m8 = (c * Q.m8 + s * norm29((K.sr() * rr) * uz)) + h6 * norm29(uz * br + ur * az);
     const Sf m0 = scale2(udr - rr, -1);
     if constexpr (kRaw) {
         // raw moments: k_3 = sum c^2 g relaxes with 1/tau_g, k_0 and k_8 take
         // equilibrium and half the source
         const Sf rr3{third64(rr.m), rr.e};
-        const Sf k3 = (c * Q.q + s * (K.sr * pK)) + scale2(h6, 1) * norm29(scale2(udr, 1) - rr);
-        const Sf w = K.r3 * norm29(Sf{(pE.a >> 1) + pE.b, pE.e});   // 3 r (p + rho u^2)
+        const Sf k3 = (c * Q.q + s * (K.sr() * pK)) + scale2(h6, 1) * norm29(scale2(udr, 1) - rr);
+        const Sf w = K.r3() * norm29(Sf{(pE.a >> 1) + pE.b, pE.e});   // 3 r (p + rho u^2)
         const Sf v = udr - rr3;             // 6 times the rest of k_8
         const int E = max(-994, max(max(max(k3.e, m0.e), max(w.e, v.e)), max(max(m7.e, m8.e), max(jz.e, jr.e)))) + 4;
         bad = bad || E > 890;
@@ -348,8 +386,8 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         gp[8] = double_cvt(third64(dm + JZ - JR), E - 2);
         gp[6] = double_cvt(third64(dm - JZ + JR), E - 2);
     } else {
-        const Sf m1 = (c * Q.q + s * (K.r3 * pK)) + h2 * rr;
-        const Sf m2 = neg((K.r3 * norm29(Sf{((pE.a + pE.b) >> 1) + (pE.a >> 2), pE.e + 1})) + (m0 + rr));
+        const Sf m1 = (c * Q.q + s * (K.r3() * pK)) + h2 * rr;
+        const Sf m2 = neg((K.r3() * norm29(Sf{((pE.a + pE.b) >> 1) + (pE.a >> 2), pE.e + 1})) + (m0 + rr));
         // 36 g = 4 m0 - m1 - 2 m2 +- 9 m7 +- 12 j (axes), 4 m0 + 2 m1 + m2 +- 9 m8
         // +- 3 j (diagonals), 4 (m0 - m1 + m2) (rest), in units of 2^E: the
         // coefficients add up to 28 at most

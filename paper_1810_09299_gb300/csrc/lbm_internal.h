@@ -33,6 +33,8 @@ struct DeviceState {
     int64_t total;
     int rate_mode;     // kRatesGeneral, or the rate pattern every case shares (see below)
     const void* tmaps;  // CUtensorMap[ncases][2 tile heights][kMapsPerCase] in device memory
+    const double* cols;  // FP64 handles: constants of the columns 0 .. ncols - 1 (ColTab64 of lbm_f64.cuh)
+    int ncols;
     int* status;        // device status word: nonzero after a bounded wait gave up
 };
 
@@ -47,6 +49,11 @@ struct DeviceState {
                                         double* aux, cudaStream_t st);                                             \
     cudaError_t launch_set_state_##NAME(const DeviceState& D, int parity, const CaseDev& C, const double* f,        \
                                         const double* g, const double* aux, cudaStream_t st);
+
+// The column table of an FP64 handle (rate mode D.rate_mode): its size, and
+// the kernel that fills it.
+size_t col_tab64_size(int ncols);
+cudaError_t launch_col_tab64(double* cols, int ncols, int rate_mode, cudaStream_t st);
 
 AXILBM_DECLARE(f64)
 AXILBM_DECLARE(f32)

@@ -491,7 +491,7 @@ __device__ __forceinline__ void node_update_grid(const CaseDev& C, const CaseVie
 // stored as they are).
 template <int RM, int LD>
 __device__ __forceinline__ void node_update64(const CaseDev& C, const CaseView<CodecF64>& V, const Win64& W, int a,
-                                              int b, double phi, int k, int j, int loc, const Col64& K, const Pre64& pre,
+                                              int b, double phi, int k, int j, int loc, const ColRef64& K, const Pre64& pre,
                                               double chz_prev, double chr_prev, double p_prev) {
     double fp[9], gp[9], chz, chr, p;
     update64<LD, RM>(C, W, a, b, phi, K, pre, chz_prev, chr_prev, p_prev, fp, gp, chz, chr, p);
@@ -569,13 +569,8 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     // collision's many per-case constants need no global loads.
     __shared__ __align__(16) CaseDev sC;
     static_assert(sizeof(CaseDev) % 4 == 0 && sizeof(CaseDev) / 4 <= kTR * BZ, "one word per thread");
-    // FP64: 1 / r of the window's columns j0 - 2 .. j0 + 33, one division per
-    // column instead of four per node (a division is a long sequence on the
-    // FP64 pipe); the same correctly rounded quotients the nodes would form
-    constexpr bool kInvrTable = sizeof(Real) == 8;
-    __shared__ Real s_invr[kInvrTable ? LD : 1];
-    __shared__ __align__(16) double s_col_raw[kU64 ? sizeof(ColTab64) / 8 : 1];
-    ColTab64& s_col = *reinterpret_cast<ColTab64*>(s_col_raw);
+    constexpr bool k64 = sizeof(Real) == 8;
+    const ColTab64 cols64{S.cols, S.ncols};  // FP64: the columns' constants, 1 / r among them
     // 16-bit storage: the column constants of the window's columns
     constexpr bool kG = Codec::kGrid;
     __shared__ float4 sgA[kG ? LD : 1], sgD[kG ? LD : 1];
@@ -633,7 +628,10 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
         if constexpr (kG) return grid_sa<Codec>(jj);
         else return 0.0f;
     };
-    Real ring_sum[kInvrTable ? kRC : 1];  // FP64: as own_sum below
+    auto put_phi = [&](int cell, Real v) {
+        if constexpr (kU64) W.put(cell, v);
+        else sphi[cell] = v;
+    };
 #pragma unroll
     for (int c = 0; c < kRC; ++c) {
         if (q + c * kTR * BZ < NRING) {
@@ -643,82 +641,45 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
             F0T rf0;
             PT rf[8];
             load_phi_raw<Codec>(node_at(ghost_z(g.k0 - 2 + ra, g.nz, g.zper), rj), rf0, rf);
-            if constexpr (kInvrTable) ring_sum[c] = phi_of<Codec>(rf0, rf, (Real)1);
+            if constexpr (k64) put_phi(ra * LD + rb, phi_of<Codec>(rf0, rf, cols64.inv_r(rj)));
             else sphi[ra * LD + rb] = phi_of<Codec>(rf0, rf, rcp_((Real)rj + (Real)0.5), sa_of(rj));
         }
     }
     const Real r = (Real)j + (Real)0.5;
     const int bo = threadIdx.x + 2;
-    Real own_sum = (Real)0, own_phi = (Real)0;  // FP64: the node's f summed; phi once the 1 / r table is filled
+    Real own_phi = (Real)0;
+    // FP64: the node's moments while other warps still wait for their loads
+    // (in FP32 and bfloat16 storage the same was slower, 0.796 against 0.735 ms
+    // and 0.761 against 0.735 ms on the 512-case batch)
+    PreCollision<Real> pre;
+    Pre64 pre6;
     if (inside) {
         if constexpr (sizeof(PT) == 2) {
             sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_(r), sa_of(j));
+        } else if constexpr (kU64) {
+            const Real f[9] = {f0raw, fraw[0], fraw[1], fraw[2], fraw[3], fraw[4], fraw[5], fraw[6], fraw[7]};
+            pre64<RM>(f, graw, pre6);
+            own_phi = pre6.T * cols64.inv_r(j);
+            put_phi((threadIdx.y + 2) * LD + bo, own_phi);
+        } else if constexpr (k64) {
+            sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, cols64.inv_r(j));
+            node_pre<Codec>(f0raw, fraw, graw, r, pre, nullptr, GridCol{});
         } else {
-            if constexpr (kU64) {
-            } else if constexpr (kInvrTable) {
-                own_sum = phi_of<Codec>(f0raw, fraw, (Real)1);
-            } else {
-                Real sum = (Real)f0_value(f0raw);
+            Real sum = (Real)f0_value(f0raw);
 #pragma unroll
-                for (int i = 1; i < 9; ++i) sum += Codec::dec_f(fraw[i - 1], (Real)w_of(i) * r);
-                sphi[(threadIdx.y + 2) * LD + bo] = sum * rcp_(r);
-            }
+            for (int i = 1; i < 9; ++i) sum += Codec::dec_f(fraw[i - 1], (Real)w_of(i) * r);
+            sphi[(threadIdx.y + 2) * LD + bo] = sum * rcp_(r);
         }
     } else {
         const int jm = ghost_r(j, g.nr);
-        if constexpr (kInvrTable) own_sum = phi_of<Codec>(f0raw, fraw, (Real)1);
+        if constexpr (k64) put_phi((threadIdx.y + 2) * LD + bo, phi_of<Codec>(f0raw, fraw, cols64.inv_r(jm)));
         else sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_((Real)jm + (Real)0.5), sa_of(jm));
     }
-    // FP64: the node's moments while other warps still wait for their loads
-    // (19.67 against 19.99 ms on the 512-case batch, bit-identical; in FP32
-    // and bfloat16 storage the same was slower, 0.796 against 0.735 ms and
-    // 0.761 against 0.735 ms)
-    constexpr bool kPreEarly = sizeof(Real) == 8;
-    PreCollision<Real> pre;
-    Pre64 pre6;
-    if constexpr (kU64) {
-        if (inside) {
-            const Real f[9] = {f0raw, fraw[0], fraw[1], fraw[2], fraw[3], fraw[4], fraw[5], fraw[6], fraw[7]};
-            pre64<RM>(f, graw, pre6);
-            own_sum = pre6.T;
-        }
-    } else if constexpr (kPreEarly) {
-        if (inside) node_pre<Codec>(f0raw, fraw, graw, r, pre, nullptr, GridCol{});
-    }
     // 3. the column tables and the case record into shared memory
-    if constexpr (kInvrTable) {
-        if (q < LD) {
-            const int jm = ghost_r(g.j0 - 2 + q, g.nr);
-            const Real ir = rcp_((Real)jm + (Real)0.5);
-            s_invr[q] = ir;
-            if constexpr (kU64) {
-                if (q >= 2 && q < kTR + 2) s_col.put(q - 2, col64<RM>(jm, ir));
-            }
-        }
-    }
     if constexpr (kG) {
         if (q < LD) grid_tab_fill<Codec>(T, q, g.j0, g.nr);
     }
     if (q < kCW) reinterpret_cast<int32_t*>(&sC)[q] = cw;
-    if constexpr (kInvrTable) {
-        // FP64: one division per column, not per node (a division is a long
-        // sequence on the FP64 pipe), so the phi of the window waits for the table
-        auto put_phi = [&](int cell, Real v) {
-            if constexpr (kU64) W.put(cell, v);
-            else sphi[cell] = v;
-        };
-        __syncthreads();
-        own_phi = own_sum * s_invr[bo];
-        put_phi((threadIdx.y + 2) * LD + bo, own_phi);
-#pragma unroll
-        for (int c = 0; c < kRC; ++c) {
-            if (q + c * kTR * BZ < NRING) {
-                int ra, rb;
-                ring_cell<TZ>(q + c * kTR * BZ, ra, rb);
-                put_phi(ra * LD + rb, ring_sum[c] * s_invr[rb]);
-            }
-        }
-    }
     __syncthreads();
     if (!inside) return;
     const CaseDev& C = sC;
@@ -747,15 +708,15 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
         node_update_grid<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
                                         chr_prev, p_prev, f, cols);
     } else if constexpr (kU64) {
-        node_update64<RM, LD>(C, V, W, threadIdx.y + 2, bo, own_phi, k, j, loc, s_col.get(threadIdx.x), pre6,
+        node_update64<RM, LD>(C, V, W, threadIdx.y + 2, bo, own_phi, k, j, loc, cols64.at(j), pre6,
                               chz_prev, chr_prev, p_prev);
     } else {
-        if constexpr (kPreEarly) {
+        if constexpr (k64) {
             node_update_pre<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, pre, chz_prev, chr_prev,
-                                           p_prev, kInvrTable ? s_invr : nullptr, NoCols{});
+                                           p_prev, k64 ? cols64.d + cols64.n + j - bo : nullptr, NoCols{});
         } else {
             node_update<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
-                                       chr_prev, p_prev, kInvrTable ? s_invr : nullptr, kKeepF ? f : nullptr,
+                                       chr_prev, p_prev, nullptr, kKeepF ? f : nullptr,
                                        NoCols{});
         }
     }
@@ -1382,9 +1343,9 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
             } else if constexpr (sizeof(Real) == 8 && RM != kRatesGeneral) {
                 Pre64 pre;
                 pre64<RM>(f, graw, pre);
-                const Real ir = rcp_(r);
-                node_update64<RM, LD>(C, V, W, threadIdx.y + 2, threadIdx.x + 2, pre.T * ir, k, j, loc, col64<RM>(j, ir),
-                                      pre, chz_prev, chr_prev, p_prev);
+                const ColTab64 cols64{S.cols, S.ncols};
+                node_update64<RM, LD>(C, V, W, threadIdx.y + 2, threadIdx.x + 2, pre.T * cols64.inv_r(j), k, j, loc,
+                                      cols64.at(j), pre, chz_prev, chr_prev, p_prev);
             } else {
                 node_update<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, threadIdx.x + 2, k, j, loc, f0raw, fraw,
                                            graw, chz_prev, chr_prev, p_prev, nullptr,
@@ -1452,8 +1413,9 @@ fields_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ til
             Pre64 pre;
             pre.bad = false;
             pre64_g<RM>(g, pre);
-            const double ir = rcp_(r), phi = node_phi_at<Codec>(V, loc, j);
-            const Macro64 m = macros64<LD, RM>(C, W, threadIdx.y + 2, threadIdx.x + 2, phi, col64<RM>(j, ir), pre,
+            const double phi = node_phi_at<Codec>(V, loc, j);
+            const ColTab64 cols64{S.cols, S.ncols};
+            const Macro64 m = macros64<LD, RM>(C, W, threadIdx.y + 2, threadIdx.x + 2, phi, cols64.at(j), pre,
                                                C.p_coupling == 1 ? nd.p() : 0.0);
             out[o] = phi;
             out[n + o] = fma(phi, C.p64.drho, C.pd.rho_g);
@@ -1673,6 +1635,8 @@ StateDev<Codec> make_state(const DeviceState& D, int parity) {
     const int a = parity & 1, b = a ^ 1;
     S.in = (const unsigned char*)D.blk[a];
     S.out = (unsigned char*)D.blk[b];
+    S.cols = D.cols;
+    S.ncols = D.ncols;
     return S;
 }
 
