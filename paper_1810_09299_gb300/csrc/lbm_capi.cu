@@ -403,6 +403,29 @@ bool encode_tensor_maps(lbm_sim* h, std::vector<CUtensorMap>& maps) {
     return true;
 }
 
+// The launch shape a handle starts with (lbm_set_variant, lbm_autotune and the
+// results know no difference).  us a step in the captured graph:
+//   4-row tiles (2) while the 8-row tiles leave half the SMs empty: the 64 x 128
+//     drop 11.0 -> 9.2 in FP64, 2.70 -> 2.38 in FP32, 3.07 -> 2.74 in bfloat16, not
+//     in FP16 (2.89 either way); the 128 x 256 drop (128 tiles of 8 rows) is equal;
+//   FP16, packed pairs of nodes (7) from 3/2 tiles of 16 rows per SM on: 64 x 180
+//     and 128 x 256 are slower there (3.40 against 3.07), 200 x 600 (266 tiles) 5.10 ->
+//     4.94, 256 x 1024 (512) 8.23 -> 7.70, 512 cases 757 -> 558;
+//   FP32, two nodes per thread (5) from two resident waves (3 CTAs per SM) on:
+//     256 x 1024 (512 tiles) 8.20 against 8.81, 8 cases (1100) 15.8 -> 15.2, 512 cases
+//     728 -> 711.
+int default_variant(const lbm_sim* h) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (2 * h->ntiles[0] <= sms && h->precision != LBM_MIX_FP16) return 2;
+    if (h->precision == LBM_MIX_FP16 && 2 * h->ntiles[7] >= 3 * sms) return 7;
+    if (h->precision == LBM_FP32 && h->ntiles[5] >= 6 * sms) return 5;
+    return 0;
+}
+
 int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** out) {
     if (!out) return LBM_ERR_INVALID_ARG;
     *out = nullptr;
@@ -515,6 +538,7 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
         h->ntiles[v] = (int)t.size();
         rc = upload_tiles(h, t, &h->tiles_d[v], true);
     }
+    if (rc == LBM_OK) h->variant = default_variant(h);
     for (int c = 0; c < n && rc == LBM_OK; ++c) {
         std::vector<TileDev> t = make_tiles(h->cases, 8, c);
         TileDev* d = nullptr;
