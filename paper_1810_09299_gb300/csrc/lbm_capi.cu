@@ -405,22 +405,29 @@ bool encode_tensor_maps(lbm_sim* h, std::vector<CUtensorMap>& maps) {
 
 // The launch shape a handle starts with (lbm_set_variant, lbm_autotune and the
 // results know no difference).  us a step in the captured graph:
-//   4-row tiles (2) while the 8-row tiles leave half the SMs empty: the 64 x 128
-//     drop 11.0 -> 9.2 in FP64, 2.70 -> 2.38 in FP32, 3.07 -> 2.74 in bfloat16, not
-//     in FP16 (2.89 either way); the 128 x 256 drop (128 tiles of 8 rows) is equal;
+//   4-row tiles (2) instead of 8-row tiles (0)
+//     where those leave half the SMs empty, FP64 and bfloat16 (a 64 x 128 drop, 32
+//     tiles of 8 rows: 11.0 -> 9.5 and 3.02 -> 2.77; FP32 2.45 and 2.39, FP16 2.90
+//     either way), and where some SMs would hold two of them and most one (101 x
+//     333, 168 tiles on 152 SMs: FP64 16.6 -> 13.4, FP32 3.35 -> 3.22, FP16 3.73 ->
+//     3.47, bfloat16 3.77 -> 3.47; 150 x 300, 190 tiles: 16.6 -> 13.7, 3.41 -> 3.35,
+//     3.59 -> 3.58, 3.98 -> 3.60).  128 tiles (128 x 256) and 250 (150 x 400) take 8
+//     rows: FP32 2.52 against 2.77 and 3.41 against 3.66.
 //   FP16, packed pairs of nodes (7) from 3/2 tiles of 16 rows per SM on: 64 x 180
-//     and 128 x 256 are slower there (3.40 against 3.07), 200 x 600 (266 tiles) 5.10 ->
+//     and 128 x 256 are slower there (3.40 against 3.02), 200 x 600 (266 tiles) 5.01 ->
 //     4.94, 256 x 1024 (512) 8.23 -> 7.70, 512 cases 757 -> 558;
 //   FP32, two nodes per thread (5) from two resident waves (3 CTAs per SM) on:
-//     256 x 1024 (512 tiles) 8.20 against 8.81, 8 cases (1100) 15.8 -> 15.2, 512 cases
-//     728 -> 711.
+//     256 x 1024 (512 tiles) 8.27 against 8.81, 8 cases (1100) 15.8 -> 15.2, 512 cases
+//     726 -> 711.
 int default_variant(const lbm_sim* h) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) {
         cudaGetLastError();
         return 0;
     }
-    if (2 * h->ntiles[0] <= sms && h->precision != LBM_MIX_FP16) return 2;
+    const int t8 = h->ntiles[0];
+    if (2 * t8 <= sms && (h->precision == LBM_FP64 || h->precision == LBM_MIX_BF16)) return 2;
+    if (t8 > sms && 3 * t8 <= 4 * sms) return 2;
     if (h->precision == LBM_MIX_FP16 && 2 * h->ntiles[7] >= 3 * sms) return 7;
     if (h->precision == LBM_FP32 && h->ntiles[5] >= 6 * sms) return 5;
     return 0;

@@ -541,15 +541,46 @@ __device__ __forceinline__ void node_update64(const CaseDev& C, const CaseView<C
     own.f0() = fp[0];
 }
 
-// One time step for every node of every tile in `tiles`: one CTA per tile of
-// BZ rows (z) x 32 columns (r), one node per thread.  Each thread first issues
-// the loads of its own node; the node's phi goes to the shared window straight
-// from those registers and only the two-node ring around the tile is
-// recomputed from neighbours' populations.
+// The shared memory of one tile's step.
 template <class Codec, int BZ, int RM>
-__global__ void __launch_bounds__(kTR * BZ, (step_min_blocks<Codec, BZ, RM>()))
-step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles, StateDev<Codec> S,
-            const CUtensorMap* __restrict__ maps, int map_set, int parity, int ntiles, int ahead) {
+struct TileShared {
+    using Real = typename Codec::Real;
+    static constexpr int LD = kTR + 4, NWIN = (BZ + 4) * LD;
+    // FP64 with a compile-time rate pattern: the update of lbm_f64.cuh, whose
+    // phi window holds unpacked numbers
+    static constexpr bool kU64 = sizeof(Real) == 8 && RM != kRatesGeneral;
+    static constexpr bool kG = Codec::kGrid;
+    // The case's parameters: read from here, the collision's many per-case
+    // constants need no global loads.
+    __align__(16) CaseDev C;
+    // 16-bit storage: the column constants of the window's columns
+    float4 gA[kG ? LD : 1], gD[kG ? LD : 1];
+    uint4 gH[kG ? LD : 1];
+    Real phi[kU64 ? 1 : NWIN];
+    long long wm[kU64 ? NWIN : 1];
+    int we[kU64 ? NWIN : 1];
+    __device__ __forceinline__ GridTab tab() { return GridTab{gA, gD, gH}; }
+    __device__ __forceinline__ Win64 win() { return Win64{wm, we}; }
+};
+// Its parts that do not change from step to step: the column table and the
+// case record, of which thread q holds word cw.
+template <class Codec, int BZ, int RM>
+__device__ __forceinline__ void fill_tile(TileShared<Codec, BZ, RM>& sh, const TileGeo& g, int q, int32_t cw) {
+    static_assert(sizeof(CaseDev) % 4 == 0 && sizeof(CaseDev) / 4 <= kTR * BZ, "one word per thread");
+    if constexpr (Codec::kGrid) {
+        if (q < kTR + 4) grid_tab_fill<Codec>(sh.tab(), q, g.j0, g.nr);
+    }
+    if (q < kCaseWords<typename Codec::Real>) reinterpret_cast<int32_t*>(&sh.C)[q] = cw;
+}
+
+// One step of the nodes of one tile of BZ rows (z) x 32 columns (r), one node
+// per thread, all threads of the CTA.  Each thread first issues the loads of
+// its own node; the node's phi goes to the shared window straight from those
+// registers and only the two-node ring around the tile is recomputed from
+// neighbours' populations.  cw: this thread's word of the case record.
+template <class Codec, int BZ, int RM>
+__device__ __forceinline__ void step_tile(const StateDev<Codec>& S, TileShared<Codec, BZ, RM>& sh, const TileGeo& g,
+                                          int q, int32_t cw) {
     using Real = typename Codec::Real;
     using PT = typename Codec::PT;
     using F0T = typename Codec::F0T;
@@ -557,46 +588,16 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     constexpr int LD = kTR + 4;
     constexpr int NRING = 4 * kTR + 4 * (TZ + 4);
     static_assert(NRING == (TZ + 4) * LD - TZ * kTR, "the ring is the window without the tile");
-    // FP64 with a compile-time rate pattern: the update of lbm_f64.cuh, whose
-    // phi window holds unpacked numbers
-    constexpr bool kU64 = sizeof(Real) == 8 && RM != kRatesGeneral;
-    constexpr int NWIN = (TZ + 4) * LD;
-    __shared__ Real sphi[kU64 ? 1 : NWIN];
-    __shared__ long long swm[kU64 ? NWIN : 1];
-    __shared__ int swe[kU64 ? NWIN : 1];
-    const Win64 W{swm, swe};
-    // The case's parameters go to shared memory: read from there, the
-    // collision's many per-case constants need no global loads.
-    __shared__ __align__(16) CaseDev sC;
-    static_assert(sizeof(CaseDev) % 4 == 0 && sizeof(CaseDev) / 4 <= kTR * BZ, "one word per thread");
-    constexpr bool k64 = sizeof(Real) == 8;
+    constexpr bool kU64 = TileShared<Codec, BZ, RM>::kU64, k64 = sizeof(Real) == 8, kG = Codec::kGrid;
+    const Win64 W = sh.win();
+    const GridTab T = sh.tab();
     const ColTab64 cols64{S.cols, S.ncols};  // FP64: the columns' constants, 1 / r among them
-    // 16-bit storage: the column constants of the window's columns
-    constexpr bool kG = Codec::kGrid;
-    __shared__ float4 sgA[kG ? LD : 1], sgD[kG ? LD : 1];
-    __shared__ uint4 sgH[kG ? LD : 1];
-    const GridTab T{sgA, sgD, sgH};
-    const TileGeo g = reinterpret_cast<const TileGeo*>(tiles + ntiles)[blockIdx.x];
-    const int q = threadIdx.y * kTR + threadIdx.x;
-    constexpr int kCW = kCaseWords<Real>;                // words of the case record
-    constexpr int kRC = (NRING + kTR * BZ - 1) / (kTR * BZ);        // ring cells per thread
+    constexpr int kRC = (NRING + kTR * BZ - 1) / (kTR * BZ);  // ring cells per thread
     constexpr int kB = Block<Codec>::bytes;
     // 1. every global load of the window phase leaves before any of them is
-    //    used, addressed from the tile's TileGeo record alone: this thread's
-    //    word of the case record, the node's own values (out of the domain:
-    //    its ghost node's f), and the f of this thread's ring cells
-    int32_t cw = 0;
-    if (q < kCW) cw = reinterpret_cast<const int32_t*>(cases + g.c)[q];
-    pdl_wait();
-    // L2 prefetch of the blocks of the tile one resident wave ahead (a CTA
-    // that will start about when this one ends): one tensor prefetch, issued
-    // by one thread; the tensor maps are absent when they could not be made
-    if (maps != nullptr && q == 0 && (int)blockIdx.x + ahead < ntiles) {
-        const TileDev tp = tiles[blockIdx.x + ahead];
-        const CUtensorMap* M = maps + ((size_t)tp.c * 2 + map_set) * kMapsPerCase + 2 + parity;
-        tensormap_acquire(M);
-        tma_prefetch_4d(M, 0, 0, tp.j0 >> 5, tp.k0);
-    }
+    //    used, addressed from the tile's TileGeo record alone: the node's own
+    //    values (out of the domain: its ghost node's f), and the f of this
+    //    thread's ring cells
     unsigned char* const base = const_cast<unsigned char*>(S.in) + (int64_t)g.blk0 * kB;  // the case's first block
     auto node_at = [&](int kk, int jj) { return Node<Codec>{base + (int64_t)(kk * g.rowblk + (jj >> 5)) * kB, jj & 31}; };
     const int j = g.j0 + threadIdx.x;
@@ -630,7 +631,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     };
     auto put_phi = [&](int cell, Real v) {
         if constexpr (kU64) W.put(cell, v);
-        else sphi[cell] = v;
+        else sh.phi[cell] = v;
     };
 #pragma unroll
     for (int c = 0; c < kRC; ++c) {
@@ -642,7 +643,7 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
             PT rf[8];
             load_phi_raw<Codec>(node_at(ghost_z(g.k0 - 2 + ra, g.nz, g.zper), rj), rf0, rf);
             if constexpr (k64) put_phi(ra * LD + rb, phi_of<Codec>(rf0, rf, cols64.inv_r(rj)));
-            else sphi[ra * LD + rb] = phi_of<Codec>(rf0, rf, rcp_((Real)rj + (Real)0.5), sa_of(rj));
+            else sh.phi[ra * LD + rb] = phi_of<Codec>(rf0, rf, rcp_((Real)rj + (Real)0.5), sa_of(rj));
         }
     }
     const Real r = (Real)j + (Real)0.5;
@@ -655,34 +656,31 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     Pre64 pre6;
     if (inside) {
         if constexpr (sizeof(PT) == 2) {
-            sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_(r), sa_of(j));
+            sh.phi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_(r), sa_of(j));
         } else if constexpr (kU64) {
             const Real f[9] = {f0raw, fraw[0], fraw[1], fraw[2], fraw[3], fraw[4], fraw[5], fraw[6], fraw[7]};
             pre64<RM>(f, graw, pre6);
             own_phi = pre6.T * cols64.inv_r(j);
             put_phi((threadIdx.y + 2) * LD + bo, own_phi);
         } else if constexpr (k64) {
-            sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, cols64.inv_r(j));
+            sh.phi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, cols64.inv_r(j));
             node_pre<Codec>(f0raw, fraw, graw, r, pre, nullptr, GridCol{});
         } else {
             Real sum = (Real)f0_value(f0raw);
 #pragma unroll
             for (int i = 1; i < 9; ++i) sum += Codec::dec_f(fraw[i - 1], (Real)w_of(i) * r);
-            sphi[(threadIdx.y + 2) * LD + bo] = sum * rcp_(r);
+            sh.phi[(threadIdx.y + 2) * LD + bo] = sum * rcp_(r);
         }
     } else {
         const int jm = ghost_r(j, g.nr);
         if constexpr (k64) put_phi((threadIdx.y + 2) * LD + bo, phi_of<Codec>(f0raw, fraw, cols64.inv_r(jm)));
-        else sphi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_((Real)jm + (Real)0.5), sa_of(jm));
+        else sh.phi[(threadIdx.y + 2) * LD + bo] = phi_of<Codec>(f0raw, fraw, rcp_((Real)jm + (Real)0.5), sa_of(jm));
     }
-    // 3. the column tables and the case record into shared memory
-    if constexpr (kG) {
-        if (q < LD) grid_tab_fill<Codec>(T, q, g.j0, g.nr);
-    }
-    if (q < kCW) reinterpret_cast<int32_t*>(&sC)[q] = cw;
+    // 3. the column table and the case record into shared memory
+    fill_tile<Codec, BZ, RM>(sh, g, q, cw);
     __syncthreads();
     if (!inside) return;
-    const CaseDev& C = sC;
+    const CaseDev& C = sh.C;
     const CaseView<Codec> V = case_view<Codec>(S, C);
     const int loc = k * C.pitch + j;
     // the lagged pressure p^{n-1}, read only under the lagged coupling
@@ -705,21 +703,45 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
 
     if constexpr (kG) {
         const TabCols cols{T, j == 0 ? bo : bo - 1, bo, j + 1 == C.nr ? bo : bo + 1};
-        node_update_grid<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
+        node_update_grid<Codec, RM, LD>(C, V, sh.phi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
                                         chr_prev, p_prev, f, cols);
     } else if constexpr (kU64) {
         node_update64<RM, LD>(C, V, W, threadIdx.y + 2, bo, own_phi, k, j, loc, cols64.at(j), pre6,
                               chz_prev, chr_prev, p_prev);
     } else {
         if constexpr (k64) {
-            node_update_pre<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, pre, chz_prev, chr_prev,
+            node_update_pre<Codec, RM, LD>(C, V, sh.phi, threadIdx.y + 2, bo, k, j, loc, pre, chz_prev, chr_prev,
                                            p_prev, k64 ? cols64.d + cols64.n + j - bo : nullptr, NoCols{});
         } else {
-            node_update<Codec, RM, LD>(C, V, sphi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
+            node_update<Codec, RM, LD>(C, V, sh.phi, threadIdx.y + 2, bo, k, j, loc, f0raw, fraw, graw, chz_prev,
                                        chr_prev, p_prev, nullptr, kKeepF ? f : nullptr,
                                        NoCols{});
         }
     }
+}
+
+// One time step for every node of every tile in `tiles`: one CTA per tile.
+template <class Codec, int BZ, int RM>
+__global__ void __launch_bounds__(kTR * BZ, (step_min_blocks<Codec, BZ, RM>()))
+step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles, StateDev<Codec> S,
+            const CUtensorMap* __restrict__ maps, int map_set, int parity, int ntiles, int ahead) {
+    __shared__ TileShared<Codec, BZ, RM> sh;
+    const TileGeo g = reinterpret_cast<const TileGeo*>(tiles + ntiles)[blockIdx.x];
+    const int q = threadIdx.y * kTR + threadIdx.x;
+    // this thread's word of the case record leaves with the loads of the window phase
+    int32_t cw = 0;
+    if (q < kCaseWords<typename Codec::Real>) cw = reinterpret_cast<const int32_t*>(cases + g.c)[q];
+    pdl_wait();
+    // L2 prefetch of the blocks of the tile one resident wave ahead (a CTA
+    // that will start about when this one ends): one tensor prefetch, issued
+    // by one thread; the tensor maps are absent when they could not be made
+    if (maps != nullptr && q == 0 && (int)blockIdx.x + ahead < ntiles) {
+        const TileDev tp = tiles[blockIdx.x + ahead];
+        const CUtensorMap* M = maps + ((size_t)tp.c * 2 + map_set) * kMapsPerCase + 2 + parity;
+        tensormap_acquire(M);
+        tma_prefetch_4d(M, 0, 0, tp.j0 >> 5, tp.k0);
+    }
+    step_tile<Codec, BZ, RM>(S, sh, g, q, cw);
 }
 
 // The step with two nodes per thread, one after the other: thread (x, y) of
