@@ -1133,7 +1133,8 @@ __device__ __forceinline__ Dest destination(int k, int j, int nr, int nz, int zp
 // pdl_trigger lets the next launch start before this CTA ends.  At a kernel's
 // start that is slower: the next step's CTAs gather on few SMs (128 x 256 drop
 // 3.44 us in FP32, 16.1 against 11.4 in FP64), so only the packed kernel uses
-// it, after its window barrier.  Without the attribute both do nothing.
+// it, after its window barrier and with more tiles than fit at once.  Without
+// the attribute both do nothing.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

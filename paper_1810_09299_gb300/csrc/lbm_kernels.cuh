@@ -777,21 +777,25 @@ step_kernel_seq2(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
     using F0T = typename Codec::F0T;
     constexpr int TZ = 2 * BZ;
     constexpr int NS = STASH ? kTR * BZ : 1;
-    __shared__ F0T st_f0[NS];
-    __shared__ PT2 st_pr[8][NS];
-    __shared__ PT st_g0[NS];
-    __shared__ Real st_chz[NS], st_chr[NS];
     constexpr int LD = kTR + 4;
     constexpr int NRING = 4 * kTR + 4 * (TZ + 4);
     static_assert(NRING == (TZ + 4) * LD - TZ * kTR, "the ring is the window without the tile");
     static_assert(sizeof(Real) == 4, "FP32 arithmetic");
-    __shared__ Real sphi[(TZ + 4) * LD];
-    __shared__ __align__(16) CaseDev sC;
     static_assert(sizeof(CaseDev) % 4 == 0 && sizeof(CaseDev) / 4 <= kTR * BZ, "one word per thread");
     constexpr bool kG = Codec::kGrid;
-    __shared__ float4 sgA[kG ? LD : 1], sgD[kG ? LD : 1];
-    __shared__ uint4 sgH[kG ? LD : 1];
-    const GridTab T{sgA, sgD, sgH};
+    __shared__ struct {
+        __align__(16) CaseDev C;
+        float4 gA[kG ? LD : 1], gD[kG ? LD : 1];
+        uint4 gH[kG ? LD : 1];
+        Real phi[(TZ + 4) * LD];
+        F0T st_f0[NS];
+        PT2 st_pr[8][NS];
+        PT st_g0[NS];
+        Real st_chz[NS], st_chr[NS];
+    } sh;
+    CaseDev& sC = sh.C;
+    Real* const sphi = sh.phi;
+    const GridTab T{sh.gA, sh.gD, sh.gH};
     const TileGeo g = reinterpret_cast<const TileGeo*>(tiles + ntiles)[blockIdx.x];
     const int q = threadIdx.y * kTR + threadIdx.x;
     constexpr int kCW = kCaseWords<Real>;  // words of the case record
@@ -882,17 +886,17 @@ step_kernel_seq2(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
         // the second node's inputs to shared memory (one slot per thread)
         const int q = threadIdx.y * kTR + threadIdx.x;
         if (in[1]) {
-            st_f0[q] = f0raw[1];
+            sh.st_f0[q] = f0raw[1];
 #pragma unroll
             for (int i = 1; i < 9; ++i) {
                 PT2 pr;
                 pr.x = fraw[1][i - 1];
                 pr.y = graw[1][i];
-                st_pr[i - 1][q] = pr;
+                sh.st_pr[i - 1][q] = pr;
             }
-            st_g0[q] = graw[1][0];
-            st_chz[q] = chz_prev[1];
-            st_chr[q] = chr_prev[1];
+            sh.st_g0[q] = graw[1][0];
+            sh.st_chz[q] = chz_prev[1];
+            sh.st_chr[q] = chr_prev[1];
         }
     }
     __syncthreads();
@@ -913,16 +917,16 @@ step_kernel_seq2(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
             // above the first node's update
             asm volatile("" ::: "memory");
             const int q = threadIdx.y * kTR + threadIdx.x;
-            f0raw[1] = st_f0[q];
+            f0raw[1] = sh.st_f0[q];
 #pragma unroll
             for (int i = 1; i < 9; ++i) {
-                const PT2 pr = st_pr[i - 1][q];
+                const PT2 pr = sh.st_pr[i - 1][q];
                 fraw[1][i - 1] = pr.x;
                 graw[1][i] = pr.y;
             }
-            graw[1][0] = st_g0[q];
-            chz_prev[1] = st_chz[q];
-            chr_prev[1] = st_chr[q];
+            graw[1][0] = sh.st_g0[q];
+            chz_prev[1] = sh.st_chz[q];
+            chr_prev[1] = sh.st_chr[q];
         }
         if constexpr (kG) {
             const TabCols cols{T, j == 0 ? bo : bo - 1, bo, j + 1 == C.nr ? bo : bo + 1};
@@ -1035,7 +1039,12 @@ __device__ __forceinline__ void pack2_finish(const CaseDev& C, const CaseView<Co
 #define AXILBM_PACK2_CTAS 3
 #endif
 
-template <class Codec, int RM>
+// EARLY: the next step's first CTAs may take the places that free up while this
+// step's last ones run (see pdl_trigger), for launches of more tiles than are
+// resident at once: 512 cases 565.1 -> 558.3 us, 256 x 1024 7.62 -> 7.55; with fewer
+// tiles they gather on few SMs (200 x 600 4.89 -> 5.40).  As a run-time branch it
+// cost 571.2: the compiler schedules around it.
+template <class Codec, int RM, bool EARLY>
 __global__ void __launch_bounds__(kTR * 8, AXILBM_PACK2_CTAS)
 step_kernel_pack2(const CaseDev* __restrict__ cases, const TileGeo* __restrict__ geo, StateDev<Codec> S,
                   const CUtensorMap* __restrict__ maps, int parity, int ntiles, int ahead) {
@@ -1046,11 +1055,15 @@ step_kernel_pack2(const CaseDev* __restrict__ cases, const TileGeo* __restrict__
     constexpr int NRING = 4 * kTR + 4 * (TZ + 4);
     static_assert(NRING <= kTR * BZ, "one ring cell per thread at most");
     constexpr int kB = Block<Codec>::bytes;
-    __shared__ float2 spair[NP * LD];
-    __shared__ __align__(16) CaseDev sC;
-    __shared__ float4 sgA[LD], sgD[LD];
-    __shared__ uint4 sgH[LD];
-    const GridTab T{sgA, sgD, sgH};
+    __shared__ struct {
+        __align__(16) CaseDev C;
+        float4 gA[LD], gD[LD];
+        uint4 gH[LD];
+        float2 pair[NP * LD];
+    } sh;
+    CaseDev& sC = sh.C;
+    float2* const spair = sh.pair;
+    const GridTab T{sh.gA, sh.gD, sh.gH};
     const TileGeo g = geo[blockIdx.x];
     const int q = threadIdx.y * kTR + threadIdx.x;
     constexpr int kCW = kCaseWords<float>;  // words of the case record
@@ -1136,10 +1149,7 @@ step_kernel_pack2(const CaseDev* __restrict__ cases, const TileGeo* __restrict__
     float2 mf[9], mg[9], g0;
     pack2_moments<Codec>(grid_col<Codec>(j), f0raw, fraw, graw, mf, mg, g0);
     __syncthreads();
-    // more tiles than CTAs at once: the next step's first CTAs may take the
-    // places that free up (512 cases 565.7 -> 558.0 us); with fewer the early start
-    // packs them unevenly on the SMs (the 200 x 600 thread 4.97 -> 5.40 us)
-    if (ntiles > ahead) pdl_trigger();
+    if constexpr (EARLY) pdl_trigger();
     if (!in[0]) return;  // the second node lies below the first
     const CaseDev& C = sC;
     const CaseView<Codec> V = case_view<Codec>(S, C);
@@ -1730,8 +1740,10 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
             break;
         case 7:
             if constexpr (Codec::kGrid)
-                launch_step_kernel(step_kernel_pack2<Codec, RM>, ntiles, dim3(kTR, 8), st, cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps, parity, ntiles,
-                    kPrefetchQuarters * sms * AXILBM_PACK2_CTAS / 4);
+                launch_step_kernel(ntiles > sms * AXILBM_PACK2_CTAS ? step_kernel_pack2<Codec, RM, true>
+                                                                    : step_kernel_pack2<Codec, RM, false>,
+                                   ntiles, dim3(kTR, 8), st, cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps,
+                                   parity, ntiles, kPrefetchQuarters * sms * AXILBM_PACK2_CTAS / 4);
             else if constexpr (sizeof(typename Codec::Real) == 4)
                 launch_step_kernel(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
             else
