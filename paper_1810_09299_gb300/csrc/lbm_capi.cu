@@ -105,8 +105,7 @@ struct lbm_sim {
     double* partials = nullptr;
     double* diag_out = nullptr;
     double* axis_rows = nullptr;   // 2 nz doubles of the tallest case
-    double* axis_out = nullptr;    // the drops record, 3 + 4 * kMaxAxisDrops doubles
-    double* axis_host = nullptr;   // pinned copy of axis_out
+    double* axis_host = nullptr;   // the drops record, 3 + 4 * kMaxAxisDrops doubles (pinned)
     // pinned host staging for small reads (a diagnostics record and the
     // status word), so that they return with one synchronisation
     double* host_small = nullptr;
@@ -170,14 +169,15 @@ cudaError_t launch_step_any(lbm_sim* h, int parity, int variant, cudaStream_t st
 }
 
 // The fields of case icase: all five, or phi alone.
-cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st, bool phi_only = false) {
+cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st, bool phi_only = false,
+                              int* status_out = nullptr) {
     const TileDev* t = h->ftiles_d[icase];
     const int n = h->nftiles[icase];
     switch (h->precision) {
-        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, h->fields, st);
-        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, h->fields, st);
-        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, h->fields, st);
-        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, h->fields, st);
+        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
+        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
+        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
+        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
     }
 }
 
@@ -486,7 +486,6 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
     A((void**)&h->partials, diag_partials_size() * sizeof(double));
     A((void**)&h->diag_out, 16 * sizeof(double));
     A((void**)&h->axis_rows, 2 * (size_t)max_nz * sizeof(double));
-    A((void**)&h->axis_out, (3 + 4 * kMaxAxisDrops) * sizeof(double));
     A((void**)&h->D.status, 128);
     if (rc == LBM_OK && cudaMallocHost((void**)&h->host_small, 16 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
@@ -609,12 +608,9 @@ int step_direct(lbm_sim* h, int64_t n) {
 }
 
 // Device status word: set by a bounded wait that gave up (TMA-staged step).  A
-// read-back enqueues its copy (into pinned memory) beside its own and looks at
-// it after the one synchronisation that ends the call.
+// read-back's last kernel also stores it here (pinned memory), and the call
+// looks at it after the one synchronisation that ends it.
 int* status_host(lbm_sim* h) { return (int*)(h->host_small + 12); }
-int enqueue_status(lbm_sim* h) {
-    return cuda_ok(h, cudaMemcpyAsync(status_host(h), h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-}
 int finish_status(lbm_sim* h) {
     const int rc = cuda_ok(h, cudaStreamSynchronize(h->stream));
     if (rc != LBM_OK) return rc;
@@ -658,8 +654,9 @@ int join_diagnostics(lbm_sim* h) {
 }
 
 // Enqueue the fields and the reductions of case icase, then the copies of the
-// 11-double record to `record` and of the device status word to `status`
-// (host memory), on stream `st`.  When st is the diagnostics stream, the
+// 11-double record to `record` (host memory; stored there by the last kernel
+// itself when it is the handle's pinned host_small) and of the device status
+// word to `status` (pinned), on stream `st`.  When st is the diagnostics stream, the
 // fields' read of the state is ordered after the work already on the handle's
 // stream, and the handle's stream waits for that read only.  Does not wait.
 int enqueue_diagnostics(lbm_sim* h, int icase, double* record, int* status, cudaStream_t st) {
@@ -680,12 +677,11 @@ int enqueue_diagnostics(lbm_sim* h, int icase, double* record, int* status, cuda
         if (rc != LBM_OK) return rc;
     }
     const lbm_params& p = h->prm[icase];
+    const bool pinned = record == h->host_small;
     rc = cuda_ok(h, launch_diag(h->fields, p.nz, p.nr, p.z_periodic, (double)h->case_steps[icase], h->partials,
-                                h->diag_out, st));
-    if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, cudaMemcpyAsync(record, h->diag_out, 11 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, cudaMemcpyAsync(status, h->D.status, sizeof(int), cudaMemcpyDeviceToHost, st));
+                                pinned ? record : h->diag_out, h->D.status, status, st));
+    if (rc == LBM_OK && !pinned)
+        rc = cuda_ok(h, cudaMemcpyAsync(record, h->diag_out, 11 * sizeof(double), cudaMemcpyDeviceToHost, st));
     if (rc != LBM_OK || !side) return rc;
     rc = cuda_ok(h, cudaEventRecord(h->ev_diag, st));
     if (rc == LBM_OK) h->diag_pending = true;
@@ -796,8 +792,7 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
     if (!h->initialized[icase]) return LBM_ERR_STATE;
     rc = join_diagnostics(h);
     if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI));
-    if (rc == LBM_OK) rc = enqueue_status(h);
+    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI, status_host(h)));
     if (rc != LBM_OK) return rc;
     const int64_t n = (int64_t)h->prm[icase].nz * h->prm[icase].nr;
     int64_t slot = 0;
@@ -851,12 +846,8 @@ int lbm_case_axis_drops(lbm_handle* h, int32_t icase, int32_t max_drops, lbm_dro
     rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, true));
     if (rc != LBM_OK) return rc;
     const lbm_params& p = h->prm[icase];
-    rc = cuda_ok(h, launch_axis_drops(h->fields, p.nz, p.nr, p.z_periodic, max_drops, h->axis_rows, h->axis_out,
-                                      h->stream));
-    if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, cudaMemcpyAsync(h->axis_host, h->axis_out, (3 + 4 * (size_t)max_drops) * sizeof(double),
-                                    cudaMemcpyDeviceToHost, h->stream));
-    if (rc == LBM_OK) rc = enqueue_status(h);
+    rc = cuda_ok(h, launch_axis_drops(h->fields, p.nz, p.nr, p.z_periodic, max_drops, h->axis_rows, h->axis_host,
+                                      h->D.status, status_host(h), h->stream));
     if (rc == LBM_OK) rc = finish_status(h);
     if (rc != LBM_OK) return rc;
     const int n = (int)h->axis_host[0];

@@ -1,5 +1,4 @@
-// lbm_diag.cu -- FP64 diagnostics of one case (compensated, deterministic
-// reductions) and the initial phase-field shapes of the paper's tests (Sec. 3).
+// lbm_diag.cu -- FP64 diagnostics of one case (deterministic reductions) and the initial phase-field shapes of the paper's tests (Sec. 3).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -16,46 +15,61 @@ namespace {
 constexpr int kDiagBlocks = kDiagPartials / 18;  // 2 x 152 SMs; fixed so the summation order is fixed
 constexpr int kDiagThreads = 256;
 
-// Neumaier compensated accumulation.
-struct KSum {
-    double s, c;
-    __device__ void add(double x) {
-        const double t = s + x;
-        if (fabs(s) >= fabs(x)) c += (s - t) + x;
-        else c += (x - t) + s;
-        s = t;
-    }
-    __device__ void merge(const KSum& o) {
-        add(o.s);
-        c += o.c;
-    }
-    __device__ double value() const { return s + c; }
-};
-
 // Quantities: 0 mass, 1 kinetic, 2 z-moment, 3 p in liquid, 4 weight in liquid,
 // 5 p in gas, 6 weight in gas (sums); 7 max |u|^2, 8 phi_min, 9 phi_max
 // (extrema); 10 non-finite count (sum).  A partial record is 18 doubles:
-// (sum, compensation) of quantities 0-6, then 7-10.
+// (sum, 0) of quantities 0-6, then 7-10.
 constexpr int kSums = 7;
 
-// A compensated pair (s, c) from lane + off of the warp (a shuffle of both).
-__device__ __forceinline__ KSum shfl_down_ksum(const KSum& x, int off) {
-    return KSum{__shfl_down_sync(0xffffffffu, x.s, off), __shfl_down_sync(0xffffffffu, x.c, off)};
-}
-
-// Combine the compensated pairs (v, vc)[0 .. count) held in shared memory with
-// stride `stride` (one per partial record) into lane 0 of the calling warp:
-// each lane merges its share in a fixed order, then a fixed shuffle tree
-// merges the lanes.  Every sum is compensated (Neumaier).
-__device__ __forceinline__ KSum warp_ksum(const double* v, const double* vc, int count, int stride) {
+// The sum of v[0 .. count) (stride `stride`, count <= 512) into every lane of the
+// calling warp, exact to its last rounding: the values as 128-bit integers in
+// units of 2^-64 of the last place of the largest one.  Compensated (Neumaier)
+// sums in FP64 took most of diag_final_kernel's 19.5 us: some 100 dependent
+// operations of a pipe that takes a warp instruction every 20 cycles; this takes
+// 8.  Values of 2^1007 and more, infinities and NaN are summed plainly.
+__device__ __forceinline__ double warp_exact_sum(const double* v, int count, int stride) {
     const int lane = threadIdx.x & 31;
-    KSum acc{0.0, 0.0};
-    for (int i = lane; i < count; i += 32) acc.merge(KSum{v[(size_t)i * stride], vc[(size_t)i * stride]});
-    for (int off = 16; off > 0; off >>= 1) {
-        const KSum o = shfl_down_ksum(acc, off);
-        if (lane + off < 32) acc.merge(o);
+    int top = 0;
+    for (int i = lane; i < count; i += 32) top = max(top, __double2hiint(v[(size_t)i * stride]) & 0x7fffffff);
+    const int E = max((int)(__reduce_max_sync(0xffffffffu, (unsigned)top) >> 20), 1);
+    if (E >= 2030) {
+        double acc = 0.0;
+        for (int i = lane; i < count; i += 32) acc += v[(size_t)i * stride];
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        return acc;
     }
-    return acc;
+    __int128 acc = 0;
+    for (int i = lane; i < count; i += 32) {
+        const double x = v[(size_t)i * stride];
+        const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+        const unsigned long long m =
+            ((unsigned long long)(((uint32_t)hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
+        const int sh = E - max(e, 1);  // subnormal numbers share the exponent of the smallest normal ones
+        const unsigned __int128 y = sh < 128 ? ((unsigned __int128)m << 64) >> sh : (unsigned __int128)0;
+        acc += hi < 0 ? -(__int128)y : (__int128)y;
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, off);
+        const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(acc >> 64), off);
+        acc += ((__int128)hi << 64) | lo;
+    }
+    // one rounding: |acc| below 2^126 with its leading bit brought to bit 62 of
+    // 64, the bits below folded into the last one
+    const bool neg = acc < 0;
+    unsigned __int128 a = neg ? -(unsigned __int128)acc : (unsigned __int128)acc;
+    const unsigned long long ah = (unsigned long long)(a >> 64), al = (unsigned long long)a;
+    if ((ah | al) == 0) return 0.0;
+    const int lead = ah ? 127 - __clzll((long long)ah) : 63 - __clzll((long long)al);
+    const int down = lead - 62;
+    unsigned long long r;
+    if (down > 0) {
+        r = (unsigned long long)(a >> down);
+        if ((a & (((unsigned __int128)1 << down) - 1)) != 0) r |= 1ull;
+    } else {
+        r = (unsigned long long)(a << -down);
+    }
+    const double d = scalbn(__ull2double_rn(r), E - 1075 - 64 + down);
+    return neg ? -d : d;
 }
 
 // The plain sum of v[0 .. count) (stride as above) into lane 0: each lane adds
@@ -102,7 +116,7 @@ __device__ __forceinline__ void warp_extrema(const double* uu, const double* lo,
 // thread holds only a few nodes and sums them plainly; the block's 256 values
 // of each quantity are then summed pairwise by one warp per quantity (warps
 // 0-6 the sums, warp 7 the extrema and the count).  The records of the blocks
-// are combined with compensated sums by diag_final_kernel.
+// are combined exactly by diag_final_kernel.
 __global__ void __launch_bounds__(kDiagThreads) diag_partial_kernel(const double* __restrict__ F, int nz, int nr,
                                                                     double* __restrict__ partials) {
     static_assert(kDiagThreads == 32 * (kSums + 1), "one warp per sum plus one");
@@ -177,48 +191,40 @@ __device__ __forceinline__ double axis_link(const double* __restrict__ F, int k,
 }
 
 // Final combination and the interface lengths, one block of kFinalThreads:
-// warps 0-6 combine one sum each over the partial records and warp 7 the
-// extrema and the count, every one in a fixed order (compensated sums), so
-// the result is deterministic.
+// warps 0-6 combine one sum each over the partial records (exact, see
+// warp_exact_sum) and warp 7 the extrema and the count, every one in a fixed
+// order, so the result is deterministic.  A case of fewer rows than blocks has
+// records only for its rows.
 constexpr int kFinalThreads = 256;
 static_assert(kFinalThreads == 32 * (kSums + 1), "one warp per sum plus one");
 __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double* __restrict__ F, int nz, int nr,
                                                                    int zper, double step,
                                                                    const double* __restrict__ partials,
-                                                                   double* __restrict__ out) {
-    __shared__ double sp[kDiagBlocks][18];
-    __shared__ double sres[18];
-    __shared__ double slen[kFinalThreads];
+                                                                   double* __restrict__ out, const int* status,
+                                                                   int* status_out) {
+    __shared__ double sres[kSums + 4];
+    __shared__ double slen[kFinalThreads / 32];
     __shared__ int sjmin;
-    const int t = threadIdx.x;
-    for (int i = t; i < kDiagBlocks * 18; i += kFinalThreads) (&sp[0][0])[i] = partials[i];
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const int records = min(nz, kDiagBlocks);
     if (t == 0) sjmin = nr;
-    __syncthreads();
-    const int w = t >> 5;
-    if (w < kSums) {
-        const KSum r = warp_ksum(&sp[0][2 * w], &sp[0][2 * w + 1], kDiagBlocks, 18);
-        if ((t & 31) == 0) {
-            sres[2 * w] = r.s;
-            sres[2 * w + 1] = r.c;
-        }
-    } else {
-        double e[4];
-        warp_extrema(&sp[0][14], &sp[0][15], &sp[0][16], &sp[0][17], kDiagBlocks, 18, e);
-        if ((t & 31) == 0)
-            for (int q = 0; q < 4; ++q) sres[14 + q] = e[q];
-    }
-    // axis half-length: per-thread sums over k = t, t + T, ... then a halving tree
+    // axis half-length: per-thread sums over k = t, t + T, ..., then a shuffle tree
     double len = 0.0;
     for (int k = t; k < nz; k += kFinalThreads) len += axis_link(F, k, nz, nr, zper);
-    slen[t] = len;
-    __syncthreads();
-    for (int stride = kFinalThreads / 2; stride > 0; stride >>= 1) {
-        if (t < stride) slen[t] += slen[t + stride];
-        __syncthreads();
+    for (int off = 16; off > 0; off >>= 1) len += __shfl_down_sync(0xffffffffu, len, off);
+    if (lane == 0) slen[w] = len;
+    if (w < kSums) {
+        const double r = warp_exact_sum(partials + 2 * w, records, 18);
+        if (lane == 0) sres[w] = r;
+    } else {
+        double e[4];
+        warp_extrema(partials + 14, partials + 15, partials + 16, partials + 17, records, 18, e);
+        if (lane == 0)
+            for (int q = 0; q < 4; ++q) sres[kSums + q] = e[q];
     }
     __syncthreads();
-    const double mass = KSum{sres[0], sres[1]}.value();
-    const double zc = KSum{sres[4], sres[5]}.value() / mass;
+    const double mass = sres[0];
+    const double zc = sres[2] / mass;
     // radial crossing on the row nearest the centroid: the first outward crossing
     int kc = (int)floor(zc);
     kc = kc < 0 ? 0 : (kc >= nz ? nz - 1 : kc);
@@ -236,22 +242,23 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
         const double a = F[(int64_t)kc * nr + sjmin] - 0.5, b = F[(int64_t)kc * nr + sjmin + 1] - 0.5;
         rc = (sjmin + 0.5) + a / (a - b);
     }
-    double axis = slen[0];
+    double axis = 0.0;
+    for (int i = 0; i < kFinalThreads / 32; ++i) axis += slen[i];
     if (!zper && F[0] - 0.5 > 0) axis += 0.5;
-    const double win = KSum{sres[8], sres[9]}.value(), wout = KSum{sres[12], sres[13]}.value();
-    const double dp = (win > 0 ? KSum{sres[6], sres[7]}.value() / win : 0.0) -
-                      (wout > 0 ? KSum{sres[10], sres[11]}.value() / wout : 0.0);
+    const double win = sres[4], wout = sres[6];
+    const double dp = (win > 0 ? sres[3] / win : 0.0) - (wout > 0 ? sres[5] / wout : 0.0);
     out[0] = step;
     out[1] = mass;
-    out[2] = KSum{sres[2], sres[3]}.value();
+    out[2] = sres[1];
     out[3] = zc;
     out[4] = dp;
-    out[5] = sqrt(sres[14]);  // |u|max from the largest |u|^2
-    out[6] = sres[15];
-    out[7] = sres[16];
+    out[5] = sqrt(sres[kSums]);  // |u|max from the largest |u|^2
+    out[6] = sres[kSums + 1];
+    out[7] = sres[kSums + 2];
     out[8] = 0.5 * axis;
     out[9] = rc;
-    out[10] = sres[17];
+    out[10] = sres[kSums + 3];
+    if (status_out) *status_out = *status;
 }
 
 // ---------------------------------------------------------------- drops on the axis
@@ -327,13 +334,15 @@ __device__ __forceinline__ double sum_rows(const double* rows, int nz, int k0, i
 }
 
 __global__ void __launch_bounds__(kAxisThreads) axis_drops_kernel(const double* __restrict__ rows_g, int nz, int zper,
-                                                                  int max_drops, double* __restrict__ out) {
+                                                                  int max_drops, double* __restrict__ out,
+                                                                  const int* status, int* status_out) {
     constexpr int kWarps = kAxisThreads / 32;
     __shared__ double sbuf[2 * kAxisRows];
     __shared__ double s_min[kWarps];
     __shared__ int s_kmin[kWarps], s_gas[kWarps], s_last[kWarps], s_cnt[kWarps];
     __shared__ int s_a[kMaxAxisDrops + 1], s_b[kMaxAxisDrops + 1];  // runs of the first drops, scan indices
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    if (t == 0) *status_out = *status;
     const bool fits = nz <= kAxisRows;
     for (int i = t; fits && i < 2 * nz; i += kAxisThreads) sbuf[i] = rows_g[i];
     __syncthreads();
@@ -521,17 +530,17 @@ __global__ void shape_kernel(int shape, ShapeArgs A, int nz, int nr, double* __r
 int diag_partials_size() { return kDiagPartials; }
 
 cudaError_t launch_diag(const double* fields, int nz, int nr, int zper, double step, double* partials, double* out,
-                        cudaStream_t st) {
-    diag_partial_kernel<<<kDiagBlocks, kDiagThreads, 0, st>>>(fields, nz, nr, partials);
-    diag_final_kernel<<<1, kFinalThreads, 0, st>>>(fields, nz, nr, zper, step, partials, out);
+                        const int* status, int* status_out, cudaStream_t st) {
+    diag_partial_kernel<<<nz < kDiagBlocks ? nz : kDiagBlocks, kDiagThreads, 0, st>>>(fields, nz, nr, partials);
+    diag_final_kernel<<<1, kFinalThreads, 0, st>>>(fields, nz, nr, zper, step, partials, out, status, status_out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_axis_drops(const double* fields, int nz, int nr, int zper, int max_drops, double* rows, double* out,
-                              cudaStream_t st) {
+                              const int* status, int* status_out, cudaStream_t st) {
     constexpr int per = kAxisThreads / 32;
     axis_rows_kernel<<<(nz + per - 1) / per, kAxisThreads, 0, st>>>(fields, nz, nr, rows);
-    axis_drops_kernel<<<1, kAxisThreads, 0, st>>>(rows, nz, zper, max_drops, out);
+    axis_drops_kernel<<<1, kAxisThreads, 0, st>>>(rows, nz, zper, max_drops, out, status, status_out);
     return cudaGetLastError();
 }
 
@@ -679,7 +688,8 @@ extern "C" int lbm_diag_reduce_noalloc(const double* d_fields, int32_t nz, int32
     }
     // Every partial slot is overwritten by the first kernel before the second
     // reads it, so nothing from an earlier call needs clearing.
-    cudaError_t e = axilbm::launch_diag(d_fields, nz, nr, z_periodic, step, scratch, d_out, (cudaStream_t)stream);
+    cudaError_t e = axilbm::launch_diag(d_fields, nz, nr, z_periodic, step, scratch, d_out, nullptr, nullptr,
+                                         (cudaStream_t)stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return LBM_ERR_CUDA;

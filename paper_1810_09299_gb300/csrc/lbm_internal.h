@@ -42,7 +42,7 @@ struct DeviceState {
     cudaError_t launch_step_##NAME(const DeviceState& D, int parity, int variant, const TileDev* tiles, int ntiles, \
                                    cudaStream_t st);                                                               \
     cudaError_t launch_fields_##NAME(const DeviceState& D, int parity, const TileDev* tiles, int ntiles,            \
-                                     bool phi_only, double* out, cudaStream_t st);                                 \
+                                     bool phi_only, double* out, int* status_out, cudaStream_t st);                \
     cudaError_t launch_init_##NAME(const DeviceState& D, int parity, const TileDev* tiles8, int ntiles,             \
                                    const double* phi0, int64_t base, cudaStream_t st);                             \
     cudaError_t launch_get_state_##NAME(const DeviceState& D, int parity, const CaseDev& C, double* f, double* g,   \
@@ -79,17 +79,19 @@ constexpr int kMapsPerCase = 4;
 
 // Diagnostics (lbm_diag.cu): reduce dense FP64 fields of one case into a
 // 11-double record; `partials` is scratch of at least diag_partials_size()
-// doubles.  Deterministic (fixed block count and order).
+// doubles.  Deterministic (fixed block count and order).  out and status_out
+// may be pinned host memory; with status_out the device status word is copied
+// there as well.
 constexpr int kDiagPartials = 304 * 18;  // 304 blocks x 18 doubles
 int diag_partials_size();
 cudaError_t launch_diag(const double* fields, int nz, int nr, int zper, double step, double* partials,
-                        double* out, cudaStream_t st);
+                        double* out, const int* status, int* status_out, cudaStream_t st);
 
 // Drops on the axis row (lbm_diag.cu): out[3 + 4 * kMaxAxisDrops] doubles,
-// rows: 2 nz doubles of scratch.
+// rows: 2 nz doubles of scratch; out and status_out as above.
 constexpr int kMaxAxisDrops = 64;
 cudaError_t launch_axis_drops(const double* fields, int nz, int nr, int zper, int max_drops, double* rows, double* out,
-                              cudaStream_t st);
+                              const int* status, int* status_out, cudaStream_t st);
 
 // Initial shapes (lbm_diag.cu): phi0 [nz][nr] on the device.
 cudaError_t launch_shape(int shape, const double* args, int nargs, int nz, int nr, double* phi0, cudaStream_t st);
