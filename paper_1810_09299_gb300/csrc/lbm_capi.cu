@@ -274,7 +274,6 @@ CaseDev make_case(const lbm_params& p, int64_t off, int64_t dense_off) {
     C.p64.dnu = p.nu_l - p.nu_g;
     C.p64.beta4 = 4.0 * C.pd.beta;
     C.p64.lam3 = 4.0 / (3.0 * p.W);
-    C.p64.neps72 = 72.0 * p.n_eps;
     C.p64.c2 = (long long)std::ldexp(0.5 * (1.0 - s), 62);
     C.p64.c4 = (long long)std::ldexp(0.25 * (1.0 - s), 62);
     auto sf = [](double x, long long& m, int32_t& e) {
@@ -286,6 +285,7 @@ CaseDev make_case(const lbm_params& p, int64_t off, int64_t dense_off) {
     sf(0.3 / 72.0 * C.p64.drho, C.p64.drho3_m, C.p64.drho3_e);
     sf((1.0 - 0.5 * s) / 3.0, C.p64.h3_m, C.p64.h3_e);
     sf((1.0 + 0.5 * s) / 3.0, C.p64.sh3_m, C.p64.sh3_e);
+    sf(72.0 * p.n_eps, C.p64.neps72_m, C.p64.neps72_e);
     return C;
 }
 

@@ -248,10 +248,9 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
     const double rho_d = fma(phi, H.drho, P.rho_g);
     const double nu = fma(phi, H.dnu, P.nu_g);
     const double tau = fma(3.0, nu, 0.5);
-    const double s_d = rcp_in(tau);
     const double rv = fma(nu, K.inv_r(), K.r());
-    const double D_d = rcp_in(rho_d * rv);
-    const Sf rho = sf_of(rho_d), s = sf_of(s_d), D = sf_of(D_d), irr = sf_of(K.inv_r() * (D_d * rv));
+    const Sf rho = sf_of(rho_d), s = rcp(sf_of(tau), m.bad), D = rcp(sf_of(rho_d * rv), m.bad);
+    const Sf irr = K.s_inv_r() * (D * sf_of(rv));
     // Eq. 4: mu~ = mu - k d_r phi / r; Eq. 30's F_z = r (F_s + G)_z
     const Sf mut = norm29(sf_of((H.beta4 * phi) * fma(phi, phi - 1.5, 0.5)) + Sf{H.mkappa_m, H.mkappa_e} * norm29(gr * K.s_inv_r() + lap));
     const Sf rm = K.r72() * mut;
@@ -268,7 +267,7 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
     const Sf A0 = uz * norm29(Z3 - A2 * uz) + K.s_i6() * Q.S0;
     const Sf A1 = norm29(sf_of(((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * K.i4()) + R3);
     // numbers that are not finite do not exist in integers: seen here, put out as NaN
-    int top = max(abs_hi(s_d), abs_hi(D_d));
+    int top = max(abs_hi(rho_d), abs_hi(nu));
     Sf ur, p, ps;
     if (C.p_coupling == 1) {
         ps = sf_of(p_prev);
@@ -285,10 +284,8 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
         const Sf qc = norm29(A0 + ca * norm29(Sf{tA.b - tA.a, tA.e}));
         const Sf disc = qb * qb + ((A2 * D) * D) * qc;
         const bool two = disc.m >= 0;
-        const double qb_d = double_of(qb);
-        const double y = rcp_in(two ? qb_d + sqrt_in(double_of(disc)) : qb_d);
-        top = max(top, abs_hi(y));
-        p = scale2(qc, two ? 1 : 0) * sf_of(y);
+        const Sf sum = qb + root(Sf{two ? disc.m : 0ll, disc.e});
+        p = scale2(qc, two ? 1 : 0) * rcp(sum, m.bad);
         ps = p;
         ur = norm29(ca + scale2(D, -1) * p);
     }
@@ -322,9 +319,7 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     {
         // r lambda / (3 (|grad phi| + n_eps)): the normal's factor of grad phi (72 in both)
         const double lam = H.lam3 * (K.r() * fma(-phi, phi, phi));
-        const double Ld = lam * rcp_in(sqrt_in(double_of(gz * gz + gr * gr)) + H.neps72);
-        top = max(top, abs_hi(Ld));
-        const Sf L = sf_of(Ld);
+        const Sf L = sf_of(lam) * rcp(root(gz * gz + gr * gr) + Sf{H.neps72_m, H.neps72_e}, bad);
         const Sf h3{H.h3_m, H.h3_e}, sh3{H.sh3_m, H.sh3_e};
         const Sf tz = h3 * norm29(L * gz - sf_of(chz_prev)) + sh3 * chz;
         const Sf tr = h3 * norm29(L * gr - sf_of(chr_prev)) + sh3 * norm29(chr);

@@ -89,12 +89,15 @@ struct Sf {
 };
 constexpr int kZeroE = -(1 << 17);
 
-// a b 2^-62, |a|, |b| < 2^62 (the low words' product, at most 4 units, is left out)
+// a b 2^-62, |a|, |b| < 2^62, short by at most 12 units (the low words' product
+// and the bits below the high words of the mixed ones are left out).  High-word
+// multiplications (30.6 per SM and cycle) rather than signed wide ones (12).
 __device__ __forceinline__ long long mul62(long long a, long long b) {
-    const int ah = (int)(a >> 32), bh = (int)(b >> 32);
-    const uint32_t al = (uint32_t)a, bl = (uint32_t)b;
-    const long long cross = (long long)ah * (int)(bl >> 1) + (long long)bh * (int)(al >> 1);
-    return (long long)(ah * 2) * (bh * 2) + (cross >> 29);
+    const int ah = (int)(a >> 32) * 2, bh = (int)(b >> 32) * 2;
+    const int al = (int)((uint32_t)a >> 1), bl = (int)((uint32_t)b >> 1);
+    const int mixed = __mulhi(ah, bl) + __mulhi(bh, al);
+    const long long high = ((long long)__mulhi(ah, bh) << 32) | (uint32_t)(ah * bh);
+    return high + (long long)mixed * 4;
 }
 __device__ __forceinline__ Sf operator*(Sf a, Sf b) { return Sf{mul62(a.m, b.m), a.e + b.e + 62}; }
 __device__ __forceinline__ Sf operator+(Sf a, Sf b) {
@@ -165,30 +168,64 @@ __device__ __forceinline__ double double_of(Sf a) {
     const double d = double_in(a.m, a.e);
     return a.e < -1000 ? 0.0 : (a.e > 900 ? nan64() : d);
 }
-// 1 / x and sqrt(x) of lbm_device.cuh's rcp64 and sqrt64 for numbers the
-// integers above can hold (x normal, or for the root zero): without their IEEE
-// forms, whose instructions a warp passes through even when no lane needs
-// them.  Zero (rcp), infinities and NaN give NaN.
-__device__ __forceinline__ double rcp_in(double x) {
-    double y0;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-    const double e = fma(-x, y0, 1.0);
-    return fma(fma(e, e, e), y0, y0);
+// The leading 64 bits of |a|, a != 0: bit 63 set.
+__device__ __forceinline__ unsigned long long lead64(long long a, int& n) {
+    const long long sg = a >> 63;
+    const unsigned long long u = (unsigned long long)((a ^ sg) - sg);
+    n = __clzll((long long)u);
+    unsigned long long v;
+    asm("shl.b64 %0, %1, %2;" : "=l"(v) : "l"(u), "r"(n));
+    return v;
 }
-__device__ __forceinline__ double sqrt_in(double x) {
-    double y0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-    const double s = x * y0;
-    const double e = fma(-s, y0, 1.0);
-    const double y = fma(s * e, fma(0.375, e, 0.5), s);
-    return (((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x)) == 0u ? 0.0 : y;
+// 1 / a, to about 2^-60 of itself; bad is raised for zero.  x = |a| scaled to
+// [1/2, 1); y0 = 1 / x from the FP32 approximation as an integer of 31 bits, e = 1 -
+// x y0 to 62 places (below 2^-22), y0 (1 + e + e^2).  An FP64 Newton step took
+// three operations of the FP64 pipe and two conversions.
+__device__ __forceinline__ Sf rcp(Sf a, bool& bad) {
+    int n;
+    const unsigned long long u = lead64(a.m, n);  // x 2^64
+    const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
+    float f;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rn(uh)));
+    const uint32_t y0 = min(__float2uint_rn(f * 0x1p62f), 0x7fffffffu);  // y 2^30
+    const long long e = (long long)((1ull << 62) - ((unsigned long long)uh * y0 + __umulhi(ul, y0)));
+    const int es = (int)(e >> 10);
+    const unsigned long long t = (unsigned long long)(e + (__mulhi(es, es) >> 10)) << 20;
+    const long long d = (((long long)__mulhi((int)(t >> 32), (int)y0) << 32) | (uint32_t)((uint32_t)(t >> 32) * y0)) +
+                        __umulhi((uint32_t)t, y0);
+    const unsigned long long y = ((unsigned long long)y0 << 32) + (unsigned long long)(d >> 18);  // y 2^62
+    bad = bad || a.m == 0;
+    const long long m = (long long)((y - 1) >> 1), sg = a.m >> 63;  // below 2^62 for x = 1/2, too
+    return Sf{(m ^ sg) - sg, n - a.e - 125};
+}
+// sqrt(a), a >= 0, to about 2^-59 of itself.  v = a scaled by an even power of two to
+// [1/4, 1); r0 = 1 / sqrt(v) from the FP32 approximation, e = 1 - v r0^2, s = v r0
+// (1 + e / 2 + 3 e^2 / 8).
+__device__ __forceinline__ Sf root(Sf a) {
+    int n;
+    unsigned long long v = lead64(a.m, n);
+    const int ex = 64 - n + a.e, odd = ex & 1;  // a = (v 2^-64) 2^ex
+    v >>= odd;
+    const uint32_t vh = (uint32_t)(v >> 32), vl = (uint32_t)v;
+    float f;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rn(vh)));
+    const uint32_t r0 = min(__float2uint_rn(f * 0x1p46f), 0x7fffffffu);  // 2^30 / sqrt(v)
+    const unsigned long long w = (unsigned long long)r0 * r0;          // 2^60 / v
+    const uint32_t wh = (uint32_t)(w >> 32), wl = (uint32_t)w;
+    const unsigned long long vw = (unsigned long long)vh * wh + __umulhi(vh, wl) + __umulhi(vl, wh);
+    const long long e = (long long)((1ull << 60) - vw);
+    const int es = (int)(e >> 8);
+    const long long t = (e >> 1) + ((__mulhi(es, es) * 3) >> 15);
+    const long long s0 = (long long)((unsigned long long)vh * r0 + __umulhi(vl, r0));  // sqrt(v) 2^62
+    const long long s = min(s0 + (mul62(s0 - 1, t << 22) >> 20), (1ll << 62) - 1);
+    return a.m == 0 ? Sf{0ll, kZeroE} : Sf{s, ((ex + odd) >> 1) - 62};
 }
 // v / 3 and v / 9: v times 2^64 / 3 (or 9), words H and L, without the low words' product
 template <uint32_t H, uint32_t L>
 __device__ __forceinline__ long long mul_const(long long v) {
     const int h = (int)(v >> 32);
-    const long long t = (long long)((unsigned long long)(uint32_t)v * H) + (long long)h * (int)L;
-    return (long long)h * (int)H + (t >> 32);
+    const int mixed = (int)__umulhi((uint32_t)v, H) + __mulhi(h, (int)L);
+    return (((long long)__mulhi(h, (int)H) << 32) | (uint32_t)(h * (int)H)) + mixed;
 }
 __device__ __forceinline__ long long third64(long long v) { return mul_const<0x55555555u, 0x55555555u>(v); }
 __device__ __forceinline__ long long ninth64(long long v) { return mul_const<0x1c71c71cu, 0x71c71c72u>(v); }
