@@ -272,20 +272,25 @@ CaseDev make_case(const lbm_params& p, int64_t off, int64_t dense_off) {
     const double s = C.pd.sf[p.collision == LBM_MRT_RAW ? 1 : 3];
     C.p64.drho = p.rho_l - p.rho_g;
     C.p64.dnu = p.nu_l - p.nu_g;
-    C.p64.beta4 = 4.0 * C.pd.beta;
-    C.p64.lam3 = 4.0 / (3.0 * p.W);
-    C.p64.c2 = (long long)std::ldexp(0.5 * (1.0 - s), 62);
-    C.p64.c4 = (long long)std::ldexp(0.25 * (1.0 - s), 62);
-    auto sf = [](double x, long long& m, int32_t& e) {
+    // derived constants to 62 bits: a constant's rounding acts on every node of
+    // every step in the same direction
+    using Wide = long double;  // at least 64 bits on x86 and on Arm
+    C.p64.c2 = (long long)std::ldexp((1 - (Wide)s) / 2, 62);
+    C.p64.c4 = (long long)std::ldexp((1 - (Wide)s) / 4, 62);
+    auto sf = [](Wide x, long long& m, int16_t& e) {
         int ex = 0;
         m = (long long)std::ldexp(std::frexp(x, &ex), 62);  // 2^61 <= |m| < 2^62
-        e = x == 0.0 ? kZeroE : ex - 62;
+        e = (int16_t)(x == 0 ? kZeroE / 8 : ex - 62);  // (a double's exponents: within +-1200)
     };
-    sf(-C.pd.kappa / 72.0, C.p64.mkappa_m, C.p64.mkappa_e);
-    sf(0.3 / 72.0 * C.p64.drho, C.p64.drho3_m, C.p64.drho3_e);
-    sf((1.0 - 0.5 * s) / 3.0, C.p64.h3_m, C.p64.h3_e);
-    sf((1.0 + 0.5 * s) / 3.0, C.p64.sh3_m, C.p64.sh3_e);
-    sf(72.0 * p.n_eps, C.p64.neps72_m, C.p64.neps72_e);
+    sf(-(Wide)p.sigma * p.W / 48, C.p64.mkappa_m, C.p64.mkappa_e);  // kappa = 3 sigma W / 2
+    sf(((Wide)p.rho_l - p.rho_g) / 240, C.p64.drho3_m, C.p64.drho3_e);
+    sf((1 - (Wide)s / 2) / 3, C.p64.h3_m, C.p64.h3_e);
+    sf((1 + (Wide)s / 2) / 3, C.p64.sh3_m, C.p64.sh3_e);
+    sf(72 * (Wide)p.n_eps, C.p64.neps72_m, C.p64.neps72_e);
+    sf(48 * (Wide)p.sigma / p.W, C.p64.beta4_m, C.p64.beta4_e);  // beta = 12 sigma / W
+    sf(4 / (3 * (Wide)p.W), C.p64.lam3_m, C.p64.lam3_e);
+    sf(C.pd.mob, C.p64.mob_m, C.p64.mob_e);
+    sf(C.pd.grav_z, C.p64.grav_m, C.p64.grav_e);
     return C;
 }
 
@@ -518,7 +523,7 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
         for (const CaseDev& C : h->cases) h->D.ncols = std::max(h->D.ncols, C.pitch);
         void* cols = nullptr;
         A(&cols, col_tab64_size(h->D.ncols));
-        if (rc == LBM_OK && launch_col_tab64((double*)cols, h->D.ncols, h->D.rate_mode, h->stream) != cudaSuccess)
+        if (rc == LBM_OK && launch_col_tab64((double*)cols, h->D.ncols, h->stream) != cudaSuccess)
             rc = LBM_ERR_CUDA;
         h->D.cols = (const double*)cols;
     }

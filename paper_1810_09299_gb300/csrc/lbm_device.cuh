@@ -60,13 +60,14 @@ static_assert(offsetof(CaseReal<float>, nu_g) == 12 && offsetof(CaseReal<float>,
 // host instead of per node on the FP64 pipe.  s: the phase-field rate of the
 // momenta (compile-time rate patterns).
 struct Case64 {
-    double drho, dnu, beta4;  // rho_l - rho_g, nu_l - nu_g, 4 beta (Eq. 4)
-    double lam3;              // 4 / (3 W): r lambda / 3 = lam3 r phi (1 - phi) (Eq. 2)
-    long long c2, c4;         // (1 - s) / 2 and (1 - s) / 4 in units of 2^-62
+    double drho, dnu;  // rho_l - rho_g, nu_l - nu_g
+    long long c2, c4;  // (1 - s) / 2 and (1 - s) / 4 in units of 2^-62
     // as m 2^e with |m| < 2^62 (Sf of lbm_fix64.cuh)
     long long mkappa_m, drho3_m, h3_m, sh3_m, neps72_m;  // -kappa / 72, 0.3 (rho_l - rho_g) / 72,
-    int32_t mkappa_e, drho3_e, h3_e, sh3_e, neps72_e;    // (1 - s/2) / 3, (1 + s/2) / 3, 72 n_eps
-    int32_t pad;
+    long long beta4_m, lam3_m, mob_m, grav_m;            // (1 - s/2) / 3, (1 + s/2) / 3, 72 n_eps,
+    int16_t mkappa_e, drho3_e, h3_e, sh3_e, neps72_e;    // 4 beta (Eq. 4), 4 / (3 W) (r lambda / 3 =
+    int16_t beta4_e, lam3_e, mob_e, grav_e;              // lam3 r phi (1 - phi), Eq. 2), M, G_z
+    int16_t pad[3];
 };
 
 // Case c owns the handle's nodes [off, off + plane): node (k, j) is node

@@ -4,22 +4,34 @@
 // What bounds it: the FP64 pipe issues 1.6 operations per SM and cycle on this
 // chip, the integer pipes about 100 instructions.  The general form of
 // lbm_device.cuh takes 383 FP64 operations per node and is bound by that pipe.
-// Here the sums of populations and of the phi stencil, both collisions and both
-// inverse transforms run in 64-bit integers (lbm_fix64.cuh) beside about 60 FP64
-// operations: what depends on phi alone, the reciprocals and the roots, and the
-// conversion of the nine g.  32 batched cases (1.89 M nodes), us a step:
+// Here the sums of populations and of the phi stencil, both collisions, both
+// inverse transforms, reciprocals and roots run in 64-bit integers
+// (lbm_fix64.cuh) beside about 10 FP64 operations (what depends on phi alone) and
+// 20 conversions.  32 batched cases (1.89 M nodes), us a step:
 //   general form, 383 operations per node                          1342
 //   the algebra below, 280                                         1005
 //   sums of populations and of the stencil in integers, 202         724
 //   collisions and inverse transforms in integers, 83               516
 //   no IEEE fallbacks, cheaper conversions and normalisations, 55   408
 //   shared alignments, the nine g converted on the FP64 pipe, 61    383
-// (all eighteen converted there: 399, none: 397).  Now the ALU is 58 % and the
-// FP64 pipe 48 % busy (ncu).  More warps do not help: 3 CTAs of 80 registers
-// (460 bytes of spill) 387 us; with 4-row tiles 4, 5, 6 CTAs 446, 442, 441.
-// The error of one step against 80-bit arithmetic is below that of the general
-// form: 7.8e-17 against 1.25e-16 (f), 7.4e-16 against 2.1e-15 (g), 1.0e-16
-// against 2.5e-16 (chi) of their 2-norms on a 64 x 128 oscillating drop.
+//   column constants from a table in device memory, 57              376
+//   high-word multiplications; reciprocals and roots in integers, 29  331
+//   every result converted on the FP64 pipe, 43                     313
+//   3 CTAs of 80 registers per SM                                   302
+//   dropped bits given back on average, constants to 62 bits        309
+// (Conversions in integers had been the better ones while the FP64 pipe was
+// busier: 399 against 383 with all of them there, 61 operations.)  At 313 us the
+// ALU is 58 % and the FP64 pipe 42 % busy (ncu); timing-only copies without the
+// mixed products of the multiplications, without the ring and without the
+// sums' conversions ran 13, 6 and 6 % faster.
+// The last line is for accuracy: integers that only drop bits err in one
+// direction, which adds up over steps.  Error against 80-bit arithmetic, 2-norm,
+// general form and here:
+//                                        f                  g                  chi
+//   drop 64 x 128, 1 step         1.25e-16 0.70e-16  2.1e-15 0.72e-15  2.5e-16 0.94e-16
+//                   10 steps       5.8e-16  4.9e-16  1.6e-14  1.7e-15  1.9e-15  4.9e-16
+//   bubble 96 x 300, 1 step       1.26e-16 0.72e-16  2.7e-16  1.1e-16  1.6e-16 0.88e-16
+//                   10 steps       6.9e-16  5.0e-16  1.5e-15  1.0e-15  9.8e-16  5.8e-16
 // The rate pattern fixes:
 //   * the phase-field collision acts on four differences of populations, not
 //     on nine moments: with t = s chi + (1 - s/2) R and T = r phi,
@@ -29,9 +41,6 @@
 //   * a unit rate on the momenta gives m+ = J + F (the definition of u,
 //     Eq. 32, in r rho u + F / 2), so Eq. 36's r rho u is never formed there;
 //   * the interface normal enters as one factor of grad phi (Eq. 2, Eq. 38).
-// Reciprocals and square roots start from the hardware's FP64 approximations
-// (MUFU, 15.7 per SM and cycle) and take one third-order step, 3 and 5
-// operations instead of the 4.5 and 7.6 of the rounded library forms.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -157,24 +166,26 @@ __device__ __forceinline__ void pre64(const double* fd, const double* gd, Pre64&
 
 // What the update takes from a node's column, r = j + 1/2.
 struct Col64 {
-    double r, inv_r, i4, i2;            // r, 1/r, -2/(15 r) (raw: -4/(15 r)), -2/r
-    Sf sr, s_inv_r, s_i6, r03, r3, r72;  // r, 1/r, 0.6/r, r/0.3, 3 r, r/72
+    double r, inv_r;                          // r, 1/r
+    Sf sr, s_inv_r, s_i6, s_i4, r03, r3, r72;  // r, 1/r, 0.6/r, -2/(15 r), r/0.3, 3 r, r/72
 };
-template <int RM>
-__device__ __forceinline__ Col64 col64(int j, double inv_r) {
+__device__ __forceinline__ Col64 col64(int j) {
     const double r = (double)j + 0.5;
-    return Col64{r, inv_r, (RM == kRatesPaperRaw ? -4.0 / 15.0 : -2.0 / 15.0) * inv_r, -2.0 * inv_r, sf_of(r),
-                 sf_of(inv_r), sf_of(0.6 * inv_r), sf_of((1.0 / 0.3) * r), sf_of(3.0 * r), sf_of((1.0 / 72.0) * r)};
+    bool bad = false;
+    const Sf s = sf_of(r), i = rcp(s, bad);
+    return Col64{r, rcp_(r), s, i, norm(i * Sf{0x2666666666666666ll, -62}), neg(norm(i * Sf{0x2222222222222222ll, -64})),
+                 norm(s * Sf{0x3555555555555555ll, -60}), sf_of(3.0 * r), norm(s * Sf{0x38e38e38e38e38e4ll, -68})};
 }
+constexpr int kColSf = 7;
 // The columns 0 .. n - 1 of a handle in device memory, filled once when it is
 // created: with them formed per tile in shared memory the window waited for a
 // chain of FP64 operations behind a barrier of its own.
 struct ColTab64 {
-    const double* d;  // [4][n] doubles, then Sf [6][n]
+    const double* d;  // [2][n] doubles, then Sf [kColSf][n]
     int n;
     __device__ __forceinline__ double inv_r(int j) const { return __ldg(d + n + j); }
     __device__ __forceinline__ const longlong2* sf(int i) const {
-        return reinterpret_cast<const longlong2*>(d + 4 * n) + (int64_t)i * n;
+        return reinterpret_cast<const longlong2*>(d + 2 * n) + (int64_t)i * n;
     }
     __device__ __forceinline__ struct ColRef64 at(int j) const;
 };
@@ -194,28 +205,17 @@ struct ColRef64 {
     }
     __device__ __forceinline__ double r() const { return dv(0); }
     __device__ __forceinline__ double inv_r() const { return dv(1); }
-    __device__ __forceinline__ double i4() const { return dv(2); }
-    __device__ __forceinline__ double i2() const { return dv(3); }
     __device__ __forceinline__ Sf sr() const { return sv(0); }
     __device__ __forceinline__ Sf s_inv_r() const { return sv(1); }
     __device__ __forceinline__ Sf s_i6() const { return sv(2); }
-    __device__ __forceinline__ Sf r03() const { return sv(3); }
-    __device__ __forceinline__ Sf r3() const { return sv(4); }
-    __device__ __forceinline__ Sf r72() const { return sv(5); }
+    __device__ __forceinline__ Sf s_i4() const { return sv(3); }
+    __device__ __forceinline__ Sf r03() const { return sv(4); }
+    __device__ __forceinline__ Sf r3() const { return sv(5); }
+    __device__ __forceinline__ Sf r72() const { return sv(6); }
 };
 __device__ __forceinline__ ColRef64 ColTab64::at(int j) const { return ColRef64{*this, j}; }
 // 16 bytes per column and Sf, 8 per double
-constexpr size_t col_tab64_bytes(int n) { return (size_t)n * (4 * 8 + 6 * 16); }
-template <int RM>
-__global__ void col_tab64_kernel(double* d, int n) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const Col64 c = col64<RM>(j, rcp_((double)j + 0.5));
-    d[j] = c.r, d[n + j] = c.inv_r, d[2 * n + j] = c.i4, d[3 * n + j] = c.i2;
-    longlong2* s = reinterpret_cast<longlong2*>(d + 4 * n);
-    const Sf v[6] = {c.sr, c.s_inv_r, c.s_i6, c.r03, c.r3, c.r72};
-    for (int i = 0; i < 6; ++i) s[(int64_t)i * n + j] = longlong2{v[i].m, (long long)v[i].e};
-}
+constexpr size_t col_tab64_bytes(int n) { return (size_t)n * (2 * 8 + kColSf * 16); }
 
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
 // a's integer in units of 2^e, e >= a.e
@@ -249,13 +249,14 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
     const double nu = fma(phi, H.dnu, P.nu_g);
     const double tau = fma(3.0, nu, 0.5);
     const double rv = fma(nu, K.inv_r(), K.r());
-    const Sf rho = sf_of(rho_d), s = rcp(sf_of(tau), m.bad), D = rcp(sf_of(rho_d * rv), m.bad);
-    const Sf irr = K.s_inv_r() * (D * sf_of(rv));
+    const Sf rho = sf_of(rho_d), st = sf_of(tau), s = rcp(st, m.bad), srv = sf_of(rv), D = rcp(rho * srv, m.bad);
+    const Sf irr = K.s_inv_r() * (D * srv), sphi = sf_of(phi);
     // Eq. 4: mu~ = mu - k d_r phi / r; Eq. 30's F_z = r (F_s + G)_z
-    const Sf mut = norm29(sf_of((H.beta4 * phi) * fma(phi, phi - 1.5, 0.5)) + Sf{H.mkappa_m, H.mkappa_e} * norm29(gr * K.s_inv_r() + lap));
+    const Sf mut = norm29((Sf{H.beta4_m, H.beta4_e} * sphi) * sf_of(fma(phi, phi - 1.5, 0.5)) +
+                          Sf{H.mkappa_m, H.mkappa_e} * norm29(gr * K.s_inv_r() + lap));
     const Sf rm = K.r72() * mut;
     Sf Fz = rm * gz;
-    if (abs_hi(P.grav_z) != 0) Fz = Fz + sf_of(K.r() * ((rho_d - P.rho_l) * P.grav_z));
+    if (abs_hi(P.grav_z) != 0) Fz = Fz + K.sr() * (sf_of(rho_d - P.rho_l) * Sf{H.grav_m, H.grav_e});
     const Sf rFsr = rm * gr;
     const Sf d3{H.drho3_m, H.drho3_e};
     const Sf Z3 = d3 * gz, R3 = d3 * gr;  // 0.3 grad rho
@@ -263,9 +264,9 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
     const Sf uz = norm29(Sf{JFz.a + (JFz.b >> 1), JFz.e}) * irr;  // Eq. 32 (z)
     const Sf rz = rho * uz;
     // Eq. 33 with s_p = tau_g / 2 (raw: 3 tau_g / 2 - 1)
-    const Sf A2 = sf_of(0.4 * rho_d);
+    const Sf A2 = rho * Sf{0x3333333333333333ll, -63};  // 0.4 rho
     const Sf A0 = uz * norm29(Z3 - A2 * uz) + K.s_i6() * Q.S0;
-    const Sf A1 = norm29(sf_of(((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * K.i4()) + R3);
+    const Sf A1 = norm29(sf_of((kRaw ? fma(1.5, tau, -1.0) : tau) * rho_d) * scale2(K.s_i4(), kRaw ? 1 : 0) + R3);
     // numbers that are not finite do not exist in integers: seen here, put out as NaN
     int top = max(abs_hi(rho_d), abs_hi(nu));
     Sf ur, p, ps;
@@ -301,7 +302,6 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
                                          const Pre64& Q, double chz_prev, double chr_prev, double p_prev, double* fp,
                                          double* gp, double& chz_out, double& chr_out, double& p_out) {
     constexpr bool kRaw = RM == kRatesPaperRaw;
-    const CaseReal<double>& P = C.pd;
     const Case64& H = C.p64;
     const Macro64 m = macros64<LD, RM>(C, W, a, b, phi, K, Q, p_prev);
     bool bad = m.bad;
@@ -309,20 +309,20 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     const Sf gz = m.gz, gr = m.gr, Z3 = m.Z3, R3 = m.R3, rho = m.rho, s = m.s, uz = m.uz, rz = m.rz, ur = m.ur, p = m.p;
     const Two JFz = m.JFz;
     const Sf rr = rho * ur;
-    const Sf Fr = (m.rFsr + m.ps) + sf_of(m.nu * K.i2()) * rr;  // Eq. 30 (r)
+    const Sf Fr = (m.rFsr + m.ps) - scale2(sf_of(m.nu) * K.s_inv_r() * rr, 1);  // Eq. 30 (r)
     p_out = double_of(p);
     // phase field (Eq. 19-23, 38): chi, then t / 3 of both directions
     const Sf T = norm_any(Q.t, Q.Ef - 1075 - kPopK);
-    const Sf chz = T * uz, chr = T * ur + sf_of(P.mob * phi);
+    const Sf chz = T * uz, chr = T * ur + Sf{H.mob_m, H.mob_e} * sf_of(phi);
     chz_out = double_of(chz);
     chr_out = double_of(chr);
     {
         // r lambda / (3 (|grad phi| + n_eps)): the normal's factor of grad phi (72 in both)
-        const double lam = H.lam3 * (K.r() * fma(-phi, phi, phi));
-        const Sf L = sf_of(lam) * rcp(root(gz * gz + gr * gr) + Sf{H.neps72_m, H.neps72_e}, bad);
+        const Sf lam = Sf{H.lam3_m, H.lam3_e} * K.sr() * sf_of_or_zero(fma(-phi, phi, phi));
+        const Sf L = lam * rcp(root(gz * gz + gr * gr) + Sf{H.neps72_m, H.neps72_e}, bad);
         const Sf h3{H.h3_m, H.h3_e}, sh3{H.sh3_m, H.sh3_e};
-        const Sf tz = h3 * norm29(L * gz - sf_of(chz_prev)) + sh3 * chz;
-        const Sf tr = h3 * norm29(L * gr - sf_of(chr_prev)) + sh3 * norm29(chr);
+        const Sf tz = h3 * norm29(L * gz - sf_of_or_zero(chz_prev)) + sh3 * chz;
+        const Sf tr = h3 * norm29(L * gr - sf_of_or_zero(chr_prev)) + sh3 * norm29(chr);
         // the sums of the inverse transform in units of the largest part, 2^E
         // (the block's values take up to 63 bits)
         const int eb = Q.Ef - 1075 - kPopK;
@@ -330,18 +330,19 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         bad = bad || E > 890;
         const long long e = ninth_double(shr64(Q.t, sb));
         const long long tz0 = in_units(tz, E), tr0 = in_units(tr, E);
-        const long long jz = mul62(shr64(Q.fz, sb), H.c2) + tz0, jr = mul62(shr64(Q.fr, sb), H.c2) + tr0;
-        const long long qz = mul62(shr64(Q.fe, sb), H.c4) + (tz0 >> 2), qr = mul62(shr64(Q.fo, sb), H.c4) + (tr0 >> 2);
-        const long long d = e >> 2, qp = qz + qr, qm = qz - qr;
-        fp[0] = double_in(e, E + 2);
-        fp[1] = double_in(e + jz, E);
-        fp[3] = double_in(e - jz, E);
-        fp[2] = double_in(e + jr, E);
-        fp[4] = double_in(e - jr, E);
-        fp[5] = double_in(d + qp, E);
-        fp[7] = double_in(d - qp, E);
-        fp[8] = double_in(d + qm, E);
-        fp[6] = double_in(d - qm, E);
+        const auto part = [&](long long v, long long c) { return v == 0 ? 0ll : mul62(shr64(v, sb), c); };
+        const long long jz = part(Q.fz, H.c2) + tz0, jr = part(Q.fr, H.c2) + tr0;
+        const long long qz = part(Q.fe, H.c4) + (tz0 >> 2), qr = part(Q.fo, H.c4) + (tr0 >> 2);
+        const long long d = (e + 2) >> 2, qp = qz + qr, qm = qz - qr;
+        fp[0] = double_cvt(e, E + 2);
+        fp[1] = double_cvt(e + jz, E);
+        fp[3] = double_cvt(e - jz, E);
+        fp[2] = double_cvt(e + jr, E);
+        fp[4] = double_cvt(e - jr, E);
+        fp[5] = double_cvt(d + qp, E);
+        fp[7] = double_cvt(d - qp, E);
+        fp[8] = double_cvt(d + qm, E);
+        fp[6] = double_cvt(d - qm, E);
     }
     // hydrodynamics (Eq. 24, 36-37)
     const Sf az = K.r03() * Z3, br = norm29(K.r03() * R3 + rho);      // grad (r rho)
@@ -371,13 +372,13 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         // 12 g in units of 2^E
         const long long ax = K3 * 3 - K8 * 6, p7 = M7 * 3;
         gp[0] = double_cvt(M0 - K3 + K8, E);
-        gp[1] = double_cvt(third64(ax + p7 + JZ * 4), E - 2);
+        gp[1] = double_cvt(third64<2>(ax + p7 + JZ * 4), E - 2);
         gp[3] = double_cvt(third64(ax + p7 - JZ * 4), E - 2);
         gp[2] = double_cvt(third64(ax - p7 + JR * 4), E - 2);
-        gp[4] = double_cvt(third64(ax - p7 - JR * 4), E - 2);
+        gp[4] = double_cvt(third64<0>(ax - p7 - JR * 4), E - 2);
         const long long dp = (K8 + M8) * 3, dm = (K8 - M8) * 3;
-        gp[5] = double_cvt(third64(dp + JZ + JR), E - 2);
-        gp[7] = double_cvt(third64(dp - JZ - JR), E - 2);
+        gp[5] = double_cvt(third64<2>(dp + JZ + JR), E - 2);
+        gp[7] = double_cvt(third64<2>(dp - JZ - JR), E - 2);
         gp[8] = double_cvt(third64(dm + JZ - JR), E - 2);
         gp[6] = double_cvt(third64(dm - JZ + JR), E - 2);
     } else {
@@ -385,7 +386,9 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         const Sf m2 = neg((K.r3() * norm29(Sf{((pE.a + pE.b) >> 1) + (pE.a >> 2), pE.e + 1})) + (m0 + rr));
         // 36 g = 4 m0 - m1 - 2 m2 +- 9 m7 +- 12 j (axes), 4 m0 + 2 m1 + m2 +- 9 m8
         // +- 3 j (diagonals), 4 (m0 - m1 + m2) (rest), in units of 2^E: the
-        // coefficients add up to 28 at most
+        // coefficients add up to 28 at most.  in_units leaves half a unit out on
+        // average; with its coefficient that is -11 to 10 units of 36 g, so the
+        // quotients take 0 to 2 units back.
         const int E = max(-994, max(max(max(m0.e, m1.e), max(m2.e, jz.e)), max(max(m7.e, m8.e), jr.e))) + 4;
         bad = bad || E > 890;
         const long long M0 = in_units(m0, E) * 4, M1 = in_units(m1, E), M2 = in_units(m2, E);
@@ -393,12 +396,12 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         const long long JZ = in_units(jz, E) * 3, JR = in_units(jr, E) * 3;
         const long long ax = M0 - M1 - M2 * 2, dg = M0 + M1 * 2 + M2;
         gp[0] = double_cvt(ninth64(M0 - (M1 - M2) * 4), E - 2);
-        gp[1] = double_cvt(ninth64(ax + M7 + JZ * 4), E - 2);
+        gp[1] = double_cvt(ninth64<2>(ax + M7 + JZ * 4), E - 2);
         gp[3] = double_cvt(ninth64(ax + M7 - JZ * 4), E - 2);
         gp[2] = double_cvt(ninth64(ax - M7 + JR * 4), E - 2);
-        gp[4] = double_cvt(ninth64(ax - M7 - JR * 4), E - 2);
-        gp[5] = double_cvt(ninth64(dg + M8 + JZ + JR), E - 2);
-        gp[7] = double_cvt(ninth64(dg + M8 - JZ - JR), E - 2);
+        gp[4] = double_cvt(ninth64<0>(ax - M7 - JR * 4), E - 2);
+        gp[5] = double_cvt(ninth64<2>(dg + M8 + JZ + JR), E - 2);
+        gp[7] = double_cvt(ninth64<2>(dg + M8 - JZ - JR), E - 2);
         gp[8] = double_cvt(ninth64(dg - M8 + JZ - JR), E - 2);
         gp[6] = double_cvt(ninth64(dg - M8 - JZ + JR), E - 2);
     }

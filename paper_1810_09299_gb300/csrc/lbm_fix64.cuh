@@ -12,9 +12,10 @@ namespace axilbm {
 // K extra bits below the last place of the largest value), added exactly, and
 // the result is rounded once to a double.  An addition costs two integer
 // instructions of the ~100 per SM and cycle instead of one of the 1.6 FP64
-// operations, a conversion into the block 0.21 and out of it 0.3 cycles per node
-// and SM against 0.62 for an FP64 operation, and both run beside the FP64 pipe.  The rounding is at most that of the FP64 sums it replaces: the bits a
-// smaller value loses lie K bits below the largest one's last place.
+// operations, a conversion into the block 0.21 cycles per node and SM against
+// 0.62 for an FP64 operation, and they run beside the FP64 pipe.  The rounding is
+// at most that of the FP64 sums it replaces: the bits a smaller value loses lie K
+// bits below the largest one's last place.
 // E is at least kMinE (values below 2^-959 lose their low bits, as subnormal
 // numbers do); from kBadE on (2^1007, infinities, NaN) the results are NaN.
 constexpr int kMinE = 64, kBadE = 2030;
@@ -42,16 +43,19 @@ __device__ __forceinline__ long long fix64(double x, int E) {
     const long long v = (long long)shr64u(m, E - exp64(x)), sg = (long long)(hi >> 31);
     return (v ^ sg) - sg;
 }
-// v 2^(E - 1075 - K) as a double (rounded to nearest, ties away from zero).
+// m 2^e as a double, rounded to nearest, for |m| < 2^63 and a result within the
+// normal numbers (or m = 0): -1000 <= e <= 900 does.  The FP64 pipe's conversion takes
+// 0.53 cycles per node and SM, a normalisation and packing in integers 0.3, but
+// the integer pipes have more to do.
+__device__ __forceinline__ double double_cvt(long long m, int e) {
+    const double d = __ll2double_rn(m);
+    const int hi = __double2hiint(d);
+    return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(d));
+}
+// v 2^(E - 1075 - K) as a double, kMinE <= E < kBadE.
 template <int K>
 __device__ __forceinline__ double unfix64(long long v, int E) {
-    const long long sg = v >> 63;
-    unsigned long long a = (unsigned long long)((v ^ sg) - sg);
-    const int n = __clzll((long long)a);
-    a <<= n & 63;
-    unsigned long long b = (a >> 11) + ((a >> 10) & 1ull) + ((unsigned long long)(uint32_t)(E + 10 - K - n) << 52);
-    b |= (unsigned long long)sg << 63;
-    return v == 0 ? 0.0 : __longlong_as_double((long long)b);
+    return double_cvt(v, E - 1075 - K);
 }
 template <int N>
 __device__ __forceinline__ int block_exp(const double* x) {
@@ -76,10 +80,9 @@ __device__ __forceinline__ double sum64(const double* f) {
 // ---------------------------------------------------------------- numbers of 62 bits
 // x = m 2^e with |m| < 2^62 in integer registers, for products and sums that
 // would wait for the FP64 pipe.  Cycles per node and SM (measured): a product
-// 0.22 (three wide multiply-adds at 16 per SM and cycle), a sum 0.09, norm29
-// 0.08, norm 0.19, sf_of 0.15, against 0.62 for an FP64 operation of either
-// kind.  A product keeps all but 1 bit of normalised operands (|m| >= 2^61) and
-// is exact to about 2^-59 of itself; a sum is exact to the last place of its
+// 0.15, a sum 0.09, norm29 0.08, norm 0.19, sf_of 0.15, against 0.62 for an FP64
+// operation of either kind.  A product keeps all but 1 bit of normalised operands (|m| >= 2^61) and
+// is exact to about 2^-58 of itself; a sum is exact to the last place of its
 // larger operand.  A factor that may have cancelled (a sum) is normalised
 // first; zero carries a large negative exponent, so that it never shifts the
 // other operand of a sum.
@@ -89,13 +92,15 @@ struct Sf {
 };
 constexpr int kZeroE = -(1 << 17);
 
-// a b 2^-62, |a|, |b| < 2^62, short by at most 12 units (the low words' product
-// and the bits below the high words of the mixed ones are left out).  High-word
-// multiplications (30.6 per SM and cycle) rather than signed wide ones (12).
+// a b 2^-62, |a|, |b| < 2^62, within 8 units: the low words' product and the bits
+// below the high words of the mixed ones are left out, about 5 units on average,
+// and 4 are added back (to a zero, too: one that must stay zero is the caller's, or has
+// the exponent kZeroE).  High-word multiplications (30.6 per SM and cycle) rather
+// than signed wide ones (12).
 __device__ __forceinline__ long long mul62(long long a, long long b) {
     const int ah = (int)(a >> 32) * 2, bh = (int)(b >> 32) * 2;
     const int al = (int)((uint32_t)a >> 1), bl = (int)((uint32_t)b >> 1);
-    const int mixed = __mulhi(ah, bl) + __mulhi(bh, al);
+    const int mixed = __mulhi(ah, bl) + __mulhi(bh, al) + 1;
     const long long high = ((long long)__mulhi(ah, bh) << 32) | (uint32_t)(ah * bh);
     return high + (long long)mixed * 4;
 }
@@ -145,27 +150,14 @@ __device__ __forceinline__ Sf sf_of(double x) {
     const long long sg = (long long)(hi >> 31);
     return Sf{(v ^ sg) - sg, exp64(x) - 1084};
 }
-// m 2^e as a double, rounded to nearest, for |m| < 2^63 and -1000 <= e <= 900.
-__device__ __forceinline__ double double_in(long long m, int e) {
-    const long long sg = m >> 63;
-    const unsigned long long x = (unsigned long long)((m ^ sg) - sg);
-    const int n = __clzll((long long)x);  // 1 .. 64
-    unsigned long long y;                 // the leading bit at 62, ten bits below the last place
-    asm("shl.b64 %0, %1, %2;" : "=l"(y) : "l"(x), "r"(n - 1));
-    y = (y + 0x200ull) >> 10;
-    const uint32_t hi = (uint32_t)(y >> 32) + ((uint32_t)(e - n + 1085) << 20);
-    return __hiloint2double((int)((n == 64 ? 0u : hi) | ((uint32_t)sg & 0x80000000u)), (int)(uint32_t)y);
+// The same with zero as zero: a number near -2^-1022 would become -1 in any larger unit.
+__device__ __forceinline__ Sf sf_of_or_zero(double x) {
+    const Sf a = sf_of(x);
+    return Sf{exp64(x) == 0 ? 0ll : a.m, a.e};
 }
-// The same by the FP64 pipe's conversion (0.53 cycles per node and SM, against
-// 0.3 on the integer pipes, which have more to do).
-__device__ __forceinline__ double double_cvt(long long m, int e) {
-    const double d = __ll2double_rn(m);
-    const int hi = __double2hiint(d);
-    return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(d));
-}
-// The same for any e: below the normal numbers zero, above them NaN.
+// m 2^e as a double for any e: below the normal numbers zero, above them NaN.
 __device__ __forceinline__ double double_of(Sf a) {
-    const double d = double_in(a.m, a.e);
+    const double d = double_cvt(a.m, a.e);
     return a.e < -1000 ? 0.0 : (a.e > 900 ? nan64() : d);
 }
 // The leading 64 bits of |a|, a != 0: bit 63 set.
@@ -220,20 +212,23 @@ __device__ __forceinline__ Sf root(Sf a) {
     const long long s = min(s0 + (mul62(s0 - 1, t << 22) >> 20), (1ll << 62) - 1);
     return a.m == 0 ? Sf{0ll, kZeroE} : Sf{s, ((ex + odd) >> 1) - 62};
 }
-// v / 3 and v / 9: v times 2^64 / 3 (or 9), words H and L, without the low words' product
-template <uint32_t H, uint32_t L>
+// v / 3 and v / 9, within 1.5 units: v times 2^64 / 3 (or 9), words H and L, without the
+// low words' product and plus Up for what the high words leave out (0 stays 0)
+template <uint32_t H, uint32_t L, uint32_t Up>
 __device__ __forceinline__ long long mul_const(long long v) {
     const int h = (int)(v >> 32);
-    const int mixed = (int)__umulhi((uint32_t)v, H) + __mulhi(h, (int)L);
+    const int mixed = (int)__umulhi((uint32_t)v, H) + __mulhi(h, (int)L) + (int)min((uint32_t)v, Up);
     return (((long long)__mulhi(h, (int)H) << 32) | (uint32_t)(h * (int)H)) + mixed;
 }
-__device__ __forceinline__ long long third64(long long v) { return mul_const<0x55555555u, 0x55555555u>(v); }
-__device__ __forceinline__ long long ninth64(long long v) { return mul_const<0x1c71c71cu, 0x71c71c72u>(v); }
+template <uint32_t Up = 1>
+__device__ __forceinline__ long long third64(long long v) { return mul_const<0x55555555u, 0x55555555u, Up>(v); }
+template <uint32_t Up = 1>
+__device__ __forceinline__ long long ninth64(long long v) { return mul_const<0x1c71c71cu, 0x71c71c72u, Up>(v); }
 // v times the double nearest 1/9 (5.6e-17 below it), for the weights of the phase
 // field: the conserved sum of f takes this factor every step.  With 1/9 itself it
 // drifts by 4e-15 instead of 1.1e-13 over 2000 steps, but the oracle and the
 // general kernels hold the weights as doubles, and on the 64 x 128 static drop runs
 // with and without that drift part by 2e-12 (phi) and 1e-11 (p) in that time.
-__device__ __forceinline__ long long ninth_double(long long v) { return mul_const<0x1c71c71cu, 0x71c71c00u>(v); }
+__device__ __forceinline__ long long ninth_double(long long v) { return mul_const<0x1c71c71cu, 0x71c71c00u, 2>(v); }
 
 }  // namespace axilbm

@@ -53,7 +53,7 @@ struct DeviceState {
 // The column table of an FP64 handle (rate mode D.rate_mode): its size, and
 // the kernel that fills it.
 size_t col_tab64_size(int ncols);
-cudaError_t launch_col_tab64(double* cols, int ncols, int rate_mode, cudaStream_t st);
+cudaError_t launch_col_tab64(double* cols, int ncols, cudaStream_t st);
 
 AXILBM_DECLARE(f64)
 AXILBM_DECLARE(f32)

@@ -132,8 +132,11 @@ __device__ __forceinline__ void ring_cell(int q, int& a, int& b) {
 #ifndef AXILBM_GRID16_CTAS
 #define AXILBM_GRID16_CTAS 4
 #endif
-// FP64 with a compile-time rate pattern: 16 warps per SM at 128 registers (the
-// figures in lbm_f64.cuh).
+// FP64 with a compile-time rate pattern: 16 warps per SM at 128 registers, or with
+// 6 tiles of 8 rows per SM and more kF64Full CTAs (24 warps, 80 registers, 176 bytes
+// of spill): 32 cases (7386 tiles) 313 -> 302 us, 256 x 1024 (1024) 47.7 -> 46.5, but
+// 200 x 600 (525) 26.3 -> 27.2 and 128 x 256 (128) 9.1 -> 11.0.
+constexpr int kF64Full = 3;
 template <class Codec, int BZ, int RM>
 constexpr int step_min_blocks() {
     constexpr int bz8 = Codec::kGrid ? AXILBM_GRID16_CTAS
@@ -721,8 +724,8 @@ __device__ __forceinline__ void step_tile(const StateDev<Codec>& S, TileShared<C
 }
 
 // One time step for every node of every tile in `tiles`: one CTA per tile.
-template <class Codec, int BZ, int RM>
-__global__ void __launch_bounds__(kTR * BZ, (step_min_blocks<Codec, BZ, RM>()))
+template <class Codec, int BZ, int RM, int MINB = step_min_blocks<Codec, BZ, RM>()>
+__global__ void __launch_bounds__(kTR * BZ, MINB)
 step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles, StateDev<Codec> S,
             const CUtensorMap* __restrict__ maps, int map_set, int parity, int ntiles, int ahead) {
     __shared__ TileShared<Codec, BZ, RM> sh;
@@ -1724,6 +1727,13 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
     const CUtensorMap* maps = (const CUtensorMap*)D.tmaps;
     switch (variant) {
         case 0:
+            if constexpr (sizeof(typename Codec::Real) == 8 && RM != kRatesGeneral) {
+                if (ntiles >= 6 * sms) {
+                    launch_step_kernel(step_kernel<Codec, 8, RM, kF64Full>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0,
+                                       parity, ntiles, kPrefetchQuarters * sms * kF64Full / 4);
+                    break;
+                }
+            }
             launch_step_kernel(step_kernel<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 8, RM>() / 4);
             break;
         case 1:

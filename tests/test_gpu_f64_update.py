@@ -46,6 +46,42 @@ def test_edges_match_oracle(nr, nz, zper, lagged, raw):
                 assert np.array_equal(a, b), v
 
 
+@pytest.mark.parametrize("raw", [0, 1])
+@pytest.mark.parametrize("nz", [3632, 3640, 3645])
+def test_many_tiles(nz, raw):
+    """33 columns are two tiles per 8 rows: 908, 910 and 912 tiles, the last from six tiles
+    per SM on (152 SMs), where another kernel takes over; against 16-row tiles."""
+    case = W.oscillating_drop(nr=33, nz=nz, R0=10.0, ratio=10.0)
+    if raw:
+        case = W.with_raw_collision(case)
+    out = []
+    for v in (0, 2):
+        sim = lbm.Simulation(case)
+        sim.set_variant(v)
+        sim.init_case(0)
+        sim.step(3)
+        out.append(sim.state(0))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("raw", [0, 1])
+def test_zero_stays_zero(raw):
+    """Where phi is exactly zero and nothing moves, f stays exactly zero."""
+    case = W.static_drop(nr=64, nz=40, R=8.0, sigma=0.0)
+    if raw:
+        case = W.with_raw_collision(case)
+    phi = W.initial_phi(case)
+    phi[phi < 1e-3] = 0.0
+    ref = oracle.Oracle(case).init(phi).step(2)
+    sim = lbm.Simulation(case)
+    sim.init_phase(0, "host_array", phi=phi)
+    sim.step(2)
+    f, rf = sim.state(0)[0], ref.populations()[0]
+    assert (rf == 0).any()
+    assert not f[rf == 0].any()
+
+
 @pytest.mark.parametrize("scale", [1e-40, 1e-200, 1e-270])
 def test_very_small_populations(scale):
     """sigma = 0 and f scaled down: phi stays proportional to the scale (n ~ 0 there),
