@@ -305,7 +305,8 @@ int lbm_autotune(lbm_handle* h, int32_t reps, int32_t* chosen);
 /* Select a step-kernel launch variant explicitly (0 .. lbm_num_variants()-1).
  * Every variant computes bit-identical results; they differ in tile height
  * (rows along z of the 32-column tile), in nodes per thread and in staging:
- *   0, 1, 2  one node per thread, tiles of 8, 16, 4 rows;
+ *   0, 1, 2  one node per thread, tiles of 8, 16, 4 rows (0: 10 or 12 rows on
+ *            grids where these fill the SMs evenly and 8 rows do not);
  *   3, 4     one node per thread, tiles of 8, 16 rows staged in shared memory
  *            by TMA copies (persistent, pipelined; needs the tensor maps);
  *   5, 6     two nodes of a column per thread, tiles of 16 rows; 6 keeps the

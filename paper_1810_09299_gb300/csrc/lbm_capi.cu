@@ -93,8 +93,8 @@ struct lbm_sim {
     DeviceState D{};
     // tiles: one list per step variant over all cases, plus the 8-row tiling
     // of each case for the field kernel
-    TileDev* tiles_d[kNumVariants] = {};
-    int ntiles[kNumVariants] = {};
+    TileDev* tiles_d[kNumShapes] = {};
+    int ntiles[kNumShapes] = {};
     std::vector<TileDev*> ftiles_d;
     std::vector<int> nftiles;
     int64_t max_nodes = 0;  // largest nz * nr of a case
@@ -125,6 +125,7 @@ struct lbm_sim {
     std::vector<void*> allocations;
     int parity = 0;
     int variant = 0;
+    int row_shape = 0;  // what variant 0 runs: itself or a shape of taller tiles
     int sticky = LBM_OK;
     int64_t launches = 0;
     cudaGraphExec_t graph = nullptr;
@@ -158,6 +159,7 @@ cudaError_t dev_alloc(lbm_sim* h, void** p, size_t bytes) {
 }
 
 cudaError_t launch_step_any(lbm_sim* h, int parity, int variant, cudaStream_t st) {
+    if (variant == 0) variant = h->row_shape;
     const TileDev* t = h->tiles_d[variant];
     const int n = h->ntiles[variant];
     switch (h->precision) {
@@ -408,16 +410,51 @@ bool encode_tensor_maps(lbm_sim* h, std::vector<CUtensorMap>& maps) {
     return true;
 }
 
+int sm_count(const lbm_sim* h) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess && sms > 0) return sms;
+    cudaGetLastError();
+    return 0;
+}
+
+// The tile height of variant 0: 8 rows, or 10 (shape 8) or 12 (9) where these come
+// to one CTA per SM and 8 rows do not, since a small grid's step lasts as long as
+// the SM with the most warps.  us a step, 8 rows, 4 rows and 10 or 12 rows:
+//                       FP64               FP32             FP16             bfloat16
+//   101 x 333 (168, 10) 13.8  11.9 10.9    3.15 3.09 2.83   3.56 3.40 3.15   3.92 3.45 3.20
+//   150 x 300 (190, 10) 14.1  12.0 11.0    3.34 3.28 2.88   3.44 3.59 3.27   3.92 3.53 3.32
+//   128 x 448 (224, 12) 13.9  11.9 11.9    3.21 3.21 3.09   3.59 3.46 3.20   3.85 3.53 3.27
+//   150 x 400 (250, 10) 14.2  14.5 20.7    3.41 3.57 3.84   3.65 3.91 3.96   3.92 3.98 4.10
+//   200 x 400 (350, 10) 20.7  19.6 20.9    4.11 3.97 3.85   4.37 4.30 3.98   4.80 4.37 4.11
+// (in brackets the tiles of 8 rows on 152 SMs and the taller tiles' rows).  So
+// 10 rows also where two CTAs per SM hold them and not the 8-row ones, but in
+// FP64, whose 10-row CTAs have an SM's registers to themselves.  Two of those
+// columns' ranges apart (525 tiles: FP32 4.87, 4.77, 5.69) 8 rows are better.
+// Rates by array (kRatesGeneral) keep 8 rows: there the compiler contracts other
+// pairs of FP32 operations in a block of 10 or 12 warps, and the results' last bits
+// would depend on the grid.
+int row_shape(const lbm_sim* h) {
+    const int sms = sm_count(h);
+    auto tiles = [&](int tz) {
+        int64_t t = 0;
+        for (const CaseDev& C : h->cases) t += (int64_t)((C.nz + tz - 1) / tz) * (C.pitch / 32);
+        return t;
+    };
+    if (h->D.rate_mode == kRatesGeneral || tiles(8) <= sms) return 0;
+    if (tiles(10) <= sms) return 8;
+    if (tiles(12) <= sms) return 9;
+    if (h->precision != LBM_FP64 && tiles(8) > 2 * sms && tiles(10) <= 2 * sms) return 8;
+    return 0;
+}
+
 // The launch shape a handle starts with (lbm_set_variant, lbm_autotune and the
 // results know no difference).  us a step in the captured graph:
 //   4-row tiles (2) instead of 8-row tiles (0)
 //     where those leave half the SMs empty, FP64 and bfloat16 (a 64 x 128 drop, 32
 //     tiles of 8 rows: 11.0 -> 9.5 and 3.02 -> 2.77; FP32 2.45 and 2.39, FP16 2.90
-//     either way), and where some SMs would hold two of them and most one (101 x
-//     333, 168 tiles on 152 SMs: FP64 16.6 -> 13.4, FP32 3.35 -> 3.22, FP16 3.73 ->
-//     3.47, bfloat16 3.77 -> 3.47; 150 x 300, 190 tiles: 16.6 -> 13.7, 3.41 -> 3.35,
-//     3.59 -> 3.58, 3.98 -> 3.60).  128 tiles (128 x 256) and 250 (150 x 400) take 8
-//     rows: FP32 2.52 against 2.77 and 3.41 against 3.66.
+//     either way), and where some SMs would hold two of them, most one and taller
+//     tiles do not help (row_shape's figures).  128 tiles (128 x 256) and 250 (150 x
+//     400) take 8 rows: FP32 2.52 against 2.77 and 3.41 against 3.66.
 //   FP16, packed pairs of nodes (7) from 3/2 tiles of 16 rows per SM on: 64 x 180
 //     and 128 x 256 are slower there (3.40 against 3.02), 200 x 600 (266 tiles) 5.01 ->
 //     4.94, 256 x 1024 (512) 8.23 -> 7.70, 512 cases 757 -> 558;
@@ -425,11 +462,8 @@ bool encode_tensor_maps(lbm_sim* h, std::vector<CUtensorMap>& maps) {
 //     256 x 1024 (512 tiles) 8.27 against 8.81, 8 cases (1100) 15.8 -> 15.2, 512 cases
 //     726 -> 711.
 int default_variant(const lbm_sim* h) {
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) {
-        cudaGetLastError();
-        return 0;
-    }
+    const int sms = sm_count(h);
+    if (sms == 0 || h->row_shape != 0) return 0;
     const int t8 = h->ntiles[0];
     if (2 * t8 <= sms && (h->precision == LBM_FP64 || h->precision == LBM_MIX_BF16)) return 2;
     if (t8 > sms && 3 * t8 <= 4 * sms) return 2;
@@ -544,7 +578,9 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
                                         h->stream);
         if (e != cudaSuccess) rc = LBM_ERR_CUDA;
     }
-    for (int v = 0; v < kNumVariants && rc == LBM_OK; ++v) {
+    h->row_shape = row_shape(h);
+    for (int v = 0; v < kNumShapes && rc == LBM_OK; ++v) {
+        if (v >= kNumVariants && v != h->row_shape) continue;
         std::vector<TileDev> t = make_tiles(h->cases, kVariantTZ[v], -1);
         h->ntiles[v] = (int)t.size();
         rc = upload_tiles(h, t, &h->tiles_d[v], true);

@@ -70,7 +70,10 @@ constexpr int kNumVariants = 8;
 // kernel of their tile height in FP64; variant 7 updates the two nodes
 // together in packed FP32x2 lanes (FP16 storage; the other precisions run
 // variant 5's kernel there)
-constexpr int kVariantTZ[kNumVariants] = {8, 16, 4, 8, 16, 16, 16, 16};
+// Shapes 8 and 9 are variant 0 with taller tiles on grids of certain sizes (row_shape
+// in lbm_capi.cu); a handle has the list of at most one of them.
+constexpr int kNumShapes = kNumVariants + 2;
+constexpr int kVariantTZ[kNumShapes] = {8, 16, 4, 8, 16, 16, 16, 16, 10, 12};
 constexpr bool kVariantTMA[kNumVariants] = {false, false, false, true, true, false, false, false};
 // tensor maps per case and tile height: the case's blocks in buffer 0 and 1
 // with a box of the tile's rows plus two above and below (staging, [0], [1]),

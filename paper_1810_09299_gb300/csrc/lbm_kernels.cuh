@@ -143,8 +143,8 @@ constexpr int step_min_blocks() {
                         : (RM == kRatesPaperRaw && sizeof(typename Codec::PT) == 2)
                             ? 4
                             : (sizeof(typename Codec::PT) == 2 ? AXILBM_STEP16_CTAS : 5);
-    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ >= 16 ? 1 : (BZ == 4 ? 4 : 2)))
-           : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
+    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ > 8 ? 1 : (BZ == 4 ? 4 : 2)))
+           : BZ == 10 || BZ == 12 ? 2 : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
                 : (BZ >= 16 ? 1 : (BZ >= 8 ? AXILBM_GENERAL_CTAS : 2 * AXILBM_GENERAL_CTAS));
 }
 
@@ -1741,6 +1741,16 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
             break;
         case 2:
             launch_step_kernel(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
+            break;
+        case 8:  // (one wave: nothing to prefetch)
+            if constexpr (RM != kRatesGeneral)
+                launch_step_kernel(step_kernel<Codec, 10, RM>, ntiles, dim3(kTR, 10), st, cs, tiles, S,
+                                   (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
+            break;
+        case 9:
+            if constexpr (RM != kRatesGeneral)
+                launch_step_kernel(step_kernel<Codec, 12, RM>, ntiles, dim3(kTR, 12), st, cs, tiles, S,
+                                   (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
             break;
         case 3: launch_tma<Codec, 8, RM>(ntiles, st, cs, tiles, S, D, parity); break;
         case 4: launch_tma<Codec, 16, RM>(ntiles, st, cs, tiles, S, D, parity); break;
