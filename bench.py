@@ -60,12 +60,12 @@ DTYPE = {"fp64": "f64", "fp32": "f32", "mix_fp16": "f32 (fp16 storage)", "mix_bf
 # full launch by the node count.  Kept only for the kernel builds captured
 # (another variant reports null).
 TRAFFIC_B_PER_NODE = {("fp32", 5, "orthogonal"): 163.88}
-# The FP64 step is bound by the FP64 pipe, not by HBM: FP64-pipe thread
-# instructions (DADD + DFMA + DMUL) per node update from one ncu capture
+# The FP64 step's share of the FP64 pipe: its thread instructions on that pipe
+# per node update from one ncu capture
 # (profiles/step_kernel_fp64_batched64cases.md), against the pipe's rate
 # measured in the same run (lbm_measure_fp64_rate: dependent FP64 FMA chains
-# timed with CUDA events).
-FP64_OPS_PER_NODE = 383.3
+# timed with CUDA events).  Most of the step runs in integers, which bound it.
+FP64_OPS_PER_NODE = 34.4
 # What the GPU parity tests hold each precision to against the FP64 oracle.
 PARITY_TOL = {
     "fp64": "phi, rho, u, p within 1e-11 (relative max-norm) of the FP64 oracle",
@@ -536,7 +536,7 @@ def batched_other(torch, args, prec, steps, raw=False):
                                "unit": "G FP64-pipe instructions/s", "frac": gops / peak,
                                "peak_kind": "measured: lbm_measure_fp64_rate (dependent FP64 FMA chains, "
                                             "CUDA events)", "peak_clocks": clk.summary(),
-                               "note": f"{FP64_OPS_PER_NODE} DADD+DFMA+DMUL per node (ncu)"}
+                               "note": f"{FP64_OPS_PER_NODE} FP64-pipe instructions per node (ncu); the step is bound by integer instructions"}
     return out
 
 

@@ -47,7 +47,8 @@ typedef enum {
 } lbm_status;
 
 /* Storage and arithmetic precision of a handle.
- *   LBM_FP64      populations and arithmetic in FP64.
+ *   LBM_FP64      populations in FP64; arithmetic in FP64, or (the paper's rates, both
+ *                 collisions) in 62-bit integers with exponents, with smaller errors.
  *   LBM_FP32      populations f_1..8 and g_0..8 in FP32, arithmetic in FP32
  *                 (reciprocals, divisions and square roots by the hardware
  *                 approximations, a few ulp, subnormal operands and results

@@ -222,8 +222,8 @@ __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7
 __device__ __forceinline__ long long in_units(Sf a, int e) { return shr64(a.m, e - a.e); }
 
 // The macroscopic step of a node of column constants K; the phi window is
-// centred on (a, b).  What depends on phi alone, the reciprocals and the square
-// roots stay on the FP64 pipe, the rest runs beside it in integers.
+// centred on (a, b).  What depends on phi alone stays on the FP64 pipe,
+// the rest runs beside it in integers.
 struct Macro64 {
     Sf gz, gr, Z3, R3;     // 72 grad phi; 0.3 grad rho
     double nu;
