@@ -586,6 +586,16 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
         rc = upload_tiles(h, t, &h->tiles_d[v], true);
     }
     if (rc == LBM_OK) h->variant = default_variant(h);
+    if (rc == LBM_OK) {
+        cudaError_t e = cudaSuccess;
+        switch (h->precision) {
+            case LBM_FP64: e = prepare_step_f64(); break;
+            case LBM_FP32: e = prepare_step_f32(); break;
+            case LBM_MIX_FP16: e = prepare_step_h16(); break;
+            default: e = prepare_step_b16(); break;
+        }
+        if (e != cudaSuccess) rc = LBM_ERR_CUDA;
+    }
     for (int c = 0; c < n && rc == LBM_OK; ++c) {
         std::vector<TileDev> t = make_tiles(h->cases, 8, c);
         TileDev* d = nullptr;

@@ -1131,10 +1131,11 @@ __device__ __forceinline__ Dest destination(int k, int j, int nr, int nz, int zp
 // 2.95 -> 2.70, 128 x 256 3.02 -> 2.76, 200 x 600 5.29 -> 5.03, 256 x 1024
 // 8.43 -> 8.20; launched one by one 5.2 -> 2.9, 6.6 -> 3.0, 8.9 -> 5.5, 11.1 -> 9.0.
 // pdl_trigger lets the next launch start before this CTA ends.  At a kernel's
-// start that is slower: the next step's CTAs gather on few SMs (128 x 256 drop
-// 3.44 us in FP32, 16.1 against 11.4 in FP64), so only the packed kernel uses
-// it, after its window barrier and with more tiles than fit at once.  Without
-// the attribute both do nothing.
+// start that is slower by itself: the next step's CTAs gather on few SMs (128 x
+// 256 drop 3.44 us in FP32, 16.1 against 11.4 in FP64).  So the one-node kernel uses
+// it only with a launch that keeps the SMs even (launch_step_spread), and the
+// packed kernel after its window barrier, with more tiles than fit at once.
+// Without the attribute both do nothing.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -34,3 +34,32 @@ def test_matches_four_row_tiles(nr, nz, coll, prec):
         out.append(sim.state(0))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "mix_fp16"])
+@pytest.mark.parametrize("nr,nz", [(33, 40), (64, 152), (128, 256), (150, 400), (200, 400)])
+def test_early_launches_beside_reads_and_another_stream(nr, nz, prec):
+    """Up to two tiles per SM the next step's blocks are launched while a step runs: steps by
+    graph and one by one, reads between them and a second handle on its own stream."""
+    torch = pytest.importorskip("torch")
+    case = W.oscillating_drop(nr=nr, nz=nz, R0=10.0, ratio=10.0, precision=prec)
+    ref = lbm.Simulation(case)
+    ref.set_variant(2)
+    ref.init_case(0)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    sims = [lbm.Simulation(case, stream=s.cuda_stream) for s in streams]
+    for s in sims:
+        s.set_variant(0)
+        s.init_case(0)
+    for n in (1, 2, 33, 64, 5):
+        ref.step(n)
+        for s in sims:
+            s.step(n)
+        want = ref.fields(0)
+        for s in sims:
+            got = s.fields(0)
+            assert all(np.array_equal(got[k], want[k]) for k in want)
+            s.diagnostics(0)
+    for s in sims:
+        for a, b in zip(s.state(0), ref.state(0)):
+            assert np.array_equal(a, b)
