@@ -1124,7 +1124,7 @@ __device__ __forceinline__ Dest destination(int k, int j, int nr, int nz, int zp
 
 // ---------------------------------------------------------------- programmatic launch
 // A step kernel is launched while the step before it still runs (the launch
-// attribute of launch_step_kernel): its CTAs take their places as that step's
+// attribute of launch_pdl): its CTAs take their places as that step's
 // CTAs end, fetch what does not change from step to step, and wait for that
 // step's completion before they read or write state.  This hides the launch
 // latency between steps; us a step in the captured graph, FP32: 64 x 128 drop
@@ -1133,11 +1133,33 @@ __device__ __forceinline__ Dest destination(int k, int j, int nr, int nz, int zp
 // pdl_trigger lets the next launch start before this CTA ends.  At a kernel's
 // start that is slower by itself: the next step's CTAs gather on few SMs (128 x
 // 256 drop 3.44 us in FP32, 16.1 against 11.4 in FP64).  So the one-node kernel uses
-// it only with a launch that keeps the SMs even (launch_step_spread), and the
-// packed kernel after its window barrier, with more tiles than fit at once.
+// it only with a launch that keeps the SMs even (launch_step_spread), the
+// packed kernel after its window barrier, with more tiles than fit at once, and the
+// kernels of a read at their start.
 // Without the attribute both do nothing.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A launch that may overlap the end of the launch before it on the stream
+// (programmatic stream serialisation).
+template <class... P, class... A>
+void launch_pdl_dyn(void (*kernel)(P...), int grid, dim3 block, size_t dyn, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <class... P, class... A>
+void launch_pdl(void (*kernel)(P...), int grid, dim3 block, cudaStream_t st, A... args) {
+    launch_pdl_dyn(kernel, grid, block, 0, st, args...);
+}
 
 // ---------------------------------------------------------------- TMA / mbarrier
 // Bulk tensor copies global -> shared completed on an mbarrier (PTX ISA,

@@ -111,15 +111,21 @@ __device__ __forceinline__ void warp_extrema(const double* uu, const double* lo,
     out[3] = nb;
 }
 
+// The kernels of a record and of the drops follow each other and the fields kernel
+// with overlapping launches (pdl_wait); what they read of one another's is not
+// marked __restrict__, so that no load of it moves above the wait.  A record right
+// after a step of the 64 x 128 drop (FP64): 78 -> 71 us; its drops 30 -> 26 us.
+//
 // One partial record per block.  Rows k = blockIdx.x, blockIdx.x + gridDim.x,
 // ...; within a row each thread takes the columns j = threadIdx.x + 256 i, so a
 // thread holds only a few nodes and sums them plainly; the block's 256 values
 // of each quantity are then summed pairwise by one warp per quantity (warps
 // 0-6 the sums, warp 7 the extrema and the count).  The records of the blocks
 // are combined exactly by diag_final_kernel.
-__global__ void __launch_bounds__(kDiagThreads) diag_partial_kernel(const double* __restrict__ F, int nz, int nr,
-                                                                    double* __restrict__ partials) {
+__global__ void __launch_bounds__(kDiagThreads) diag_partial_kernel(const double* F, int nz, int nr, double* partials) {
     static_assert(kDiagThreads == 32 * (kSums + 1), "one warp per sum plus one");
+    pdl_trigger();
+    pdl_wait();
     const int64_t n = (int64_t)nz * nr;
     double acc[kSums] = {};
     double uu_max = 0.0, pmin = INFINITY, pmax = -INFINITY, bad = 0.0;
@@ -176,7 +182,7 @@ __global__ void __launch_bounds__(kDiagThreads) diag_partial_kernel(const double
 // Contribution of the axis link (k, k+1) to the length of the phi > 1/2 set on
 // the axis row (linear crossing); the last link wraps when z is periodic and
 // is half a cell at a wall.
-__device__ __forceinline__ double axis_link(const double* __restrict__ F, int k, int nz, int nr, int zper) {
+__device__ __forceinline__ double axis_link(const double* F, int k, int nz, int nr, int zper) {
     const double a = F[(int64_t)k * nr] - 0.5;
     int kn = k + 1;
     if (kn >= nz) {
@@ -197,10 +203,9 @@ __device__ __forceinline__ double axis_link(const double* __restrict__ F, int k,
 // records only for its rows.
 constexpr int kFinalThreads = 256;
 static_assert(kFinalThreads == 32 * (kSums + 1), "one warp per sum plus one");
-__global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double* __restrict__ F, int nz, int nr,
+__global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double* F, int nz, int nr,
                                                                    int zper, double step,
-                                                                   const double* __restrict__ partials,
-                                                                   double* __restrict__ out, const int* status,
+                                                                   const double* partials, double* out, const int* status,
                                                                    int* status_out) {
     __shared__ double sres[kSums + 4];
     __shared__ double slen[kFinalThreads / 32];
@@ -208,6 +213,7 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const int records = min(nz, kDiagBlocks);
     if (t == 0) sjmin = nr;
+    pdl_wait();
     // axis half-length: per-thread sums over k = t, t + T, ..., then a shuffle tree
     double len = 0.0;
     for (int k = t; k < nz; k += kFinalThreads) len += axis_link(F, k, nz, nr, zper);
@@ -288,9 +294,10 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
 constexpr int kAxisThreads = 256;
 constexpr int kAxisRows = 2816;  // rows whose two doubles fit 44 KB of shared memory
 
-__global__ void __launch_bounds__(kAxisThreads) axis_rows_kernel(const double* __restrict__ F, int nz, int nr,
-                                                                 double* __restrict__ rows) {
+__global__ void __launch_bounds__(kAxisThreads) axis_rows_kernel(const double* F, int nz, int nr, double* rows) {
     const int k = blockIdx.x * (kAxisThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    pdl_trigger();
+    pdl_wait();
     if (k >= nz) return;
     const double* P = F + (int64_t)k * nr;
     double s = 0.0;
@@ -333,8 +340,8 @@ __device__ __forceinline__ double sum_rows(const double* rows, int nz, int k0, i
     return s;
 }
 
-__global__ void __launch_bounds__(kAxisThreads) axis_drops_kernel(const double* __restrict__ rows_g, int nz, int zper,
-                                                                  int max_drops, double* __restrict__ out,
+__global__ void __launch_bounds__(kAxisThreads) axis_drops_kernel(const double* rows_g, int nz, int zper,
+                                                                  int max_drops, double* out,
                                                                   const int* status, int* status_out) {
     constexpr int kWarps = kAxisThreads / 32;
     __shared__ double sbuf[2 * kAxisRows];
@@ -342,6 +349,7 @@ __global__ void __launch_bounds__(kAxisThreads) axis_drops_kernel(const double* 
     __shared__ int s_kmin[kWarps], s_gas[kWarps], s_last[kWarps], s_cnt[kWarps];
     __shared__ int s_a[kMaxAxisDrops + 1], s_b[kMaxAxisDrops + 1];  // runs of the first drops, scan indices
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    pdl_wait();
     if (t == 0) *status_out = *status;
     const bool fits = nz <= kAxisRows;
     for (int i = t; fits && i < 2 * nz; i += kAxisThreads) sbuf[i] = rows_g[i];
@@ -531,16 +539,16 @@ int diag_partials_size() { return kDiagPartials; }
 
 cudaError_t launch_diag(const double* fields, int nz, int nr, int zper, double step, double* partials, double* out,
                         const int* status, int* status_out, cudaStream_t st) {
-    diag_partial_kernel<<<nz < kDiagBlocks ? nz : kDiagBlocks, kDiagThreads, 0, st>>>(fields, nz, nr, partials);
-    diag_final_kernel<<<1, kFinalThreads, 0, st>>>(fields, nz, nr, zper, step, partials, out, status, status_out);
+    launch_pdl(diag_partial_kernel, nz < kDiagBlocks ? nz : kDiagBlocks, dim3(kDiagThreads), st, fields, nz, nr, partials);
+    launch_pdl(diag_final_kernel, 1, dim3(kFinalThreads), st, fields, nz, nr, zper, step, partials, out, status, status_out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_axis_drops(const double* fields, int nz, int nr, int zper, int max_drops, double* rows, double* out,
                               const int* status, int* status_out, cudaStream_t st) {
     constexpr int per = kAxisThreads / 32;
-    axis_rows_kernel<<<(nz + per - 1) / per, kAxisThreads, 0, st>>>(fields, nz, nr, rows);
-    axis_drops_kernel<<<1, kAxisThreads, 0, st>>>(rows, nz, zper, max_drops, out, status, status_out);
+    launch_pdl(axis_rows_kernel, (nz + per - 1) / per, dim3(kAxisThreads), st, fields, nz, nr, rows);
+    launch_pdl(axis_drops_kernel, 1, dim3(kAxisThreads), st, rows, nz, zper, max_drops, out, status, status_out);
     return cudaGetLastError();
 }
 

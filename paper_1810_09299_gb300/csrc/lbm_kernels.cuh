@@ -1419,6 +1419,8 @@ fields_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ til
     __shared__ int swe[kU64 ? NWIN : 1];
     const Win64 W{swm, swe};
     const TileDev t = tiles[blockIdx.x];
+    pdl_trigger();
+    pdl_wait();
     if (status_out != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *status_out = *status;
     const CaseDev& C = cases[t.c];
     const CaseView<Codec> V = case_view<Codec>(S, C);
@@ -1699,28 +1701,6 @@ void launch_tma(int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* t
         cs, tiles, ntiles, S, (const CUtensorMap*)D.tmaps, BZ == 8 ? 0 : 1, parity, D.status);
 }
 
-// A step launch that may overlap the end of the launch before it on the stream
-// (programmatic stream serialisation; see pdl_wait).
-template <class... P, class... A>
-void launch_step_kernel_dyn(void (*kernel)(P...), int grid, dim3 block, size_t dyn, cudaStream_t st, A... args) {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = dyn;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
-template <class... P, class... A>
-void launch_step_kernel(void (*kernel)(P...), int grid, dim3 block, cudaStream_t st, A... args) {
-    launch_step_kernel_dyn(kernel, grid, block, 0, st, args...);
-}
-
 // Grids of at most two tiles per SM, in one wave: the launch after a step starts
 // when that step's CTAs have started (EARLY), and each CTA asks for so much shared
 // memory that an SM takes no more of them than the grid needs.  Without the second
@@ -1754,7 +1734,7 @@ bool launch_step_spread(int ntiles, int sms, cudaStream_t st, const CaseDev* cs,
                           2 * (spread_bytes<Codec, BZ, RM>(2) + sizeof(TileShared<Codec, BZ, RM>) + kCtaReserved) <= kSmBytes,
                       "one and two CTAs fit");
         if (ntiles > 2 * sms) return false;
-        launch_step_kernel_dyn(spread_kernel<Codec, BZ, RM>, ntiles, dim3(kTR, BZ),
+        launch_pdl_dyn(spread_kernel<Codec, BZ, RM>, ntiles, dim3(kTR, BZ),
                                spread_bytes<Codec, BZ, RM>(ntiles > sms ? 2 : 1), st, cs, tiles, S,
                                (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
         return true;
@@ -1796,56 +1776,56 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
             if (launch_step_spread<Codec, 8, RM>(ntiles, sms, st, cs, tiles, S, parity)) break;
             if constexpr (sizeof(typename Codec::Real) == 8 && RM != kRatesGeneral) {
                 if (ntiles >= 6 * sms) {
-                    launch_step_kernel(step_kernel<Codec, 8, RM, kF64Full>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0,
+                    launch_pdl(step_kernel<Codec, 8, RM, kF64Full>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0,
                                        parity, ntiles, kPrefetchQuarters * sms * kF64Full / 4);
                     break;
                 }
             }
-            launch_step_kernel(step_kernel<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 8, RM>() / 4);
+            launch_pdl(step_kernel<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 8, RM>() / 4);
             break;
         case 1:
-            launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+            launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         case 2:
-            launch_step_kernel(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
+            launch_pdl(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
             break;
         case 8:  // (one wave: nothing to prefetch)
             if (launch_step_spread<Codec, 10, RM>(ntiles, sms, st, cs, tiles, S, parity)) break;
             if constexpr (RM != kRatesGeneral && !kSpread<Codec, RM>)
-                launch_step_kernel(step_kernel<Codec, 10, RM>, ntiles, dim3(kTR, 10), st, cs, tiles, S,
+                launch_pdl(step_kernel<Codec, 10, RM>, ntiles, dim3(kTR, 10), st, cs, tiles, S,
                                    (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
             break;
         case 9:
             if (launch_step_spread<Codec, 12, RM>(ntiles, sms, st, cs, tiles, S, parity)) break;
             if constexpr (RM != kRatesGeneral && !kSpread<Codec, RM>)
-                launch_step_kernel(step_kernel<Codec, 12, RM>, ntiles, dim3(kTR, 12), st, cs, tiles, S,
+                launch_pdl(step_kernel<Codec, 12, RM>, ntiles, dim3(kTR, 12), st, cs, tiles, S,
                                    (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
             break;
         case 3: launch_tma<Codec, 8, RM>(ntiles, st, cs, tiles, S, D, parity); break;
         case 4: launch_tma<Codec, 16, RM>(ntiles, st, cs, tiles, S, D, parity); break;
         case 5:
             if constexpr (sizeof(typename Codec::Real) == 4)
-                launch_step_kernel(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
+                launch_pdl(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
             else
-                launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         case 7:
             if constexpr (Codec::kGrid)
-                launch_step_kernel(ntiles > sms * AXILBM_PACK2_CTAS ? step_kernel_pack2<Codec, RM, true>
+                launch_pdl(ntiles > sms * AXILBM_PACK2_CTAS ? step_kernel_pack2<Codec, RM, true>
                                                                     : step_kernel_pack2<Codec, RM, false>,
                                    ntiles, dim3(kTR, 8), st, cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps,
                                    parity, ntiles, kPrefetchQuarters * sms * AXILBM_PACK2_CTAS / 4);
             else if constexpr (sizeof(typename Codec::Real) == 4)
-                launch_step_kernel(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
+                launch_pdl(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
             else
-                launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         default:
             if constexpr (sizeof(typename Codec::Real) == 4)
-                launch_step_kernel(step_kernel_seq2<Codec, 8, RM, true>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles,
+                launch_pdl(step_kernel_seq2<Codec, 8, RM, true>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles,
                     kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM, true>() / 4);
             else
-                launch_step_kernel(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
     }
 }
@@ -1871,16 +1851,12 @@ cudaError_t launch_fields_t(const DeviceState& D, int parity, const TileDev* til
     const CaseDev* cs = (const CaseDev*)D.cases;
     const dim3 block(kTR, 8);
     constexpr bool f64 = sizeof(typename Codec::Real) == 8;
-    if (phi_only) fields_kernel<Codec, kRatesGeneral, true><<<ntiles, block, 0, st>>>(cs, tiles, S, out, D.status,
-                                                                                      status_out);
-    else if (f64 && D.rate_mode == kRatesPaper)
-        fields_kernel<Codec, f64 ? kRatesPaper : kRatesGeneral, false><<<ntiles, block, 0, st>>>(cs, tiles, S, out, D.status,
-                                                                                      status_out);
+    auto launch = [&](auto* kernel) { launch_pdl(kernel, ntiles, block, st, cs, tiles, S, out, D.status, status_out); };
+    if (phi_only) launch(fields_kernel<Codec, kRatesGeneral, true>);
+    else if (f64 && D.rate_mode == kRatesPaper) launch(fields_kernel<Codec, f64 ? kRatesPaper : kRatesGeneral, false>);
     else if (f64 && D.rate_mode == kRatesPaperRaw)
-        fields_kernel<Codec, f64 ? kRatesPaperRaw : kRatesGeneral, false><<<ntiles, block, 0, st>>>(cs, tiles, S, out, D.status,
-                                                                                      status_out);
-    else fields_kernel<Codec, kRatesGeneral, false><<<ntiles, block, 0, st>>>(cs, tiles, S, out, D.status,
-                                                                                      status_out);
+        launch(fields_kernel<Codec, f64 ? kRatesPaperRaw : kRatesGeneral, false>);
+    else launch(fields_kernel<Codec, kRatesGeneral, false>);
     return cudaGetLastError();
 }
 
