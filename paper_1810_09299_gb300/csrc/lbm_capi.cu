@@ -170,16 +170,17 @@ cudaError_t launch_step_any(lbm_sim* h, int parity, int variant, cudaStream_t st
     }
 }
 
-// The fields of case icase: all five, or phi alone.
+// The fields of case icase: all five, or phi alone, into h->fields or out.
 cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st, bool phi_only = false,
-                              int* status_out = nullptr) {
+                              int* status_out = nullptr, double* out = nullptr) {
     const TileDev* t = h->ftiles_d[icase];
     const int n = h->nftiles[icase];
+    if (!out) out = h->fields;
     switch (h->precision) {
-        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
-        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
-        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
-        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, h->fields, status_out, st);
+        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, out, status_out, st);
+        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, out, status_out, st);
+        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, out, status_out, st);
+        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, out, status_out, st);
     }
 }
 
@@ -690,6 +691,22 @@ void touch_pages(void* dst, size_t bytes) {
     p[bytes - 1] = 0;
 }
 
+// The address under which kernels store into page-locked host memory, or null for
+// any other memory, and for a range that is not page-locked to its end or not aligned.
+double* mapped_doubles(double* host, size_t bytes) {
+    if (((uintptr_t)host & (sizeof(double) - 1)) != 0) return nullptr;
+    cudaPointerAttributes a{}, b{};
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
+        cudaPointerGetAttributes(&b, (char*)host + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
+        (char*)b.devicePointer - (char*)a.devicePointer != (ptrdiff_t)bytes - 1)
+        return nullptr;
+    return (double*)a.devicePointer;
+}
+
 int check_case(lbm_sim* h, int icase) {
     if (icase < 0 || icase >= h->ncases) return LBM_ERR_INVALID_ARG;
     return LBM_OK;
@@ -843,9 +860,16 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
     if (!h->initialized[icase]) return LBM_ERR_STATE;
     rc = join_diagnostics(h);
     if (rc != LBM_OK) return rc;
-    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI, status_host(h)));
-    if (rc != LBM_OK) return rc;
     const int64_t n = (int64_t)h->prm[icase].nz * h->prm[icase].nr;
+    // phi or all five into page-locked memory: stored there by the kernel, without a
+    // copy behind it (us a call, 256 x 416: FP32 phi 20.7 -> 16.4, all five 47.0 -> 35.8;
+    // FP64 29.4 -> 17.8 and 52.2 -> 42.2; 64 x 128: FP32 15.6 -> 12.2 and 21.4 -> 15.3)
+    double* direct = nullptr;
+    if (mask == LBM_FIELD_PHI || mask == 31)
+        direct = mapped_doubles(host_out, (mask == 31 ? 5 : 1) * n * sizeof(double));
+    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI, status_host(h), direct));
+    if (rc != LBM_OK) return rc;
+    if (direct) return finish_status(h);
     int64_t slot = 0;
     for (int b = 0; b < 5;) {
         int e = b;  // neighbouring planes leave in one copy

@@ -25,6 +25,30 @@ def test_phi_alone_is_the_phi_of_all_fields(nr, nz, raw, prec):
     assert np.array_equal(sim.fields(0, which=("phi",))["phi"], sim.fields(0)["phi"])
 
 
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "mix_fp16", "mix_bf16"])
+@pytest.mark.parametrize("nr,nz", [(2, 2), (33, 17), (97, 65)])
+def test_fields_into_page_locked_memory(nr, nz, prec):
+    """Stored there by the kernel where the address is aligned, by a copy where it is not or
+    where planes are left out: the same values, and nothing beyond them."""
+    torch = pytest.importorskip("torch")
+    sim = lbm.Simulation(W.oscillating_drop(nr=nr, nz=nz, R0=0.3 * nr, ratio=10.0, precision=prec))
+    sim.init_case(0)
+    sim.step(2)
+    n = nr * nz
+    planes = list(sim.fields(0).values())
+    for mask in (1, 31, 3, 16):
+        want = np.concatenate([planes[i].ravel() for i in range(5) if mask & (1 << i)])
+        for offset in (0, 8, 4):
+            buf = torch.zeros(8 * (5 * n + 4), dtype=torch.uint8, pin_memory=True)
+            rc = lbm.lib().lbm_case_get_fields(sim._h, 0, mask, ctypes.cast(buf.data_ptr() + offset,
+                                                                            ctypes.POINTER(ctypes.c_double)))
+            assert rc == lbm.LBM_OK
+            raw = buf.numpy()
+            got = np.frombuffer(raw[offset:offset + 8 * want.size].tobytes())
+            assert np.array_equal(got, want)
+            assert not raw[:offset].any() and not raw[offset + 8 * want.size:].any()
+
+
 @pytest.mark.parametrize("zper", [0, 1])
 @pytest.mark.parametrize("nz,period", [(2, 2), (3, 3), (255, 7), (256, 2), (257, 16),  # a scan thread's share
                                        (2816, 40), (2817, 40), (5000, 999),            # rows in shared memory, or not
