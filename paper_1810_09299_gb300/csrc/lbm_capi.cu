@@ -587,7 +587,8 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
         rc = upload_tiles(h, t, &h->tiles_d[v], true);
     }
     if (rc == LBM_OK) h->variant = default_variant(h);
-    if (rc == LBM_OK) {
+    // (the grids whose variant 0 may take them; the first call loads the kernels)
+    if (rc == LBM_OK && h->ntiles[h->row_shape] <= 2 * sm_count(h)) {
         cudaError_t e = cudaSuccess;
         switch (h->precision) {
             case LBM_FP64: e = prepare_step_f64(); break;
