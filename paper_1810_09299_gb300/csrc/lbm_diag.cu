@@ -111,14 +111,29 @@ __device__ __forceinline__ void warp_extrema(const double* uu, const double* lo,
     out[3] = nb;
 }
 
+// A double as an integer of the same order (and back): extrema and thresholds are
+// compared beside the FP64 pipe.
+__device__ __forceinline__ long long ordered(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double unordered(long long b) {
+    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
+}
+// phi of these bits: of a finite phi, b > kLiquid where phi > 0.99 and b < kGas
+// where phi < 0.01 (negative ones have negative bits)
+constexpr long long kLiquid = 0x3fefae147ae147aell, kGas = 0x3f847ae147ae147bll;
+
 // The kernels of a record and of the drops follow each other and the fields kernel
 // with overlapping launches (pdl_wait); what they read of one another's is not
 // marked __restrict__, so that no load of it moves above the wait.  A record right
 // after a step of the 64 x 128 drop (FP64): 78 -> 71 us; its drops 30 -> 26 us.
 //
 // One partial record per block.  Rows k = blockIdx.x, blockIdx.x + gridDim.x,
-// ...; within a row each thread takes the columns j = threadIdx.x + 256 i, so a
-// thread holds only a few nodes and sums them plainly; the block's 256 values
+// ...; of these each thread takes the columns j = threadIdx.x + 256 i, so it
+// holds only a few nodes and sums them plainly, a column's before they are
+// weighted with its r: 7 FP64 operations per node instead of some 25
+// (256 x 1024: 20.9 -> 13.7 us, a whole record 77 -> 51 us in FP32); the block's 256 values
 // of each quantity are then summed pairwise by one warp per quantity (warps
 // 0-6 the sums, warp 7 the extrema and the count).  The records of the blocks
 // are combined exactly by diag_final_kernel.
@@ -128,39 +143,43 @@ __global__ void __launch_bounds__(kDiagThreads) diag_partial_kernel(const double
     pdl_wait();
     const int64_t n = (int64_t)nz * nr;
     double acc[kSums] = {};
-    double uu_max = 0.0, pmin = INFINITY, pmax = -INFINITY, bad = 0.0;
-    for (int k = blockIdx.x; k < nz; k += gridDim.x) {
-        const double z = k + 0.5;
-        for (int j = threadIdx.x; j < nr; j += blockDim.x) {
+    long long uu_max = 0, pmin = ordered(INFINITY), pmax = ordered(-INFINITY);
+    int bad = 0;
+    for (int j = threadIdx.x; j < nr; j += blockDim.x) {
+        double phi_s = 0.0, uu_s = 0.0, z_s = 0.0, p_liq = 0.0, p_gas = 0.0, z = blockIdx.x + 0.5;
+        int n_liq = 0, n_gas = 0;
+        for (int k = blockIdx.x; k < nz; k += gridDim.x, z += (double)gridDim.x) {
             const int64_t o = (int64_t)k * nr + j;
-            const double r = j + 0.5;
             const double phi = F[o], rho = F[n + o], uz = F[2 * n + o], ur = F[3 * n + o], p = F[4 * n + o];
-            if (!isfinite(phi) || !isfinite(uz) || !isfinite(ur) || !isfinite(p)) {
-                bad += 1.0;
+            if (max(max(abs_hi(phi), abs_hi(p)), max(abs_hi(uz), abs_hi(ur))) >= 0x7ff00000) {
+                ++bad;
                 continue;
             }
             const double uu = uz * uz + ur * ur;
-            acc[0] += r * phi;
-            acc[1] += 0.5 * r * rho * uu;
-            acc[2] += r * z * phi;
-            if (phi > 0.99) {
-                acc[3] += r * p;
-                acc[4] += r;
-            }
-            if (phi < 0.01) {
-                acc[5] += r * p;
-                acc[6] += r;
-            }
-            uu_max = fmax(uu_max, uu);
-            pmin = fmin(pmin, phi);
-            pmax = fmax(pmax, phi);
+            phi_s += phi;
+            uu_s += rho * uu;
+            z_s += z * phi;
+            const long long b = __double_as_longlong(phi);
+            if (b > kLiquid) p_liq += p, ++n_liq;  // phi > 0.99
+            if (b < kGas) p_gas += p, ++n_gas;     // phi < 0.01
+            uu_max = max(uu_max, __double_as_longlong(uu));
+            pmin = min(pmin, ordered(phi));
+            pmax = max(pmax, ordered(phi));
         }
+        const double r = j + 0.5;
+        acc[0] += r * phi_s;
+        acc[1] += 0.5 * r * uu_s;
+        acc[2] += r * z_s;
+        acc[3] += r * p_liq;
+        acc[4] += r * n_liq;
+        acc[5] += r * p_gas;
+        acc[6] += r * n_gas;
     }
     __shared__ double sh[kSums + 4][kDiagThreads];
     for (int q = 0; q < kSums; ++q) sh[q][threadIdx.x] = acc[q];
-    sh[kSums][threadIdx.x] = uu_max;
-    sh[kSums + 1][threadIdx.x] = pmin;
-    sh[kSums + 2][threadIdx.x] = pmax;
+    sh[kSums][threadIdx.x] = __longlong_as_double(uu_max);
+    sh[kSums + 1][threadIdx.x] = unordered(pmin);
+    sh[kSums + 2][threadIdx.x] = unordered(pmax);
     sh[kSums + 3][threadIdx.x] = bad;
     __syncthreads();
     const int w = threadIdx.x >> 5;
@@ -209,6 +228,7 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
                                                                    int* status_out) {
     __shared__ double sres[kSums + 4];
     __shared__ double slen[kFinalThreads / 32];
+    __shared__ double s_dp[2], s_umax;
     __shared__ int sjmin;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const int records = min(nz, kDiagBlocks);
@@ -234,6 +254,12 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
     // radial crossing on the row nearest the centroid: the first outward crossing
     int kc = (int)floor(zc);
     kc = kc < 0 ? 0 : (kc >= nz ? nz - 1 : kc);
+    // the record's other divisions and its root, a warp each
+    if (lane == 0) {
+        if (w == 1) s_dp[0] = sres[4] > 0 ? sres[3] / sres[4] : 0.0;
+        if (w == 2) s_dp[1] = sres[6] > 0 ? sres[5] / sres[6] : 0.0;
+        if (w == 3) s_umax = sqrt(sres[kSums]);  // |u|max from the largest |u|^2
+    }
     for (int j = t; j + 1 < nr; j += kFinalThreads) {
         const double a = F[(int64_t)kc * nr + j] - 0.5, b = F[(int64_t)kc * nr + j + 1] - 0.5;
         if (a > 0 && b <= 0) {
@@ -251,14 +277,12 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
     double axis = 0.0;
     for (int i = 0; i < kFinalThreads / 32; ++i) axis += slen[i];
     if (!zper && F[0] - 0.5 > 0) axis += 0.5;
-    const double win = sres[4], wout = sres[6];
-    const double dp = (win > 0 ? sres[3] / win : 0.0) - (wout > 0 ? sres[5] / wout : 0.0);
     out[0] = step;
     out[1] = mass;
     out[2] = sres[1];
     out[3] = zc;
-    out[4] = dp;
-    out[5] = sqrt(sres[kSums]);  // |u|max from the largest |u|^2
+    out[4] = s_dp[0] - s_dp[1];
+    out[5] = s_umax;
     out[6] = sres[kSums + 1];
     out[7] = sres[kSums + 2];
     out[8] = 0.5 * axis;

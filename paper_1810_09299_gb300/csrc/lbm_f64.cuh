@@ -217,7 +217,6 @@ __device__ __forceinline__ ColRef64 ColTab64::at(int j) const { return ColRef64{
 // 16 bytes per column and Sf, 8 per double
 constexpr size_t col_tab64_bytes(int n) { return (size_t)n * (2 * 8 + kColSf * 16); }
 
-__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
 // a's integer in units of 2^e, e >= a.e
 __device__ __forceinline__ long long in_units(Sf a, int e) { return shr64(a.m, e - a.e); }
 

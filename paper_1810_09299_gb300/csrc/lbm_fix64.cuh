@@ -21,6 +21,7 @@ namespace axilbm {
 constexpr int kMinE = 64, kBadE = 2030;
 
 __device__ __forceinline__ int exp64(double x) { return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu); }
+__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
 // shifts whose amounts may exceed 63 (PTX: all bits leave, or the sign fills)
 __device__ __forceinline__ unsigned long long shr64u(unsigned long long v, int s) {
     unsigned long long r;
