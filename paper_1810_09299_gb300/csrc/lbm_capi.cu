@@ -452,7 +452,7 @@ int row_shape(const lbm_sim* h) {
 // results know no difference).  us a step in the captured graph:
 //   4-row tiles (2) instead of 8-row tiles (0)
 //     where those leave half the SMs empty, FP64 and bfloat16 (a 64 x 128 drop, 32
-//     tiles of 8 rows: 9.2 -> 7.9 and 3.02 -> 2.77; FP32 2.45 and 2.39, FP16 2.90
+//     tiles of 8 rows: 9.2 -> 7.8 and 3.02 -> 2.77; FP32 2.32 and 2.45, FP16 2.90
 //     either way), and where some SMs would hold two of them, most one and taller
 //     tiles do not help (row_shape's figures).  128 tiles (128 x 256) and 250 (150 x
 //     400) take 8 rows: FP32 2.52 against 2.77 and 3.41 against 3.66.
