@@ -226,7 +226,7 @@ __device__ __forceinline__ long long in_units(Sf a, int e) { return shr64(a.m, e
 struct Macro64 {
     Sf gz, gr, Z3, R3;     // 72 grad phi; 0.3 grad rho
     double nu;
-    Sf rho, s, D;          // s = 1 / tau_g, D = 1 / (r rho + nu rho / r)
+    Sf rho, s;             // s = 1 / tau_g
     Sf uz, rz, ur, p, ps;  // rz = rho u_z; ps: the p of Eq. 30 and Eq. 32
     Sf rFsr;               // r F_s,r
     Two JFz;               // J_z and F_z (Eq. 30)
@@ -290,7 +290,7 @@ __device__ __forceinline__ Macro64 macros64(const CaseDev& C, const Win64& W, in
         ur = norm29(ca + scale2(D, -1) * p);
     }
     m.bad = m.bad || Q.bad || top >= 0x7ff00000;
-    m.Z3 = Z3, m.R3 = R3, m.nu = nu, m.rho = rho, m.s = s, m.D = D;
+    m.Z3 = Z3, m.R3 = R3, m.nu = nu, m.rho = rho, m.s = s;
     m.uz = uz, m.rz = rz, m.ur = ur, m.p = p, m.ps = ps, m.rFsr = rFsr, m.JFz = JFz;
     return m;
 }

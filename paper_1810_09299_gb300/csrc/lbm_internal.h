@@ -51,7 +51,7 @@ struct DeviceState {
     cudaError_t launch_set_state_##NAME(const DeviceState& D, int parity, const CaseDev& C, const double* f,        \
                                         const double* g, const double* aux, cudaStream_t st);
 
-// The column table of an FP64 handle (rate mode D.rate_mode): its size, and
+// The column table of an FP64 handle: its size, and
 // the kernel that fills it.
 size_t col_tab64_size(int ncols);
 cudaError_t launch_col_tab64(double* cols, int ncols, cudaStream_t st);

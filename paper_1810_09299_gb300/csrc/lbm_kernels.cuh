@@ -135,17 +135,17 @@ __device__ __forceinline__ void ring_cell(int q, int& a, int& b) {
 // FP64 with a compile-time rate pattern: 16 warps per SM at 128 registers, or with
 // 6 tiles of 8 rows per SM and more kF64Full CTAs (24 warps, 80 registers, 176 bytes
 // of spill): 32 cases (7386 tiles) 313 -> 302 us, 256 x 1024 (1024) 47.7 -> 46.5, but
-// 200 x 600 (525) 26.3 -> 27.2 and 128 x 256 (128) 9.1 -> 11.0.  The 4-row tiles, which
-// serve grids of fewer tiles than SMs, take 136 registers (3 CTAs per SM; with 4 at
-// 128: 64 x 128 7.94 against 7.76, raw moments 8.22 against 7.81).
-constexpr int kF64Full = 3;
+// 200 x 600 (525) 26.3 -> 27.2 and 128 x 256 (128) 9.1 -> 11.0.  4-row tiles
+// that have an SM each take 136 registers (kF64Few CTAs; with 4 at 128: 64 x 128 7.94
+// against 7.76, raw moments 8.22 against 7.81; 200 x 600, 1050 tiles, 26.7 against 31.1).
+constexpr int kF64Full = 3, kF64Few = 3;
 template <class Codec, int BZ, int RM>
 constexpr int step_min_blocks() {
     constexpr int bz8 = Codec::kGrid ? AXILBM_GRID16_CTAS
                         : (RM == kRatesPaperRaw && sizeof(typename Codec::PT) == 2)
                             ? 4
                             : (sizeof(typename Codec::PT) == 2 ? AXILBM_STEP16_CTAS : 5);
-    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ > 8 ? 1 : (BZ == 4 ? 3 : 2)))
+    return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ > 8 ? 1 : (BZ == 4 ? 4 : 2)))
            : BZ == 10 || BZ == 12 ? 2 : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
                 : (BZ >= 16 ? 1 : (BZ >= 8 ? AXILBM_GENERAL_CTAS : 2 * AXILBM_GENERAL_CTAS));
 }
@@ -1789,6 +1789,13 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
             launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
             break;
         case 2:
+            if constexpr (sizeof(typename Codec::Real) == 8 && RM != kRatesGeneral) {
+                if (ntiles <= sms) {
+                    launch_pdl(step_kernel<Codec, 4, RM, kF64Few>, ntiles, dim3(kTR, 4), st, cs, tiles, S,
+                               (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
+                    break;
+                }
+            }
             launch_pdl(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
             break;
         case 8:  // (one wave: nothing to prefetch)
