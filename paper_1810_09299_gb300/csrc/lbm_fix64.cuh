@@ -22,6 +22,7 @@ constexpr int kMinE = 64, kBadE = 2030;
 
 __device__ __forceinline__ int exp64(double x) { return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu); }
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+#ifdef __CUDACC__
 // shifts whose amounts may exceed 63 (PTX: all bits leave, or the sign fills)
 __device__ __forceinline__ unsigned long long shr64u(unsigned long long v, int s) {
     unsigned long long r;
@@ -33,6 +34,34 @@ __device__ __forceinline__ long long shr64(long long v, int s) {
     asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
     return r;
 }
+__device__ __forceinline__ unsigned long long shl64u(unsigned long long v, int s) {
+    unsigned long long r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+    return r;
+}
+// places from the leading non-sign bit to bit 63 (31); -1 for 0 and -1
+__device__ __forceinline__ int lead_shift64(long long v) {
+    int r;
+    asm("bfind.shiftamt.s64 %0, %1;" : "=r"(r) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ int lead_shift32(int v) {
+    int r;
+    asm("bfind.shiftamt.s32 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
+}
+// 1 / x and 1 / sqrt(x) within 1 ulp and 2^-22.9 (the PTX ISA's bounds)
+__device__ __forceinline__ float rcp_start(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rsqrt_start(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+#endif  // a host compiler includes this file after its own definitions of these and of CUDA's intrinsics
 __device__ __forceinline__ double nan64() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 // x in the block of exponent E >= exp64(x), truncated towards zero.
@@ -93,11 +122,12 @@ struct Sf {
 };
 constexpr int kZeroE = -(1 << 17);
 
-// a b 2^-62, |a|, |b| < 2^62, within 8 units: the low words' product and the bits
-// below the high words of the mixed ones are left out, about 5 units on average,
-// and 4 are added back (to a zero, too: one that must stay zero is the caller's, or has
-// the exponent kZeroE).  High-word multiplications (30.6 per SM and cycle) rather
-// than signed wide ones (12).
+// a b 2^-62, |a|, |b| < 2^62 (-2^62 too), within 10 units: the bits below the high
+// words of the mixed products (up to 8 units), the low words' product (4) and their last
+// bits (1 each, either way) are left out, about 5 units on average, and 4 are added back
+// (to a zero, too: one that must stay zero is the caller's, or has the exponent
+// kZeroE).  High-word multiplications (30.6 per SM and cycle) rather than signed wide
+// ones (12).
 __device__ __forceinline__ long long mul62(long long a, long long b) {
     const int ah = (int)(a >> 32) * 2, bh = (int)(b >> 32) * 2;
     const int al = (int)((uint32_t)a >> 1), bl = (int)((uint32_t)b >> 1);
@@ -127,19 +157,13 @@ __device__ __forceinline__ Sf scale2(Sf a, int n) { return Sf{a.m, a.e + n}; }  
 __device__ __forceinline__ Sf neg(Sf a) { return Sf{-a.m, a.e}; }
 // The same value with 2^61 <= |m| < 2^62 (zero: see above).
 __device__ __forceinline__ Sf norm(Sf a) {
-    int sh;  // places from the leading non-sign bit to bit 63; -1 for 0 and -1
-    asm("bfind.shiftamt.s64 %0, %1;" : "=r"(sh) : "l"(a.m));
-    Sf r;
-    asm("shl.b64 %0, %1, %2;" : "=l"(r.m) : "l"(a.m), "r"(sh - 2));
-    r.e = sh < 0 ? kZeroE : a.e - (sh - 2);
-    return r;
+    const int sh = lead_shift64(a.m);
+    return Sf{(long long)shl64u((unsigned long long)a.m, sh - 2), sh < 0 ? kZeroE : a.e - (sh - 2)};
 }
 // The same by at most 29 places, from the high word alone: enough for a factor
 // that is a sum, since bits further down carry the sum's own rounding.
 __device__ __forceinline__ Sf norm29(Sf a) {
-    uint32_t sh;
-    asm("bfind.shiftamt.s32 %0, %1;" : "=r"(sh) : "r"((int)(a.m >> 32)));
-    const int n = (int)min(sh, 31u) - 2;
+    const int n = (int)min((uint32_t)lead_shift32((int)(a.m >> 32)), 31u) - 2;
     return Sf{a.m << n, a.e - n};
 }
 // An ordinary double (zero and subnormal numbers count as numbers near 2^-1022;
@@ -166,21 +190,17 @@ __device__ __forceinline__ unsigned long long lead64(long long a, int& n) {
     const long long sg = a >> 63;
     const unsigned long long u = (unsigned long long)((a ^ sg) - sg);
     n = __clzll((long long)u);
-    unsigned long long v;
-    asm("shl.b64 %0, %1, %2;" : "=l"(v) : "l"(u), "r"(n));
-    return v;
+    return shl64u(u, n);
 }
-// 1 / a, to about 2^-60 of itself; bad is raised for zero.  x = |a| scaled to
-// [1/2, 1); y0 = 1 / x from the FP32 approximation as an integer of 31 bits, e = 1 -
-// x y0 to 62 places (below 2^-22), y0 (1 + e + e^2).  An FP64 Newton step took
-// three operations of the FP64 pipe and two conversions.
+// 1 / a, within 2^-59.9 of itself, also from a start one ulp off; bad is raised for
+// zero.  x = |a| scaled to [1/2, 1); y0 = 1 / x from the FP32 approximation as an integer
+// of 31 bits, e = 1 - x y0 to 62 places (below 2^-22), y0 (1 + e + e^2).  An FP64 Newton
+// step took three operations of the FP64 pipe and two conversions.
 __device__ __forceinline__ Sf rcp(Sf a, bool& bad) {
     int n;
     const unsigned long long u = lead64(a.m, n);  // x 2^64
     const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
-    float f;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rn(uh)));
-    const uint32_t y0 = min(__float2uint_rn(f * 0x1p62f), 0x7fffffffu);  // y 2^30
+    const uint32_t y0 = min(__float2uint_rn(rcp_start(__uint2float_rn(uh)) * 0x1p62f), 0x7fffffffu);  // y 2^30
     const long long e = (long long)((1ull << 62) - ((unsigned long long)uh * y0 + __umulhi(ul, y0)));
     const int es = (int)(e >> 10);
     const unsigned long long t = (unsigned long long)(e + (__mulhi(es, es) >> 10)) << 20;
@@ -191,18 +211,16 @@ __device__ __forceinline__ Sf rcp(Sf a, bool& bad) {
     const long long m = (long long)((y - 1) >> 1), sg = a.m >> 63;  // below 2^62 for x = 1/2, too
     return Sf{(m ^ sg) - sg, n - a.e - 125};
 }
-// sqrt(a), a >= 0, to about 2^-59 of itself.  v = a scaled by an even power of two to
-// [1/4, 1); r0 = 1 / sqrt(v) from the FP32 approximation, e = 1 - v r0^2, s = v r0
-// (1 + e / 2 + 3 e^2 / 8).
+// sqrt(a), a >= 0, within 2^-58.8 of itself, also from a start one ulp off.  v = a
+// scaled by an even power of two to [1/4, 1); r0 = 1 / sqrt(v) from the FP32
+// approximation, e = 1 - v r0^2, s = v r0 (1 + e / 2 + 3 e^2 / 8).
 __device__ __forceinline__ Sf root(Sf a) {
     int n;
     unsigned long long v = lead64(a.m, n);
     const int ex = 64 - n + a.e, odd = ex & 1;  // a = (v 2^-64) 2^ex
     v >>= odd;
     const uint32_t vh = (uint32_t)(v >> 32), vl = (uint32_t)v;
-    float f;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rn(vh)));
-    const uint32_t r0 = min(__float2uint_rn(f * 0x1p46f), 0x7fffffffu);  // 2^30 / sqrt(v)
+    const uint32_t r0 = min(__float2uint_rn(rsqrt_start(__uint2float_rn(vh)) * 0x1p46f), 0x7fffffffu);  // 2^30 / sqrt(v)
     const unsigned long long w = (unsigned long long)r0 * r0;          // 2^60 / v
     const uint32_t wh = (uint32_t)(w >> 32), wl = (uint32_t)w;
     const unsigned long long vw = (unsigned long long)vh * wh + __umulhi(vh, wl) + __umulhi(vl, wh);
@@ -210,7 +228,8 @@ __device__ __forceinline__ Sf root(Sf a) {
     const int es = (int)(e >> 8);
     const long long t = (e >> 1) + ((__mulhi(es, es) * 3) >> 15);
     const long long s0 = (long long)((unsigned long long)vh * r0 + __umulhi(vl, r0));  // sqrt(v) 2^62
-    const long long s = min(s0 + (mul62(s0 - 1, t << 22) >> 20), (1ll << 62) - 1);
+    // (s0 passes 2^62 where v is just below 1 and r0 above 1 / sqrt(v): halved for the product)
+    const long long s = min(s0 + (mul62(s0 >> 1, t << 23) >> 20), (1ll << 62) - 1);
     return a.m == 0 ? Sf{0ll, kZeroE} : Sf{s, ((ex + odd) >> 1) - 62};
 }
 // v / 3 and v / 9, within 1.5 units: v times 2^64 / 3 (or 9), words H and L, without the
