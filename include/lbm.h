@@ -355,6 +355,12 @@ int lbm_diag_reduce_noalloc(const double* d_fields, int32_t nz, int32_t nr, int3
  * `stream`.  The context stays usable: the kernel leaves no work in flight. */
 int lbm_selftest_bounded_wait(int32_t tries, void* stream, int32_t* device_status_word);
 
+/* Whether a read of `bytes` bytes into host_out (phi alone, or all five fields) is
+ * stored there by the kernel itself: 1 where one page-locked allocation or registration
+ * that the GPU may write holds the whole range at an 8-byte aligned address, else 0 (the
+ * read goes through a copy).  Looks the address up only; touches no memory. */
+int lbm_selftest_direct_read(double* host_out, int64_t bytes);
+
 /* Measured throughput of the GPU's FP64 pipe (no paper counterpart: the
  * denominator of the FP64 step's arithmetic roofline, whose step is bound by
  * that pipe rather than by memory).  Launches 4 blocks of 256 threads per SM,

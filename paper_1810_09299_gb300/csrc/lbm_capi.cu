@@ -692,20 +692,35 @@ void touch_pages(void* dst, size_t bytes) {
     p[bytes - 1] = 0;
 }
 
-// The address under which kernels store into page-locked host memory, or null for
-// any other memory, and for a range that is not page-locked to its end or not aligned.
+// The address under which kernels store into page-locked host memory, or null for any
+// other memory and where no single allocation or registration that the GPU may write
+// holds the whole range: its two ends may lie in two registrations with pages between
+// them that the GPU cannot reach.  One driver query answers all of it.
 double* mapped_doubles(double* host, size_t bytes) {
     if (((uintptr_t)host & (sizeof(double) - 1)) != 0) return nullptr;
-    cudaPointerAttributes a{}, b{};
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
-        cudaPointerGetAttributes(&b, (char*)host + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
+    static const auto query = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return (PFN_cuPointerGetAttributes_v7000)fn;
+    }();
+    if (!query) return nullptr;
+    unsigned type = 0, managed = 0, access = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,      CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_POINTER,   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE,       CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
+    void* into[] = {&type, &managed, &dev, &start, &size, &access};
+    if (query(6, what, into, (CUdeviceptr)host) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed ||
+        access != CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE || dev == 0 || dev < start || dev - start > size ||
+        size - (dev - start) < bytes)
         return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-        (char*)b.devicePointer - (char*)a.devicePointer != (ptrdiff_t)bytes - 1)
-        return nullptr;
-    return (double*)a.devicePointer;
+    return (double*)dev;
 }
 
 int check_case(lbm_sim* h, int icase) {
@@ -885,6 +900,10 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
         b = e > b ? e : b + 1;
     }
     return finish_status(h);
+}
+
+int lbm_selftest_direct_read(double* host_out, int64_t bytes) {
+    return bytes > 0 && mapped_doubles(host_out, (size_t)bytes) != nullptr;
 }
 
 int lbm_get_fields(lbm_handle* h, int32_t mask, double* host_out) { return lbm_case_get_fields(h, 0, mask, host_out); }
