@@ -451,9 +451,9 @@ int row_shape(const lbm_sim* h) {
 // The launch shape a handle starts with (lbm_set_variant, lbm_autotune and the
 // results know no difference).  us a step in the captured graph:
 //   4-row tiles (2) instead of 8-row tiles (0)
-//     where those leave half the SMs empty, FP64 and bfloat16 (a 64 x 128 drop, 32
-//     tiles of 8 rows: 9.2 -> 7.8 and 3.02 -> 2.77; FP32 2.32 and 2.45, FP16 2.90
-//     either way), and where some SMs would hold two of them, most one and taller
+//     where those leave half the SMs empty, but in FP16 (a 64 x 128 drop, 32 tiles of
+//     8 rows: FP64 9.2 -> 7.8, bfloat16 3.02 -> 2.75, FP32 2.50 -> 2.38, FP16 2.83 and
+//     2.95), and where some SMs would hold two of them, most one and taller
 //     tiles do not help (row_shape's figures).  128 tiles (128 x 256) and 250 (150 x
 //     400) take 8 rows: FP32 2.52 against 2.77 and 3.41 against 3.66.
 //   FP16, packed pairs of nodes (7) from 3/2 tiles of 16 rows per SM on: 64 x 180
@@ -466,7 +466,7 @@ int default_variant(const lbm_sim* h) {
     const int sms = sm_count(h);
     if (sms == 0 || h->row_shape != 0) return 0;
     const int t8 = h->ntiles[0];
-    if (2 * t8 <= sms && (h->precision == LBM_FP64 || h->precision == LBM_MIX_BF16)) return 2;
+    if (2 * t8 <= sms && h->precision != LBM_MIX_FP16) return 2;
     if (t8 > sms && 3 * t8 <= 4 * sms) return 2;
     if (h->precision == LBM_MIX_FP16 && 2 * h->ntiles[7] >= 3 * sms) return 7;
     if (h->precision == LBM_FP32 && h->ntiles[5] >= 6 * sms) return 5;
@@ -587,17 +587,6 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
         rc = upload_tiles(h, t, &h->tiles_d[v], true);
     }
     if (rc == LBM_OK) h->variant = default_variant(h);
-    // (the grids whose variant 0 may take them; the first call loads the kernels)
-    if (rc == LBM_OK && h->ntiles[h->row_shape] <= 2 * sm_count(h)) {
-        cudaError_t e = cudaSuccess;
-        switch (h->precision) {
-            case LBM_FP64: e = prepare_step_f64(); break;
-            case LBM_FP32: e = prepare_step_f32(); break;
-            case LBM_MIX_FP16: e = prepare_step_h16(); break;
-            default: e = prepare_step_b16(); break;
-        }
-        if (e != cudaSuccess) rc = LBM_ERR_CUDA;
-    }
     for (int c = 0; c < n && rc == LBM_OK; ++c) {
         std::vector<TileDev> t = make_tiles(h->cases, 8, c);
         TileDev* d = nullptr;

@@ -1131,34 +1131,31 @@ __device__ __forceinline__ Dest destination(int k, int j, int nr, int nz, int zp
 // 2.95 -> 2.70, 128 x 256 3.02 -> 2.76, 200 x 600 5.29 -> 5.03, 256 x 1024
 // 8.43 -> 8.20; launched one by one 5.2 -> 2.9, 6.6 -> 3.0, 8.9 -> 5.5, 11.1 -> 9.0.
 // pdl_trigger lets the next launch start before this CTA ends.  At a kernel's
-// start that is slower by itself: the next step's CTAs gather on few SMs (128 x
-// 256 drop 3.44 us in FP32, 16.1 against 11.4 in FP64).  So the one-node kernel uses
-// it only with a launch that keeps the SMs even (launch_step_spread), the
-// packed kernel after its window barrier, with more tiles than fit at once, and the
-// kernels of a read at their start.
+// start that is slower: the next step's CTAs gather on few SMs (128 x 256 drop 3.44 us
+// in FP32, 16.1 against 11.4 in FP64).  Dynamic shared memory that leaves an SM room for no
+// more CTAs than the grid needs keeps the SMs even and gained a single handle 2.56 ->
+// 2.38 us, but those places are then taken from every other handle: eight 128 x 256
+// FP32 handles on as many streams took 1.70 us a step each instead of 0.78 (four 1.70
+// and 1.20).  So the one-node kernel does not use it, the packed kernel
+// does after its window barrier, with more tiles than fit at once, and the kernels of
+// a read at their start.
 // Without the attribute both do nothing.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A launch that may overlap the end of the launch before it on the stream
 // (programmatic stream serialisation).
 template <class... P, class... A>
-void launch_pdl_dyn(void (*kernel)(P...), int grid, dim3 block, size_t dyn, cudaStream_t st, A... args) {
+void launch_pdl(void (*kernel)(P...), int grid, dim3 block, cudaStream_t st, A... args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = dyn;
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
-template <class... P, class... A>
-void launch_pdl(void (*kernel)(P...), int grid, dim3 block, cudaStream_t st, A... args) {
-    launch_pdl_dyn(kernel, grid, block, 0, st, args...);
 }
 
 // ---------------------------------------------------------------- TMA / mbarrier

@@ -39,7 +39,6 @@ struct DeviceState {
 };
 
 #define AXILBM_DECLARE(NAME)                                                                                       \
-    cudaError_t prepare_step_##NAME();                                                                             \
     cudaError_t launch_step_##NAME(const DeviceState& D, int parity, int variant, const TileDev* tiles, int ntiles, \
                                    cudaStream_t st);                                                               \
     cudaError_t launch_fields_##NAME(const DeviceState& D, int parity, const TileDev* tiles, int ntiles,            \

@@ -726,8 +726,7 @@ __device__ __forceinline__ void step_tile(const StateDev<Codec>& S, TileShared<C
 }
 
 // One time step for every node of every tile in `tiles`: one CTA per tile.
-// EARLY: the next step's CTAs take their places while this one runs.
-template <class Codec, int BZ, int RM, int MINB = step_min_blocks<Codec, BZ, RM>(), bool EARLY = false>
+template <class Codec, int BZ, int RM, int MINB = step_min_blocks<Codec, BZ, RM>()>
 __global__ void __launch_bounds__(kTR * BZ, MINB)
 step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles, StateDev<Codec> S,
             const CUtensorMap* __restrict__ maps, int map_set, int parity, int ntiles, int ahead) {
@@ -737,7 +736,6 @@ step_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles
     // this thread's word of the case record leaves with the loads of the window phase
     int32_t cw = 0;
     if (q < kCaseWords<typename Codec::Real>) cw = reinterpret_cast<const int32_t*>(cases + g.c)[q];
-    if constexpr (EARLY) pdl_trigger();
     pdl_wait();
     // L2 prefetch of the blocks of the tile one resident wave ahead (a CTA
     // that will start about when this one ends): one tensor prefetch, issued
@@ -1703,64 +1701,6 @@ void launch_tma(int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* t
         cs, tiles, ntiles, S, (const CUtensorMap*)D.tmaps, BZ == 8 ? 0 : 1, parity, D.status);
 }
 
-// Grids of at most two tiles per SM, in one wave: the launch after a step starts
-// when that step's CTAs have started (EARLY), and each CTA asks for so much shared
-// memory that an SM takes no more of them than the grid needs.  Without the second
-// the next step's CTAs gather on the SMs that are free first; with it they start as
-// CTAs end, one for one, and their launch and first loads are hidden.  us a step,
-// without and with:
-//                          FP32         FP16         bfloat16     FP64
-//   64 x 128  (32 tiles)   2.50 2.32    2.83 2.82    3.02 3.09    9.22 9.23
-//   128 x 256 (128)        2.56 2.38    2.96 2.91    3.09 3.21    9.36 9.29
-//   101 x 333 (136 of 10)  2.82 2.63    3.14 3.14    3.21 3.19    10.97 10.89
-//   150 x 300 (150 of 10)  2.89 2.71    3.28 3.18    3.34 3.28    11.02 10.91
-//   150 x 400 (250)        3.40 3.33    3.65 3.52    3.92 4.00    14.30 14.26
-//   200 x 400 (280 of 10)  3.85 3.76    3.99 3.89    4.12 4.05    20.63 20.59
-// (3.45 tiles per SM, 200 x 600: 4.86 and 5.45.)  So FP32 and FP16 storage only.  The
-// trigger after the wait or after the window barrier gains nothing (2.57, 2.56).
-constexpr size_t kSmBytes = 228 * 1024, kCtaReserved = 1024;  // shared memory of an SM, of it per CTA for the system
-template <class Codec, int RM>
-constexpr bool kSpread = sizeof(typename Codec::Real) == 4 && (sizeof(typename Codec::PT) == 4 || Codec::kGrid) &&
-                         RM != kRatesGeneral;
-template <class Codec, int BZ, int RM>
-constexpr auto spread_kernel = step_kernel<Codec, BZ, RM, step_min_blocks<Codec, BZ, RM>(), true>;
-template <class Codec, int BZ, int RM>
-constexpr size_t spread_bytes(int per_sm) {  // per_sm CTAs fit an SM, one more does not
-    return kSmBytes / (per_sm + 1) + kCtaReserved - sizeof(TileShared<Codec, BZ, RM>);
-}
-template <class Codec, int BZ, int RM>
-bool launch_step_spread(int ntiles, int sms, cudaStream_t st, const CaseDev* cs, const TileDev* tiles,
-                        const StateDev<Codec>& S, int parity) {
-    if constexpr (kSpread<Codec, RM>) {
-        static_assert(spread_bytes<Codec, BZ, RM>(1) + sizeof(TileShared<Codec, BZ, RM>) <= kSmBytes / 2 + kCtaReserved &&
-                          2 * (spread_bytes<Codec, BZ, RM>(2) + sizeof(TileShared<Codec, BZ, RM>) + kCtaReserved) <= kSmBytes,
-                      "one and two CTAs fit");
-        if (ntiles > 2 * sms) return false;
-        launch_pdl_dyn(spread_kernel<Codec, BZ, RM>, ntiles, dim3(kTR, BZ),
-                               spread_bytes<Codec, BZ, RM>(ntiles > sms ? 2 : 1), st, cs, tiles, S,
-                               (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
-        return true;
-    }
-    return false;
-}
-// Lets this device's spread kernels have that much shared memory (when a handle is created).
-template <class Codec>
-cudaError_t prepare_step_t() {
-    cudaError_t e = cudaSuccess;
-    auto allow = [&](auto* kernel, size_t bytes) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    };
-    if constexpr (kSpread<Codec, kRatesPaper>) {
-        allow(spread_kernel<Codec, 8, kRatesPaper>, spread_bytes<Codec, 8, kRatesPaper>(1));
-        allow(spread_kernel<Codec, 10, kRatesPaper>, spread_bytes<Codec, 10, kRatesPaper>(1));
-        allow(spread_kernel<Codec, 12, kRatesPaper>, spread_bytes<Codec, 12, kRatesPaper>(1));
-        allow(spread_kernel<Codec, 8, kRatesPaperRaw>, spread_bytes<Codec, 8, kRatesPaperRaw>(1));
-        allow(spread_kernel<Codec, 10, kRatesPaperRaw>, spread_bytes<Codec, 10, kRatesPaperRaw>(1));
-        allow(spread_kernel<Codec, 12, kRatesPaperRaw>, spread_bytes<Codec, 12, kRatesPaperRaw>(1));
-    }
-    return e;
-}
-
 template <class Codec, int RM>
 void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* tiles,
                        const StateDev<Codec>& S, const DeviceState& D, int parity) {
@@ -1775,7 +1715,6 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
     const CUtensorMap* maps = (const CUtensorMap*)D.tmaps;
     switch (variant) {
         case 0:
-            if (launch_step_spread<Codec, 8, RM>(ntiles, sms, st, cs, tiles, S, parity)) break;
             if constexpr (sizeof(typename Codec::Real) == 8 && RM != kRatesGeneral) {
                 if (ntiles >= 6 * sms) {
                     launch_pdl(step_kernel<Codec, 8, RM, kF64Full>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0,
@@ -1799,14 +1738,12 @@ void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* 
             launch_pdl(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
             break;
         case 8:  // (one wave: nothing to prefetch)
-            if (launch_step_spread<Codec, 10, RM>(ntiles, sms, st, cs, tiles, S, parity)) break;
-            if constexpr (RM != kRatesGeneral && !kSpread<Codec, RM>)
+            if constexpr (RM != kRatesGeneral)
                 launch_pdl(step_kernel<Codec, 10, RM>, ntiles, dim3(kTR, 10), st, cs, tiles, S,
                                    (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
             break;
         case 9:
-            if (launch_step_spread<Codec, 12, RM>(ntiles, sms, st, cs, tiles, S, parity)) break;
-            if constexpr (RM != kRatesGeneral && !kSpread<Codec, RM>)
+            if constexpr (RM != kRatesGeneral)
                 launch_pdl(step_kernel<Codec, 12, RM>, ntiles, dim3(kTR, 12), st, cs, tiles, S,
                                    (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
             break;
@@ -1900,7 +1837,6 @@ cudaError_t launch_set_state_t(const DeviceState& D, int parity, const CaseDev& 
 
 #define AXILBM_INSTANTIATE(NAME, CODEC)                                                                          \
     namespace axilbm {                                                                                           \
-    cudaError_t prepare_step_##NAME() { return prepare_step_t<CODEC>(); }                                        \
     cudaError_t launch_step_##NAME(const DeviceState& D, int parity, int variant, const TileDev* tiles,          \
                                    int ntiles, cudaStream_t st) {                                                \
         return launch_step_t<CODEC>(D, parity, variant, tiles, ntiles, st);                                      \
