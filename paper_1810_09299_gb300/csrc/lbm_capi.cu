@@ -422,11 +422,11 @@ int sm_count(const lbm_sim* h) {
 // to one CTA per SM and 8 rows do not, since a small grid's step lasts as long as
 // the SM with the most warps.  us a step, 8 rows, 4 rows and 10 or 12 rows:
 //                       FP64               FP32             FP16             bfloat16
-//   101 x 333 (168, 10) 13.8  11.9 10.9    3.15 3.09 2.83   3.56 3.40 3.15   3.92 3.45 3.20
-//   150 x 300 (190, 10) 14.1  12.0 11.0    3.34 3.28 2.88   3.44 3.59 3.27   3.92 3.53 3.32
-//   128 x 448 (224, 12) 13.9  11.9 11.9    3.21 3.21 3.09   3.59 3.46 3.20   3.85 3.53 3.27
+//   101 x 333 (168, 10) 13.8  11.9 10.8    3.15 3.08 2.82   3.56 3.34 3.14   3.92 3.46 3.15
+//   150 x 300 (190, 10) 14.1  12.1 10.9    3.34 3.21 2.82   3.44 3.59 3.28   3.92 3.53 3.27
+//   128 x 448 (224, 12) 13.9  11.9 11.9    3.21 3.27 3.02   3.59 3.52 3.15   3.85 3.59 3.21
 //   150 x 400 (250, 10) 14.2  14.5 20.7    3.41 3.57 3.84   3.65 3.91 3.96   3.92 3.98 4.10
-//   200 x 400 (350, 10) 20.7  19.6 20.9    4.11 3.97 3.85   4.37 4.30 3.98   4.80 4.37 4.11
+//   200 x 400 (350, 10) 20.7  19.6 20.9    4.11 3.98 3.79   4.37 4.30 4.03   4.80 4.42 4.11
 // (in brackets the tiles of 8 rows on 152 SMs and the taller tiles' rows).  So
 // 10 rows also where two CTAs per SM hold them and not the 8-row ones, but in
 // FP64, whose 10-row CTAs have an SM's registers to themselves.  Two of those

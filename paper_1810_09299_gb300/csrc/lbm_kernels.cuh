@@ -139,6 +139,12 @@ __device__ __forceinline__ void ring_cell(int q, int& a, int& b) {
 // that have an SM each take 136 registers (kF64Few CTAs; with 4 at 128: 64 x 128 7.94
 // against 7.76, raw moments 8.22 against 7.81; 200 x 600, 1050 tiles, 26.7 against 31.1).
 constexpr int kF64Full = 3, kF64Few = 3;
+// Tiles of 10 and 12 rows (row_shape in lbm_capi.cu) have an SM or half of one to
+// themselves, but handles on other streams may want the rest of it: as many warps per
+// SM as 8-row tiles, as far as the registers go.  With 2 CTAs (102 and 80 registers)
+// eight 150 x 300 handles took 1.52 us a step each in FP32, 1.47 in FP16 and 1.57 in
+// bfloat16; now 1.10, 1.22 and 1.31 (8-row tiles 1.13, 1.21 and 1.22), one handle alone as
+// before.  bfloat16 with 4 CTAs spills (3.23 -> 3.59 alone).
 template <class Codec, int BZ, int RM>
 constexpr int step_min_blocks() {
     constexpr int bz8 = Codec::kGrid ? AXILBM_GRID16_CTAS
@@ -146,7 +152,7 @@ constexpr int step_min_blocks() {
                             ? 4
                             : (sizeof(typename Codec::PT) == 2 ? AXILBM_STEP16_CTAS : 5);
     return sizeof(typename Codec::Real) == 8 ? (RM == kRatesGeneral ? 1 : (BZ > 8 ? 1 : (BZ == 4 ? 4 : 2)))
-           : BZ == 10 || BZ == 12 ? 2 : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
+           : BZ == 10 || BZ == 12 ? (sizeof(typename Codec::PT) == 4 && BZ == 10 ? 4 : 3) : RM != kRatesGeneral ? (BZ >= 16 ? 2 : (BZ >= 8 ? bz8 : 8))
                 : (BZ >= 16 ? 1 : (BZ >= 8 ? AXILBM_GENERAL_CTAS : 2 * AXILBM_GENERAL_CTAS));
 }
 

@@ -9,10 +9,11 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec", ["fp32", "mix_fp16"])
-@pytest.mark.parametrize("nr,nz", [(64, 128), (128, 256)])
+@pytest.mark.parametrize("nr,nz", [(64, 128), (128, 256), (150, 300)])
 def test_eight_handles_share_the_sms(nr, nz, prec):
-    """Each grid has at most one tile per SM, and an SM holds the tiles of four handles or more:
-    eight handles take two rounds of places, each as long as a step alone or twice that."""
+    """Each grid has at most one tile per SM (150 x 300: of 10 rows), and an SM holds the tiles of three
+    handles or more: eight handles take two rounds of places, each as long as a step alone or twice
+    that, or three rounds."""
     torch = pytest.importorskip("torch")
 
     def us_per_step(n):
