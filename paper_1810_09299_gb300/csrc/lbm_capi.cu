@@ -411,13 +411,6 @@ bool encode_tensor_maps(lbm_sim* h, std::vector<CUtensorMap>& maps) {
     return true;
 }
 
-int sm_count(const lbm_sim* h) {
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess && sms > 0) return sms;
-    cudaGetLastError();
-    return 0;
-}
-
 // The tile height of variant 0: 8 rows, or 10 (shape 8) or 12 (9) where these come
 // to one CTA per SM and 8 rows do not, since a small grid's step lasts as long as
 // the SM with the most warps.  us a step, 8 rows, 4 rows and 10 or 12 rows:
@@ -435,7 +428,7 @@ int sm_count(const lbm_sim* h) {
 // pairs of FP32 operations in a block of 10 or 12 warps, and the results' last bits
 // would depend on the grid.
 int row_shape(const lbm_sim* h) {
-    const int sms = sm_count(h);
+    const int sms = h->D.sms;
     auto tiles = [&](int tz) {
         int64_t t = 0;
         for (const CaseDev& C : h->cases) t += (int64_t)((C.nz + tz - 1) / tz) * (C.pitch / 32);
@@ -463,8 +456,8 @@ int row_shape(const lbm_sim* h) {
 //     256 x 1024 (512 tiles) 8.27 against 8.81, 8 cases (1100) 15.8 -> 15.2, 512 cases
 //     726 -> 711.
 int default_variant(const lbm_sim* h) {
-    const int sms = sm_count(h);
-    if (sms == 0 || h->row_shape != 0) return 0;
+    const int sms = h->D.sms;
+    if (h->row_shape != 0) return 0;
     const int t8 = h->ntiles[0];
     if (2 * t8 <= sms && h->precision != LBM_MIX_FP16) return 2;
     if (t8 > sms && 3 * t8 <= 4 * sms) return 2;
@@ -488,6 +481,10 @@ int create_impl(const lbm_params* cases, int32_t n, void* stream, lbm_handle** o
         cudaGetLastError();
         delete h;
         return LBM_ERR_CUDA;
+    }
+    if (cudaDeviceGetAttribute(&h->D.sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || h->D.sms < 1) {
+        cudaGetLastError();
+        h->D.sms = 1;
     }
     h->stream = (cudaStream_t)stream;
     h->precision = cases[0].precision;

@@ -35,6 +35,7 @@ struct DeviceState {
     const void* tmaps;  // CUtensorMap[ncases][2 tile heights][kMapsPerCase] in device memory
     const double* cols;  // FP64 handles: constants of the columns 0 .. ncols - 1 (ColTab64 of lbm_f64.cuh)
     int ncols;
+    int sms;            // SMs of the handle's device (1 if unknown)
     int* status;        // device status word: nonzero after a bounded wait gave up
 };
 

@@ -1708,78 +1708,65 @@ void launch_tma(int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* t
 }
 
 template <class Codec, int RM>
-void launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* tiles,
-                       const StateDev<Codec>& S, const DeviceState& D, int parity) {
-    // prefetch distance: the CTAs resident at once (SMs x CTAs per SM)
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-    }
-    const CUtensorMap* maps = (const CUtensorMap*)D.tmaps;
+cudaError_t launch_step_rates(int variant, int ntiles, cudaStream_t st, const CaseDev* cs, const TileDev* tiles,
+                              const StateDev<Codec>& S, const DeviceState& D, int parity) {
+    using Real = typename Codec::Real;
+    constexpr bool k64 = sizeof(Real) == 8;
+    const CUtensorMap* const maps = (const CUtensorMap*)D.tmaps;
+    // `ctas` resident at once per SM: the L2 prefetch reaches that many tiles ahead (0: a
+    // grid of one wave, nothing to prefetch); map_set: the tensor maps of the tile height
+    auto launch = [&](auto* kernel, int warps, int ctas, int map_set) {
+        launch_pdl(kernel, ntiles, dim3(kTR, (unsigned)warps), st, cs, tiles, S, ctas ? maps : nullptr, map_set, parity,
+                   ntiles, kPrefetchQuarters * D.sms * ctas / 4);
+    };
+    auto tall = [&] { launch(step_kernel<Codec, 16, RM>, 16, step_min_blocks<Codec, 16, RM>(), 1); };
+    auto two_nodes = [&] {
+        if constexpr (k64) tall();
+        else launch(step_kernel_seq2<Codec, 8, RM>, 8, seq2_min_blocks<Codec, 8, RM>(), 1);
+    };
     switch (variant) {
         case 0:
-            if constexpr (sizeof(typename Codec::Real) == 8 && RM != kRatesGeneral) {
-                if (ntiles >= 6 * sms) {
-                    launch_pdl(step_kernel<Codec, 8, RM, kF64Full>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0,
-                                       parity, ntiles, kPrefetchQuarters * sms * kF64Full / 4);
+            if constexpr (k64 && RM != kRatesGeneral) {
+                if (ntiles >= 6 * D.sms) {
+                    launch(step_kernel<Codec, 8, RM, kF64Full>, 8, kF64Full, 0);
                     break;
                 }
             }
-            launch_pdl(step_kernel<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 8, RM>() / 4);
+            launch(step_kernel<Codec, 8, RM>, 8, step_min_blocks<Codec, 8, RM>(), 0);
             break;
-        case 1:
-            launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
-            break;
+        case 1: tall(); break;
         case 2:
-            if constexpr (sizeof(typename Codec::Real) == 8 && RM != kRatesGeneral) {
-                if (ntiles <= sms) {
-                    launch_pdl(step_kernel<Codec, 4, RM, kF64Few>, ntiles, dim3(kTR, 4), st, cs, tiles, S,
-                               (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
+            if constexpr (k64 && RM != kRatesGeneral) {
+                if (ntiles <= D.sms) {
+                    launch(step_kernel<Codec, 4, RM, kF64Few>, 4, 0, 0);
                     break;
                 }
             }
-            launch_pdl(step_kernel<Codec, 4, RM>, ntiles, dim3(kTR, 4), st, cs, tiles, S, maps, 0, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 4, RM>() / 4);
-            break;
-        case 8:  // (one wave: nothing to prefetch)
-            if constexpr (RM != kRatesGeneral)
-                launch_pdl(step_kernel<Codec, 10, RM>, ntiles, dim3(kTR, 10), st, cs, tiles, S,
-                                   (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
-            break;
-        case 9:
-            if constexpr (RM != kRatesGeneral)
-                launch_pdl(step_kernel<Codec, 12, RM>, ntiles, dim3(kTR, 12), st, cs, tiles, S,
-                                   (const CUtensorMap*)nullptr, 0, parity, ntiles, 0);
+            launch(step_kernel<Codec, 4, RM>, 4, step_min_blocks<Codec, 4, RM>(), 0);
             break;
         case 3: launch_tma<Codec, 8, RM>(ntiles, st, cs, tiles, S, D, parity); break;
         case 4: launch_tma<Codec, 16, RM>(ntiles, st, cs, tiles, S, D, parity); break;
-        case 5:
-            if constexpr (sizeof(typename Codec::Real) == 4)
-                launch_pdl(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
-            else
-                launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
-            break;
+        case 5: two_nodes(); break;
         case 7:
             if constexpr (Codec::kGrid)
-                launch_pdl(ntiles > sms * AXILBM_PACK2_CTAS ? step_kernel_pack2<Codec, RM, true>
-                                                                    : step_kernel_pack2<Codec, RM, false>,
-                                   ntiles, dim3(kTR, 8), st, cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps,
-                                   parity, ntiles, kPrefetchQuarters * sms * AXILBM_PACK2_CTAS / 4);
-            else if constexpr (sizeof(typename Codec::Real) == 4)
-                launch_pdl(step_kernel_seq2<Codec, 8, RM>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM>() / 4);
-            else
-                launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+                launch_pdl(ntiles > D.sms * AXILBM_PACK2_CTAS ? step_kernel_pack2<Codec, RM, true>
+                                                              : step_kernel_pack2<Codec, RM, false>,
+                           ntiles, dim3(kTR, 8), st, cs, reinterpret_cast<const TileGeo*>(tiles + ntiles), S, maps, parity,
+                           ntiles, kPrefetchQuarters * D.sms * AXILBM_PACK2_CTAS / 4);
+            else two_nodes();
+            break;
+        case 8:
+        case 9:
+            if constexpr (RM == kRatesGeneral) return cudaErrorInvalidConfiguration;  // (row_shape gives none)
+            else if (variant == 8) launch(step_kernel<Codec, 10, RM>, 10, 0, 0);
+            else launch(step_kernel<Codec, 12, RM>, 12, 0, 0);
             break;
         default:
-            if constexpr (sizeof(typename Codec::Real) == 4)
-                launch_pdl(step_kernel_seq2<Codec, 8, RM, true>, ntiles, dim3(kTR, 8), st, cs, tiles, S, maps, 1, parity, ntiles,
-                    kPrefetchQuarters * sms * seq2_min_blocks<Codec, 8, RM, true>() / 4);
-            else
-                launch_pdl(step_kernel<Codec, 16, RM>, ntiles, dim3(kTR, 16), st, cs, tiles, S, maps, 1, parity, ntiles, kPrefetchQuarters * sms * step_min_blocks<Codec, 16, RM>() / 4);
+            if constexpr (k64) tall();
+            else launch(step_kernel_seq2<Codec, 8, RM, true>, 8, seq2_min_blocks<Codec, 8, RM, true>(), 1);
             break;
     }
+    return cudaGetLastError();
 }
 
 template <class Codec>
@@ -1788,11 +1775,11 @@ cudaError_t launch_step_t(const DeviceState& D, int parity, int variant, const T
     if (ntiles <= 0) return cudaSuccess;
     StateDev<Codec> S = make_state<Codec>(D, parity);
     const CaseDev* cs = (const CaseDev*)D.cases;
-    if (D.rate_mode == kRatesPaper) launch_step_rates<Codec, kRatesPaper>(variant, ntiles, st, cs, tiles, S, D, parity);
-    else if (D.rate_mode == kRatesPaperRaw)
-        launch_step_rates<Codec, kRatesPaperRaw>(variant, ntiles, st, cs, tiles, S, D, parity);
-    else launch_step_rates<Codec, kRatesGeneral>(variant, ntiles, st, cs, tiles, S, D, parity);
-    return cudaGetLastError();
+    if (D.rate_mode == kRatesPaper)
+        return launch_step_rates<Codec, kRatesPaper>(variant, ntiles, st, cs, tiles, S, D, parity);
+    if (D.rate_mode == kRatesPaperRaw)
+        return launch_step_rates<Codec, kRatesPaperRaw>(variant, ntiles, st, cs, tiles, S, D, parity);
+    return launch_step_rates<Codec, kRatesGeneral>(variant, ntiles, st, cs, tiles, S, D, parity);
 }
 
 template <class Codec>
