@@ -355,6 +355,10 @@ int lbm_diag_reduce_noalloc(const double* d_fields, int32_t nz, int32_t nr, int3
  * `stream`.  The context stays usable: the kernel leaves no work in flight. */
 int lbm_selftest_bounded_wait(int32_t tries, void* stream, int32_t* device_status_word);
 
+/* The same on the handle's own status word: its next read is that of a handle whose
+ * staged step gave up (LBM_ERR_TIMEOUT, the caller's memory untouched). */
+int lbm_selftest_handle_wait(lbm_handle* h, int32_t tries);
+
 /* Whether a read of `bytes` bytes into host_out (phi alone, or all five fields) is
  * stored there by the kernel itself: 1 where one page-locked allocation or registration
  * that the GPU may write holds the whole range at an 8-byte aligned address, else 0 (the

@@ -6,6 +6,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
+#include <errno.h>
+#include <sys/mman.h>
 #include <unistd.h>
 
 #include <algorithm>
@@ -127,6 +129,7 @@ struct lbm_sim {
     int variant = 0;
     int row_shape = 0;  // what variant 0 runs: itself or a shape of taller tiles
     int sticky = LBM_OK;
+    bool staged = false;  // a TMA-staged step ran since the status word was last seen to be zero
     int64_t launches = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_variant = -1;
@@ -171,16 +174,15 @@ cudaError_t launch_step_any(lbm_sim* h, int parity, int variant, cudaStream_t st
 }
 
 // The fields of case icase: all five, or phi alone, into h->fields or out.
-cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st, bool phi_only = false,
-                              int* status_out = nullptr, double* out = nullptr) {
+cudaError_t launch_fields_any(lbm_sim* h, int icase, cudaStream_t st, bool phi_only = false, double* out = nullptr) {
     const TileDev* t = h->ftiles_d[icase];
     const int n = h->nftiles[icase];
     if (!out) out = h->fields;
     switch (h->precision) {
-        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, out, status_out, st);
-        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, out, status_out, st);
-        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, out, status_out, st);
-        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, out, status_out, st);
+        case LBM_FP64: return launch_fields_f64(h->D, h->parity, t, n, phi_only, out, st);
+        case LBM_FP32: return launch_fields_f32(h->D, h->parity, t, n, phi_only, out, st);
+        case LBM_MIX_FP16: return launch_fields_h16(h->D, h->parity, t, n, phi_only, out, st);
+        default: return launch_fields_b16(h->D, h->parity, t, n, phi_only, out, st);
     }
 }
 
@@ -637,6 +639,7 @@ int capture_graph(lbm_sim* h) {
 }
 
 int step_direct(lbm_sim* h, int64_t n) {
+    h->staged |= n > 0 && kVariantTMA[h->variant];
     for (int64_t s = 0; s < n; ++s) {
         cudaError_t e = launch_step_any(h, h->parity, h->variant, h->stream);
         if (e != cudaSuccess) return cuda_ok(h, e);
@@ -646,9 +649,10 @@ int step_direct(lbm_sim* h, int64_t n) {
     return LBM_OK;
 }
 
-// Device status word: set by a bounded wait that gave up (TMA-staged step).  A
-// read-back's last kernel also stores it here (pinned memory), and the call
-// looks at it after the one synchronisation that ends it.
+// Device status word: set by a bounded wait that gave up (TMA-staged step).  The last
+// kernel of the records and of the drops also stores it here (pinned memory), and the
+// call looks at it after the one synchronisation that ends it, before it writes to the
+// caller's memory.
 int* status_host(lbm_sim* h) { return (int*)(h->host_small + 12); }
 int finish_status(lbm_sim* h) {
     const int rc = cuda_ok(h, cudaStreamSynchronize(h->stream));
@@ -657,13 +661,24 @@ int finish_status(lbm_sim* h) {
         h->sticky = LBM_ERR_TIMEOUT;
         return LBM_ERR_TIMEOUT;
     }
+    h->staged = false;
     return LBM_OK;
 }
+// The same before a read whose copy or kernel writes to the caller's memory itself: a
+// wait of its own, and only after steps that can raise the word.
+int check_status(lbm_sim* h) {
+    if (!h->staged) return LBM_OK;
+    const int rc = cuda_ok(h, cudaMemcpyAsync(status_host(h), h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    return rc != LBM_OK ? rc : finish_status(h);
+}
 
-// Write to each page of a pageable host destination before the copy into it:
-// pages that the process has never touched are otherwise mapped one by one
+// Have the pages of a pageable host destination mapped before the copy into it:
+// pages that the process has never written to are otherwise mapped one by one
 // from the GPU's side of the copy (the f, g, aux of a 1024 x 256 case into fresh
-// arrays: 35 ms against 2).  Memory known to CUDA is left alone.
+// arrays: 35 ms against 2).  The bytes keep their values, since the copy may still fail (an
+// atomic OR with zero does so too, but on Arm it faults as a read first: 15 ms); a
+// kernel without MADV_POPULATE_WRITE (before Linux 5.14) leaves it to the copy.  Memory
+// known to CUDA is left alone.
 void touch_pages(void* dst, size_t bytes) {
     cudaPointerAttributes at{};
     if (bytes < kTouchBytes) return;
@@ -672,10 +687,12 @@ void touch_pages(void* dst, size_t bytes) {
         return;
     }
     if (at.type != cudaMemoryTypeUnregistered) return;
-    static const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
-    volatile char* p = (volatile char*)dst;
-    for (size_t o = 0; o < bytes; o += page) p[o] = 0;
-    p[bytes - 1] = 0;
+    constexpr int kPopulateWrite = 23;  // MADV_POPULATE_WRITE
+    static const uintptr_t page = (uintptr_t)std::max(4096l, sysconf(_SC_PAGESIZE));
+    const uintptr_t start = (uintptr_t)dst & ~(page - 1);
+    const int saved = errno;
+    madvise((void*)start, (uintptr_t)dst + bytes - start, kPopulateWrite);
+    errno = saved;
 }
 
 // The address under which kernels store into page-locked host memory, or null for any
@@ -841,6 +858,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
         if (left >= kGraphSteps) {
             rc = capture_graph(h);
             if (rc != LBM_OK) return rc;
+            h->staged |= kVariantTMA[h->variant];
             while (left >= kGraphSteps) {
                 cudaError_t e = cudaGraphLaunch(h->graph, h->stream);
                 if (e != cudaSuccess) return cuda_ok(h, e);
@@ -860,7 +878,8 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
     if (rc != LBM_OK) return rc;
     if (check_case(h, icase) != LBM_OK || !host_out || mask <= 0 || mask > 31) return LBM_ERR_INVALID_ARG;
     if (!h->initialized[icase]) return LBM_ERR_STATE;
-    rc = join_diagnostics(h);
+    rc = check_status(h);
+    if (rc == LBM_OK) rc = join_diagnostics(h);
     if (rc != LBM_OK) return rc;
     const int64_t n = (int64_t)h->prm[icase].nz * h->prm[icase].nr;
     // phi or all five into page-locked memory: stored there by the kernel, without a
@@ -869,9 +888,9 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
     double* direct = nullptr;
     if (mask == LBM_FIELD_PHI || mask == 31)
         direct = mapped_doubles(host_out, (mask == 31 ? 5 : 1) * n * sizeof(double));
-    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI, status_host(h), direct));
+    rc = cuda_ok(h, launch_fields_any(h, icase, h->stream, mask == LBM_FIELD_PHI, direct));
     if (rc != LBM_OK) return rc;
-    if (direct) return finish_status(h);
+    if (direct) return cuda_ok(h, cudaStreamSynchronize(h->stream));
     int64_t slot = 0;
     for (int b = 0; b < 5;) {
         int e = b;  // neighbouring planes leave in one copy
@@ -885,7 +904,14 @@ int lbm_case_get_fields(lbm_handle* h, int32_t icase, int32_t mask, double* host
         }
         b = e > b ? e : b + 1;
     }
-    return finish_status(h);
+    return cuda_ok(h, cudaStreamSynchronize(h->stream));
+}
+
+int lbm_selftest_handle_wait(lbm_handle* h, int32_t tries) {
+    int rc = enter(h);
+    if (rc != LBM_OK) return rc;
+    h->staged = true;
+    return lbm_selftest_bounded_wait(tries, h->stream, h->D.status);
 }
 
 int lbm_selftest_direct_read(double* host_out, int64_t bytes) {

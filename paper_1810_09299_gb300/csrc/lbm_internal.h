@@ -43,7 +43,7 @@ struct DeviceState {
     cudaError_t launch_step_##NAME(const DeviceState& D, int parity, int variant, const TileDev* tiles, int ntiles, \
                                    cudaStream_t st);                                                               \
     cudaError_t launch_fields_##NAME(const DeviceState& D, int parity, const TileDev* tiles, int ntiles,            \
-                                     bool phi_only, double* out, int* status_out, cudaStream_t st);                \
+                                     bool phi_only, double* out, cudaStream_t st);                                 \
     cudaError_t launch_init_##NAME(const DeviceState& D, int parity, const TileDev* tiles8, int ntiles,             \
                                    const double* phi0, int64_t base, cudaStream_t st);                             \
     cudaError_t launch_get_state_##NAME(const DeviceState& D, int parity, const CaseDev& C, double* f, double* g,   \

@@ -1408,14 +1408,13 @@ step_kernel_pipe(const CaseDev* __restrict__ cases, const TileDev* __restrict__ 
 }
 
 // phi, rho, u_z, u_r, p of one case into dense FP64 arrays out[5][nz][nr]; with
-// PHI phi alone, which needs no window.  status_out (pinned host memory, or
-// null) takes the device status word along.  RM is the handle's rate mode in
+// PHI phi alone, which needs no window.  RM is the handle's rate mode in
 // FP64 (the update's own macroscopic step, lbm_f64.cuh: 116 -> 80 us for the
 // diagnostics of a 600 x 200 case) and kRatesGeneral otherwise.
 template <class Codec, int RM, bool PHI>
 __global__ void __launch_bounds__(kTR * 8)
 fields_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ tiles, StateDev<Codec> S,
-              double* __restrict__ out, const int* status, int* status_out) {
+              double* __restrict__ out) {
     using Real = typename Codec::Real;
     constexpr int TZ = 8;
     constexpr int LD = kTR + 4, NWIN = PHI ? 1 : (TZ + 4) * LD;
@@ -1427,7 +1426,6 @@ fields_kernel(const CaseDev* __restrict__ cases, const TileDev* __restrict__ til
     const TileDev t = tiles[blockIdx.x];
     pdl_trigger();
     pdl_wait();
-    if (status_out != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *status_out = *status;
     const CaseDev& C = cases[t.c];
     const CaseView<Codec> V = case_view<Codec>(S, C);
     const int j = t.j0 + threadIdx.x, k = t.k0 + threadIdx.y;
@@ -1784,13 +1782,13 @@ cudaError_t launch_step_t(const DeviceState& D, int parity, int variant, const T
 
 template <class Codec>
 cudaError_t launch_fields_t(const DeviceState& D, int parity, const TileDev* tiles, int ntiles, bool phi_only,
-                            double* out, int* status_out, cudaStream_t st) {
+                            double* out, cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
     StateDev<Codec> S = make_state<Codec>(D, parity);
     const CaseDev* cs = (const CaseDev*)D.cases;
     const dim3 block(kTR, 8);
     constexpr bool f64 = sizeof(typename Codec::Real) == 8;
-    auto launch = [&](auto* kernel) { launch_pdl(kernel, ntiles, block, st, cs, tiles, S, out, D.status, status_out); };
+    auto launch = [&](auto* kernel) { launch_pdl(kernel, ntiles, block, st, cs, tiles, S, out); };
     if (phi_only) launch(fields_kernel<Codec, kRatesGeneral, true>);
     else if (f64 && D.rate_mode == kRatesPaper) launch(fields_kernel<Codec, f64 ? kRatesPaper : kRatesGeneral, false>);
     else if (f64 && D.rate_mode == kRatesPaperRaw)
@@ -1835,8 +1833,8 @@ cudaError_t launch_set_state_t(const DeviceState& D, int parity, const CaseDev& 
         return launch_step_t<CODEC>(D, parity, variant, tiles, ntiles, st);                                      \
     }                                                                                                            \
     cudaError_t launch_fields_##NAME(const DeviceState& D, int parity, const TileDev* tiles, int ntiles,         \
-                                     bool phi_only, double* out, int* status_out, cudaStream_t st) {             \
-        return launch_fields_t<CODEC>(D, parity, tiles, ntiles, phi_only, out, status_out, st);                  \
+                                     bool phi_only, double* out, cudaStream_t st) {                              \
+        return launch_fields_t<CODEC>(D, parity, tiles, ntiles, phi_only, out, st);                              \
     }                                                                                                            \
     cudaError_t launch_init_##NAME(const DeviceState& D, int parity, const TileDev* tiles8, int ntiles,          \
                                    const double* phi0, int64_t base, cudaStream_t st) {                          \

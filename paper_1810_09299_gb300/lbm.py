@@ -38,6 +38,7 @@ EXPORTS = (
     "lbm_kernel_launches", "lbm_destroy", "lbm_strerror", "lbm_diag_reduce_noalloc",
     "lbm_selftest_bounded_wait", "lbm_case_diagnostics_enqueue", "lbm_diagnostics_wait", "lbm_init_phase_all",
     "lbm_case_axis_drops", "lbm_measure_fp64_rate", "lbm_selftest_direct_read",
+    "lbm_selftest_handle_wait",
 )
 MAX_AXIS_DROPS = 64
 DIAG_SLOTS = 4
@@ -116,6 +117,7 @@ def lib():
         "lbm_case_axis_drops": (ctypes.c_int, [vp, i32, i32, ctypes.POINTER(LbmDrop), ctypes.POINTER(i32), dp]),
         "lbm_measure_fp64_rate": (ctypes.c_int, [i32, vp, dp]),
         "lbm_selftest_direct_read": (ctypes.c_int, [vp, i64]),
+        "lbm_selftest_handle_wait": (ctypes.c_int, [vp, i32]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
