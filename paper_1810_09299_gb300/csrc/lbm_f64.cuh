@@ -356,6 +356,9 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
     const Sf m7 = (c * Q.m7 + s * (K.sr() * norm29(Sf{E12.a - E12.b, E12.e}))) + scale2(h6, 1) * norm29(Sf{PP.a - PP.b, PP.e});
     const Sf m8 = (c * Q.m8 + s * norm29((K.sr() * rr) * uz)) + h6 * norm29(uz * br + ur * az);
     const Sf m0 = scale2(udr - rr, -1);
+    // no part reaches one unit: g is zero (in_units makes -1 of the negative ones)
+    constexpr int kRestE = -990 - 62;
+    bool rest;
     if constexpr (kRaw) {
         // raw moments: k_3 = sum c^2 g relaxes with 1/tau_g, k_0 and k_8 take
         // equilibrium and half the source
@@ -363,8 +366,10 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         const Sf k3 = (c * Q.q + s * (K.sr() * pK)) + scale2(h6, 1) * norm29(scale2(udr, 1) - rr);
         const Sf w = K.r3() * norm29(Sf{(pE.a >> 1) + pE.b, pE.e});   // 3 r (p + rho u^2)
         const Sf v = udr - rr3;             // 6 times the rest of k_8
-        const int E = max(-994, max(max(max(k3.e, m0.e), max(w.e, v.e)), max(max(m7.e, m8.e), max(jz.e, jr.e)))) + 4;
+        const int top_e = max(max(max(k3.e, m0.e), max(w.e, v.e)), max(max(m7.e, m8.e), max(jz.e, jr.e)));
+        const int E = max(-994, top_e) + 4;
         bad = bad || E > 890;
+        rest = top_e < kRestE;
         const long long M0 = in_units(m0, E), K3 = in_units(k3, E), M7 = in_units(m7, E), M8 = in_units(m8, E);
         const long long K8 = ninth64(in_units(w, E)) + (third64(in_units(v, E)) >> 1);
         const long long JZ = in_units(jz, E), JR = in_units(jr, E);
@@ -388,8 +393,10 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         // coefficients add up to 28 at most.  in_units leaves half a unit out on
         // average; with its coefficient that is -11 to 10 units of 36 g, so the
         // quotients take 0 to 2 units back.
-        const int E = max(-994, max(max(max(m0.e, m1.e), max(m2.e, jz.e)), max(max(m7.e, m8.e), jr.e))) + 4;
+        const int top_e = max(max(max(m0.e, m1.e), max(m2.e, jz.e)), max(max(m7.e, m8.e), jr.e));
+        const int E = max(-994, top_e) + 4;
         bad = bad || E > 890;
+        rest = top_e < kRestE;
         const long long M0 = in_units(m0, E) * 4, M1 = in_units(m1, E), M2 = in_units(m2, E);
         const long long M7 = in_units(m7, E) * 9, M8 = in_units(m8, E) * 9;
         const long long JZ = in_units(jz, E) * 3, JR = in_units(jr, E) * 3;
@@ -404,10 +411,17 @@ __device__ __forceinline__ void update64(const CaseDev& C, const Win64& W, int a
         gp[8] = double_cvt(ninth64(dg - M8 + JZ - JR), E - 2);
         gp[6] = double_cvt(ninth64(dg - M8 - JZ + JR), E - 2);
     }
-    if (bad || top >= 0x7ff00000) {
+    // not a number, or at rest: both rare, one branch around them
+    const bool none = bad || top >= 0x7ff00000;
+    if (none || rest) {
+        const double v = none ? nan64() : 0.0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) fp[i] = gp[i] = nan64();
-        chz_out = chr_out = p_out = nan64();
+        for (int i = 0; i < 9; ++i) gp[i] = v;
+        if (none) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fp[i] = v;
+            chz_out = chr_out = p_out = v;
+        }
     }
 }
 
