@@ -130,7 +130,7 @@ typedef struct {
  * whose oscillation gives the frequency of Sec. 3.2 (Eq. 43-45) -- all FP64,
  * computed on the device in a fixed order (deterministic): each of a fixed set
  * of blocks sums its nodes plainly and then pairwise, and the block results
- * are added exactly and rounded once.  A node whose phi, u_z, u_r
+ * are added in 128-bit integers (longer ones where larger results cancel) to one rounding.  A node whose phi, u_z, u_r
  * or p is not finite is left out of every sum and extremum and counted in
  * nonfinite.
  *   mass               sum over nodes of r phi (equal to the sum of all f_i).

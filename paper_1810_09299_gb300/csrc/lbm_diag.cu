@@ -21,43 +21,82 @@ constexpr int kDiagThreads = 256;
 // (sum, 0) of quantities 0-6, then 7-10.
 constexpr int kSums = 7;
 
-// The sum of v[0 .. count) (stride `stride`, count <= 512) into every lane of the
-// calling warp, exact to its last rounding: the values as 128-bit integers in
-// units of 2^-64 of the last place of the largest one.  Compensated (Neumaier)
-// sums in FP64 took most of diag_final_kernel's 19.5 us: some 100 dependent
-// operations of a pipe that takes a warp instruction every 20 cycles; this takes
-// 8.  Values of 2^1007 and more, infinities and NaN are summed plainly.
-__device__ __forceinline__ double warp_exact_sum(const double* v, int count, int stride) {
+// The bits of x below 2^(L - 1075), in units of 2^(e - 1075).
+__device__ __forceinline__ unsigned long long bits_below(double x, int L, int& e) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    const unsigned long long m =
+        ((unsigned long long)(((uint32_t)hi & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
+    e = max(ex, 1);  // subnormal numbers share the exponent of the smallest normal ones
+    const int n = L - e;
+    return n >= 53 ? m : n <= 0 ? 0ull : m & ((1ull << n) - 1);
+}
+// The warp's sum of the bits of v[0 .. count) below 2^(L - 1075), in units of 2^(E - 1139), E
+// the exponent field of the largest value that has any; what lies below one unit is left out.
+__device__ __forceinline__ __int128 warp_window_sum(const double* v, int count, int stride, int L, int& E) {
     const int lane = threadIdx.x & 31;
-    int top = 0;
-    for (int i = lane; i < count; i += 32) top = max(top, __double2hiint(v[(size_t)i * stride]) & 0x7fffffff);
-    const int E = max((int)(__reduce_max_sync(0xffffffffu, (unsigned)top) >> 20), 1);
-    if (E >= 2030) {
-        double acc = 0.0;
-        for (int i = lane; i < count; i += 32) acc += v[(size_t)i * stride];
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        return acc;
-    }
+    int top = 1, e;
+    for (int i = lane; i < count; i += 32)
+        if (bits_below(v[(size_t)i * stride], L, e) != 0) top = max(top, e);
+    E = (int)__reduce_max_sync(0xffffffffu, (unsigned)top);
     __int128 acc = 0;
     for (int i = lane; i < count; i += 32) {
         const double x = v[(size_t)i * stride];
-        const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-        const unsigned long long m =
-            ((unsigned long long)(((uint32_t)hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
-        const int sh = E - max(e, 1);  // subnormal numbers share the exponent of the smallest normal ones
+        const unsigned long long m = bits_below(x, L, e);
+        const int sh = E - e;
         const unsigned __int128 y = sh < 128 ? ((unsigned __int128)m << 64) >> sh : (unsigned __int128)0;
-        acc += hi < 0 ? -(__int128)y : (__int128)y;
+        acc += __double2hiint(x) < 0 ? -(__int128)y : (__int128)y;
     }
     for (int off = 16; off > 0; off >>= 1) {
         const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, off);
         const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(acc >> 64), off);
         acc += ((__int128)hi << 64) | lo;
     }
+    return acc;
+}
+// The rest of a sum whose largest values cancelled: window after window below the first
+// one (sum acc, exponent E), each in four exact parts that are added up with compensation.
+__device__ __noinline__ double warp_cancelled_sum(const double* v, int count, int stride, __int128 acc, int E) {
+    double s = 0.0, c = 0.0;
+    for (;;) {
+        const bool neg = acc < 0;
+        const unsigned __int128 a = neg ? -(unsigned __int128)acc : (unsigned __int128)acc;
+        for (int k = 96; k >= 0; k -= 32) {
+            const double part = scalbn((double)(uint32_t)(a >> k), E - 1139 + k), x = neg ? -part : part, t = s + x;
+            c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+            s = t;
+        }
+        if (E <= 65) return s + c;  // (the unit is below the smallest number)
+        int next;
+        acc = warp_window_sum(v, count, stride, E - 64, next);
+        E = next;
+    }
+}
+// The sum of v[0 .. count) (stride `stride`, count <= 512) into every lane of the
+// calling warp: the values as 128-bit integers in units of 2^-64 of the last place of
+// the largest one, rounded once.  A value may lose what lies below a unit; where so much
+// cancels that this could count (the sum is below 2^74 units, of which at most 512 are
+// lost), the bits below are added as well.  Compensated (Neumaier) sums in FP64
+// took most of diag_final_kernel's 19.5 us: some 100 dependent operations of a pipe
+// that takes a warp instruction every 20 cycles; this takes 8.  Values of 2^1007 and
+// more, infinities and NaN are summed plainly.
+__device__ __forceinline__ double warp_exact_sum(const double* v, int count, int stride) {
+    const int lane = threadIdx.x & 31;
+    int top = 0;
+    for (int i = lane; i < count; i += 32) top = max(top, __double2hiint(v[(size_t)i * stride]) & 0x7fffffff);
+    int E = max((int)(__reduce_max_sync(0xffffffffu, (unsigned)top) >> 20), 1);
+    if (E >= 2030) {
+        double acc = 0.0;
+        for (int i = lane; i < count; i += 32) acc += v[(size_t)i * stride];
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        return acc;
+    }
+    const __int128 acc = warp_window_sum(v, count, stride, 4096, E);
     // one rounding: |acc| below 2^126 with its leading bit brought to bit 62 of
     // 64, the bits below folded into the last one
     const bool neg = acc < 0;
     unsigned __int128 a = neg ? -(unsigned __int128)acc : (unsigned __int128)acc;
     const unsigned long long ah = (unsigned long long)(a >> 64), al = (unsigned long long)a;
+    if (ah < 1024 && E > 65) return warp_cancelled_sum(v, count, stride, acc, E);
     if ((ah | al) == 0) return 0.0;
     const int lead = ah ? 127 - __clzll((long long)ah) : 63 - __clzll((long long)al);
     const int down = lead - 62;
