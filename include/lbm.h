@@ -333,7 +333,7 @@ int64_t lbm_kernel_launches(const lbm_handle* h);
  *             lbm_diagnostics); step is copied into the first entry.
  *   stream    cudaStream_t the work is enqueued on (NULL: default stream);
  *             the call returns without synchronising.
- * Nothing is allocated: the only scratch is a fixed 43,776-byte static device
+ * Nothing is allocated: the only scratch is a fixed 26,752-byte static device
  * array of the library, held on every GPU that loads it until the process
  * exits.  Requires nz, nr >= 1 and nz * nr <= 2^31 - 1, else
  * LBM_ERR_INVALID_ARG.  The first call on a device looks up that array's

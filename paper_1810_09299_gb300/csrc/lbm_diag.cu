@@ -12,13 +12,12 @@ namespace axilbm {
 
 namespace {
 
-constexpr int kDiagBlocks = kDiagPartials / 18;  // 2 x 152 SMs; fixed so the summation order is fixed
+constexpr int kDiagBlocks = kDiagPartials / kDiagRecord;  // 2 x 152 SMs; fixed so the summation order is fixed
 constexpr int kDiagThreads = 256;
 
 // Quantities: 0 mass, 1 kinetic, 2 z-moment, 3 p in liquid, 4 weight in liquid,
 // 5 p in gas, 6 weight in gas (sums); 7 max |u|^2, 8 phi_min, 9 phi_max
-// (extrema); 10 non-finite count (sum).  A partial record is 18 doubles:
-// (sum, 0) of quantities 0-6, then 7-10.
+// (extrema); 10 non-finite count (sum).  A partial record holds them in this order.
 constexpr int kSums = 7;
 
 // The bits of x below 2^(L - 1075), in units of 2^(e - 1075).
@@ -222,18 +221,15 @@ __global__ void __launch_bounds__(kDiagThreads) diag_partial_kernel(const double
     sh[kSums + 3][threadIdx.x] = bad;
     __syncthreads();
     const int w = threadIdx.x >> 5;
-    double* out = partials + (size_t)blockIdx.x * 18;
+    double* out = partials + (size_t)blockIdx.x * kDiagRecord;
     if (w < kSums) {
         const double t = warp_sum(sh[w], kDiagThreads, 1);
-        if ((threadIdx.x & 31) == 0) {
-            out[2 * w] = t;
-            out[2 * w + 1] = 0.0;
-        }
+        if ((threadIdx.x & 31) == 0) out[w] = t;
     } else {
         double e[4];
         warp_extrema(sh[kSums], sh[kSums + 1], sh[kSums + 2], sh[kSums + 3], kDiagThreads, 1, e);
         if ((threadIdx.x & 31) == 0)
-            for (int q = 0; q < 4; ++q) out[14 + q] = e[q];
+            for (int q = 0; q < 4; ++q) out[kSums + q] = e[q];
     }
 }
 
@@ -279,11 +275,12 @@ __global__ void __launch_bounds__(kFinalThreads) diag_final_kernel(const double*
     for (int off = 16; off > 0; off >>= 1) len += __shfl_down_sync(0xffffffffu, len, off);
     if (lane == 0) slen[w] = len;
     if (w < kSums) {
-        const double r = warp_exact_sum(partials + 2 * w, records, 18);
+        const double r = warp_exact_sum(partials + w, records, kDiagRecord);
         if (lane == 0) sres[w] = r;
     } else {
         double e[4];
-        warp_extrema(partials + 14, partials + 15, partials + 16, partials + 17, records, 18, e);
+        const double* x = partials + kSums;
+        warp_extrema(x, x + 1, x + 2, x + 3, records, kDiagRecord, e);
         if (lane == 0)
             for (int q = 0; q < 4; ++q) sres[kSums + q] = e[q];
     }
@@ -718,7 +715,7 @@ extern "C" int lbm_measure_fp64_rate(int32_t iters, void* stream, double* fma_pe
 // partial sums, is a fixed static device array of this module.
 namespace {
 
-constexpr int kScratchDoubles = axilbm::kDiagPartials;  // 304 blocks x 18 doubles = 43,776 bytes
+constexpr int kScratchDoubles = axilbm::kDiagPartials;  // 304 blocks x 11 doubles = 26,752 bytes
 constexpr int64_t kNoAllocMaxNodes = 2147483647;       // nz * nr must fit a signed 32-bit count
 constexpr int kMaxDevices = 64;
 

@@ -86,7 +86,8 @@ constexpr int kMapsPerCase = 4;
 // doubles.  Deterministic (fixed block count and order).  out and status_out
 // may be pinned host memory; with status_out the device status word is copied
 // there as well.
-constexpr int kDiagPartials = 304 * 18;  // 304 blocks x 18 doubles
+constexpr int kDiagRecord = 11;                   // one block's partial results
+constexpr int kDiagPartials = 304 * kDiagRecord;  // of 304 blocks
 int diag_partials_size();
 cudaError_t launch_diag(const double* fields, int nz, int nr, int zper, double step, double* partials,
                         double* out, const int* status, int* status_out, cudaStream_t st);
