@@ -48,7 +48,9 @@ typedef enum {
 
 /* Storage and arithmetic precision of a handle.
  *   LBM_FP64      populations in FP64; arithmetic in FP64, or (the paper's rates, both
- *                 collisions) in 62-bit integers with exponents, with smaller errors.
+ *                 collisions) in 62-bit integers with exponents, with smaller errors;
+ *                 there u, p and chi below 2^-939 become zero, and results of 2^948 and
+ *                 more not-a-number.
  *   LBM_FP32      populations f_1..8 and g_0..8 in FP32, arithmetic in FP32
  *                 (reciprocals, divisions and square roots by the hardware
  *                 approximations, a few ulp, subnormal operands and results
@@ -130,9 +132,9 @@ typedef struct {
  * whose oscillation gives the frequency of Sec. 3.2 (Eq. 43-45) -- all FP64,
  * computed on the device in a fixed order (deterministic): each of a fixed set
  * of blocks sums its nodes plainly and then pairwise, and the block results
- * are added in 128-bit integers (longer ones where larger results cancel) to one rounding.  A node whose phi, u_z, u_r
- * or p is not finite is left out of every sum and extremum and counted in
- * nonfinite.
+ * are added in 128-bit integers (longer ones where larger results cancel) to
+ * one rounding.  A node whose phi, u_z, u_r or p is not finite is left out of
+ * every sum and extremum and counted in nonfinite.
  *   mass               sum over nodes of r phi (equal to the sum of all f_i).
  *   kinetic            sum of 0.5 r rho |u|^2.
  *   z_centroid         sum r z phi / sum r phi.
@@ -366,8 +368,8 @@ int lbm_selftest_handle_wait(lbm_handle* h, int32_t tries);
 int lbm_selftest_direct_read(double* host_out, int64_t bytes);
 
 /* Measured throughput of the GPU's FP64 pipe (no paper counterpart: the
- * denominator of the FP64 step's arithmetic roofline, whose step is bound by
- * that pipe rather than by memory).  Launches 4 blocks of 256 threads per SM,
+ * denominator of the FP64 step's share of that pipe, which bounds handles with
+ * rates by array).  Launches 4 blocks of 256 threads per SM,
  * each thread running 8 independent chains of `iters` dependent FP64 fused
  * multiply-adds, after one untimed warm-up launch, and writes the FMA count
  * over the CUDA-event time of the timed launch to *fma_per_second.  Allocates

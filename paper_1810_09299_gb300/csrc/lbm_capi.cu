@@ -450,7 +450,7 @@ int row_shape(const lbm_sim* h) {
 //     8 rows: FP64 9.2 -> 7.8, bfloat16 3.02 -> 2.75, FP32 2.50 -> 2.38, FP16 2.83 and
 //     2.95), and where some SMs would hold two of them, most one and taller
 //     tiles do not help (row_shape's figures).  128 tiles (128 x 256) and 250 (150 x
-//     400) take 8 rows: FP32 2.52 against 2.77 and 3.41 against 3.66.
+//     400) take 8 rows: FP32 2.51 against 2.96 and 3.40 against 3.66.
 //   FP16, packed pairs of nodes (7) from 3/2 tiles of 16 rows per SM on: 64 x 180
 //     and 128 x 256 are slower there (3.40 against 3.02), 200 x 600 (266 tiles) 5.01 ->
 //     4.94, 256 x 1024 (512) 8.23 -> 7.70, 512 cases 757 -> 558;

@@ -6,8 +6,10 @@
 // lbm_device.cuh takes 383 FP64 operations per node and is bound by that pipe.
 // Here the sums of populations and of the phi stencil, both collisions, both
 // inverse transforms, reciprocals and roots run in 64-bit integers
-// (lbm_fix64.cuh) beside about 10 FP64 operations (what depends on phi alone) and
-// 20 conversions.  32 batched cases (1.89 M nodes), us a step:
+// (lbm_fix64.cuh); what depends on phi alone and the results' conversions stay
+// on the FP64 pipe: 34.4 instructions per node there now (ncu, the phi ring's share
+// and conversions included).  32 batched cases (1.89 M nodes), us a step; the counts
+// are those written in the source, without the ring:
 //   general form, 383 operations per node                          1342
 //   the algebra below, 280                                         1005
 //   sums of populations and of the stencil in integers, 202         724
@@ -16,12 +18,12 @@
 //   shared alignments, the nine g converted on the FP64 pipe, 61    383
 //   column constants from a table in device memory, 57              376
 //   high-word multiplications; reciprocals and roots in integers, 29  331
-//   every result converted on the FP64 pipe, 43                     313
+//   every result converted on the FP64 pipe                         313
 //   3 CTAs of 80 registers per SM                                   302
 //   dropped bits given back on average, constants to 62 bits        309
 // (Conversions in integers had been the better ones while the FP64 pipe was
-// busier: 399 against 383 with all of them there, 61 operations.)  At 313 us the
-// ALU is 58 % and the FP64 pipe 42 % busy (ncu); timing-only copies without the
+// busier: 399 against 383 with all of them there, 61 operations.)  Now the ALU is 60 %
+// and the FP64 pipe 34 % busy (ncu); timing-only copies without the
 // mixed products of the multiplications, without the ring and without the
 // sums' conversions ran 13, 6 and 6 % faster.
 // The last line is for accuracy: integers that only drop bits err in one
