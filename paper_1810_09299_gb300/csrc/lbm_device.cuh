@@ -596,10 +596,10 @@ __device__ __forceinline__ float rcp_(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// 1 / x: y0 from the hardware, e = 1 - x y0 (below 2^-19.9 over 2^28 mantissas), y0 (1 +
-// e + e^2): what the series leaves out is below 2^-59, so the last rounding is all
-// that is left.  Outside 2^-1000 .. 2^1000 (and for 0, infinities and NaN) the IEEE
-// division.
+// 1 / x: y0 from the hardware, e = 1 - x y0 (below 2^-19.9 over 2^28 mantissas), the
+// geometric series y0 (1 + e + e^2): what it leaves out is below 2^-59, so the last
+// rounding is all that is left.  Outside 2^-1000 .. 2^1000 (and for 0, infinities and
+// NaN) the IEEE division.
 __device__ __forceinline__ double rcp64(double x) {
     double y0;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
